@@ -680,7 +680,8 @@ struct Workspace {
     float *patch = nullptr;    // [rows][kmax * cells] mutated-channel values
     float *zb = nullptr;
     int64_t z_stride = 0;
-    float *gap_tmp = nullptr;
+    float *tmp = nullptr;      // stage scratch rows (stage_scratch)
+    LstmWs lw;                 // a mutated LSTM layer's scratch (lw.proj = tmp)
     int64_t rows = 0;
     TcDeltaWs dw;              // tensor-core delta scratch (GF / WS slots of a batch)
     // unchanged-row elimination: per-row flags, per-block counts, the compacted row
@@ -693,6 +694,10 @@ int64_t gap_map_stride(const Stage &S)
     const int mh = S.pool ? S.oh / 2 : S.oh, mw = S.pool ? S.ow / 2 : S.ow;
     return round4((int64_t)mh * mw * S.oc);
 }
+
+// Scratch floats per row of a stage: the map before global average pooling, or an LSTM's
+// input sums.
+int64_t stage_scratch(const Stage &S) { return S.gap ? gap_map_stride(S) : lstm_proj_floats(S); }
 
 // Bytes per batch row for a group at layer l (vanilla: every stage input from 1,
 // plus z_l).
@@ -710,13 +715,15 @@ int64_t row_bytes(const mure_model *m, int l, bool vanilla, bool z_rows = false)
     const Stage &S = m->st[l];
     b += (int64_t)S.oc * (S.gap ? 1 : (S.pool ? (S.oh / 2) * (S.ow / 2) : S.oh * S.ow));  // patch values (bound)
     int64_t g = 0;
-    for (int v = vanilla ? 0 : l + 1; v < m->L; ++v)
-        if (m->st[v].gap) g = std::max(g, gap_map_stride(m->st[v]));
+    for (int v = vanilla ? 0 : l + 1; v < m->L; ++v) g = std::max(g, stage_scratch(m->st[v]));
+    // a mutated LSTM layer: its inputs' sums (bound: per row) and its mutated units' (bound: all)
+    if (S.kind == MURE_NODE_LSTM) g = std::max(g, stage_scratch(S)) + stage_scratch(S);
     return (b + g) * 4;
 }
 
 void alloc_workspace(mure_ctx *c, Scratch &sc, const mure_model *m, int64_t rows, bool vanilla, int lmin,
-                     int64_t patch_floats, int delta_slots, int delta_k, Workspace &ws, bool z_rows = false)
+                     int64_t patch_floats, int delta_slots, int delta_k, int lstm_kmax, int64_t lstm_groups,
+                     Workspace &ws, bool z_rows = false)
 {
     ws.rows = rows;
     if (delta_slots > 0) {
@@ -744,9 +751,19 @@ void alloc_workspace(mure_ctx *c, Scratch &sc, const mure_model *m, int64_t rows
         ws.zb = sc.get<float>(rows * zs);
     }
     int64_t g = 0;
-    for (int v = 0; v < m->L; ++v)
-        if (m->st[v].gap) g = std::max(g, gap_map_stride(m->st[v]));
-    if (g) ws.gap_tmp = sc.get<float>(rows * g);
+    for (int v = 0; v < m->L; ++v) g = std::max(g, stage_scratch(m->st[v]));
+    if (g) ws.tmp = sc.get<float>(rows * g);
+    ws.lw.proj = ws.tmp;
+    if (lstm_kmax > 0) {
+        int64_t steps = 0, cin = 0;
+        for (const Stage &S : m->st)
+            if (S.kind == MURE_NODE_LSTM) {
+                steps = std::max<int64_t>(steps, S.iw);
+                cin = std::max<int64_t>(cin, S.ic);
+            }
+        ws.lw.projx = sc.get<float>(rows * steps * 4 * lstm_kmax);
+        ws.lw.cols = sc.get<float>(lstm_groups * cin * 4 * lstm_kmax);
+    }
 }
 
 // One batch: G mutants of group l (starting at group position g0) x an input tile.
@@ -805,7 +822,7 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
         acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[v + 1].size * 4;
         timed(v, 2 * S.macs * rm.R, [&] {
             return launch_stage_simt(S, xsrc(S.in_src), rm, z_out, z_stride, skip_of(S), ws.xb[v + 1], m->xd[v + 1].stride,
-                                     ws.gap_tmp, s);
+                                     ws.tmp, s);
         });
     };
     const Stage &Sl = m->st[l];
@@ -822,7 +839,9 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
             for (int v = 0; v < l; ++v) stage(v, nullptr, 0);
         acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[l + 1].size * 4;
         timed(l, 2 * Sl.macs * rm.R, [&] {
-            return launch_lstm(Sl, xsrc(Sl.in_src), rm, nullptr, 0, ws.xb[l + 1], m->xd[l + 1].stride, &pa, s);
+            LstmWs lw = ws.lw;
+            lw.kmax = dt.kmax_layer[l];
+            return launch_lstm(Sl, xsrc(Sl.in_src), rm, nullptr, 0, ws.xb[l + 1], m->xd[l + 1].stride, &pa, lw, s);
         });
         for (int v = l + 1; v < L - 1; ++v) stage(v, nullptr, 0);
         const Stage &SLr = m->st[L - 1];
@@ -942,7 +961,7 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
                 acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[l + 2].size * 4;
                 timed(l + 1, 2 * Sn.macs * rm.R, [&] {
                     return launch_tc(Sn, base, rm, nullptr, 0, skip_of(Sn), ws.xb[l + 2], m->xd[l + 2].stride,
-                                     ws.gap_tmp, s, &ov);
+                                     ws.tmp, s, &ov);
                 });
                 vstart = l + 2;
             } else if (Sn.variant > 0 && !skip_reader) {
@@ -972,7 +991,7 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
                 const FinalFuse ff{SLast.W, SLast.b, SLast.oc, SLast.K, SLast.act1, fa};
                 timed(L - 2, 2 * (Sv.macs + SLast.macs) * rm.R, [&] {
                     return launch_tc(Sv, xsrc(Sv.in_src), rm, nullptr, 0, skip_of(Sv), ws.xb[L - 1], m->xd[L - 1].stride,
-                                     ws.gap_tmp, s, nullptr, &ff);
+                                     ws.tmp, s, nullptr, &ff);
                 });
                 break;
             }
@@ -1068,7 +1087,7 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
     auto fused_last = [&](Src x, const Overlay *ovp) {
         const Stage &S = m->st[L - 2];
         timed(L - 2, 2 * (S.macs + SLast.macs) * rm.R, [&] {
-            return launch_tc(S, x, rm, nullptr, 0, skip_of(S), ws.xb[L - 1], m->xd[L - 1].stride, ws.gap_tmp, s, ovp, &ff);
+            return launch_tc(S, x, rm, nullptr, 0, skip_of(S), ws.xb[L - 1], m->xd[L - 1].stride, ws.tmp, s, ovp, &ff);
         });
     };
     const bool fuse = L >= 2 && tc_final_fusable(m->st[L - 2], SLast);
@@ -1079,7 +1098,7 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
         }
         acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[l + 2].size * 4;
         timed(l + 1, 2 * Sn.macs * rm.R, [&] {
-            return launch_tc(Sn, base, rm, nullptr, 0, skip_of(Sn), ws.xb[l + 2], m->xd[l + 2].stride, ws.gap_tmp, s,
+            return launch_tc(Sn, base, rm, nullptr, 0, skip_of(Sn), ws.xb[l + 2], m->xd[l + 2].stride, ws.tmp, s,
                              &ov);
         });
     } else if (Sn.variant > 0 && !skip_reader) {
@@ -1185,8 +1204,12 @@ void evaluate(mure_ctx *c, const mure_model *m, const mure_cache *ca, const mure
             delta_slots = (int)std::max<int64_t>(delta_slots, gb * std::max(dt.kmax_layer[l], 1));
             delta_k = std::max(delta_k, m->st[l].K);
         }
+        int lstm_kmax = 0;   // neurons per mutant of the mutated LSTM layers
+        for (int l = 0; l < m->L; ++l)
+            if (m->st[l].kind == MURE_NODE_LSTM) lstm_kmax = std::max(lstm_kmax, dt.kmax_layer[l]);
         Workspace ws;
-        alloc_workspace(c, sc, m, rows, vanilla, lmin, patch_floats, delta_slots, delta_k, ws, dt.has_later);
+        alloc_workspace(c, sc, m, rows, vanilla, lmin, patch_floats, delta_slots, delta_k, lstm_kmax,
+                        std::min(Gmax, gbig), ws, dt.has_later);
         FAILIF(o->skip_unchanged != 0 && o->skip_unchanged != 1, c, MURE_ERR_INVALID_ARG, "skip_unchanged must be 0 or 1");
         if (!vanilla && o->skip_unchanged) {
             ec.skip_unchanged = true;
@@ -1331,9 +1354,8 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
                                 on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
         Scratch sc(c);
         int64_t g = 0;
-        for (int v = 0; v < L; ++v)
-            if (m->st[v].gap) g = std::max(g, gap_map_stride(m->st[v]));
-        float *gap_tmp = g ? sc.get<float>(ca->n_pad * g) : nullptr;
+        for (int v = 0; v < L; ++v) g = std::max(g, stage_scratch(m->st[v]));
+        float *tmp = g ? sc.get<float>(ca->n_pad * g) : nullptr;
         // intermediate activations: in the cache (full) or in scratch rows (vanilla
         // only needs the predictions)
         std::vector<float *> xs(L + 1), zs(L);
@@ -1344,7 +1366,7 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
             const Stage &S = m->st[v];
             const Src skip = S.has_add ? Src{xs[S.skip_src], m->xd[S.skip_src].stride, 0} : Src{nullptr, 0, 0};
             c->launches += launch_stage_simt(S, Src{xs[S.in_src], m->xd[S.in_src].stride, 0}, rm, zs[v], m->zd[v].stride, skip,
-                                             xs[v + 1], m->xd[v + 1].stride, gap_tmp, s);
+                                             xs[v + 1], m->xd[v + 1].stride, tmp, s);
             check_launch(c);
         }
         FinalArgs fa{};
@@ -1521,8 +1543,10 @@ mure_status mure_model_load(mure_ctx *c, const mure_model_desc *d, mure_model **
             const int64_t nb = S.kind == MURE_NODE_LSTM ? 4 * (int64_t)S.oc : S.oc;
             S.b = (float *)dalloc(c, nb * 4);
             Wt.resize(nw);
-            for (int o = 0; o < S.oc; ++o)
-                for (int k = 0; k < S.K; ++k) Wt[(int64_t)k * S.oc + o] = n.W[(int64_t)o * S.K + k];
+            // [K][oc]; an LSTM's four gate rows per unit as columns: [cin + units][4 oc]
+            const int wrows = S.kind == MURE_NODE_LSTM ? 4 * S.oc : S.oc, wcols = (int)(nw / wrows);
+            for (int o = 0; o < wrows; ++o)
+                for (int k = 0; k < wcols; ++k) Wt[(int64_t)k * wrows + o] = n.W[(int64_t)o * wcols + k];
             CK(c, cudaMemcpyAsync(S.W, n.W, nw * 4, cudaMemcpyHostToDevice, c->stream));
             CK(c, cudaMemcpyAsync(S.Wt, Wt.data(), nw * 4, cudaMemcpyHostToDevice, c->stream));
             if (n.b) CK(c, cudaMemcpyAsync(S.b, n.b, nb * 4, cudaMemcpyHostToDevice, c->stream));

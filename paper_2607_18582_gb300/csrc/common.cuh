@@ -47,7 +47,8 @@ struct Stage {
     int *err = nullptr;       // device error word of the context (bounded waits)
     const int64_t *wait_limit = nullptr;   // host: the context's wait limit (0 = default)
     float *W = nullptr;       // device [oc][K]
-    float *Wt = nullptr;      // device [K][oc] (the same weights, K-major rows)
+    float *Wt = nullptr;      // device [K][oc] (the same weights, K-major rows; an LSTM's
+                              // [cin + units][4 u + gate])
     float *b = nullptr;       // device [oc]
     float sigma_std = 0.f;    // population std of W (host copy, fp32-rounded for info)
 };
@@ -151,9 +152,10 @@ struct Overlay {
     const int32_t *op = nullptr;
 };
 
-// Stage v over R rows: z (optional) and y = post(act1(conv(x) + b)).
+// Stage v over R rows: z (optional) and y = post(act1(conv(x) + b)).  tmp: the stage's row
+// scratch (the map before global average pooling; an LSTM's input sums).
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip,
-                      float *y_out, int64_t y_stride, float *gap_tmp, cudaStream_t s);
+                      float *y_out, int64_t y_stride, float *tmp, cudaStream_t s);
 
 // The shared-memory direct convolution for small inputs (variant of a stage, 0 when
 // the geometry is not one it compiles) and its launcher.
@@ -205,8 +207,17 @@ int recurrent_supported(const Stage &S);
 int launch_embed(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, float *y_out, int64_t y_stride,
                  cudaStream_t s);
 struct PatchArgs;
+// Scratch of an LSTM layer: the input part of every gate's sum, [rows][steps][4 units] (rows
+// that read cached inputs: one per input of the tile), and, for a mutated layer of at most
+// kmax neurons per mutant, the same for the mutated units, rows x steps x 4 kmax, with their
+// input weights, mutants x cin x 4 kmax.
+struct LstmWs {
+    float *proj = nullptr, *projx = nullptr, *cols = nullptr;
+    int kmax = 0;
+};
+int64_t lstm_proj_floats(const Stage &S);   // proj floats per row (0: not an LSTM layer)
 int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, float *y_out, int64_t y_stride,
-                const PatchArgs *pa, cudaStream_t s);
+                const PatchArgs *pa, const LstmWs &lw, cudaStream_t s);
 
 // Global average pooling of R rows of a [P][C] map.
 int launch_gap(const float *in, int64_t in_stride, int P, int C, int R, float *y, int64_t y_stride, cudaStream_t s);

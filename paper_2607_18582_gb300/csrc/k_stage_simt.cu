@@ -195,12 +195,16 @@ __global__ void __launch_bounds__(256) k_dwconv(const StageParams p)
 }
 
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out,
-                      int64_t y_stride, float *gap_tmp, cudaStream_t s)
+                      int64_t y_stride, float *tmp, cudaStream_t s)
 {
     if (rm.R <= 0) return 0;
-    if (S.tc) return launch_tc(S, x, rm, z_out, z_stride, skip, y_out, y_stride, gap_tmp, s);
+    if (S.tc) return launch_tc(S, x, rm, z_out, z_stride, skip, y_out, y_stride, tmp, s);
     if (S.kind == MURE_NODE_EMBED) return launch_embed(S, x, rm, z_out, z_stride, y_out, y_stride, s);
-    if (S.kind == MURE_NODE_LSTM) return launch_lstm(S, x, rm, z_out, z_stride, y_out, y_stride, nullptr, s);
+    if (S.kind == MURE_NODE_LSTM) {
+        LstmWs lw;
+        lw.proj = tmp;
+        return launch_lstm(S, x, rm, z_out, z_stride, y_out, y_stride, nullptr, lw, s);
+    }
     if (S.kind == MURE_NODE_DWCONV) {
         StageParams p{};
         p.x = x.p; p.x_stride = x.stride; p.x_per_input = x.per_input;
@@ -225,10 +229,10 @@ int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     p.skip = skip.p; p.skip_stride = skip.stride; p.skip_per_input = skip.per_input;
     p.sk_w = S.sk_w; p.sk_c = S.sc_c; p.sk_stride = S.sc_stride;
     p.z = z_out; p.z_stride = z_stride;
-    // with global average pooling the post-op map goes to gap_tmp first
+    // with global average pooling the post-op map goes to the scratch first
     const int mh = S.pool ? S.oh / 2 : S.oh, mw = S.pool ? S.ow / 2 : S.ow;
     const int64_t map_stride = round4((int64_t)mh * mw * S.oc);
-    p.y = S.gap ? gap_tmp : y_out;
+    p.y = S.gap ? tmp : y_out;
     p.y_stride = S.gap ? map_stride : y_stride;
     p.pw = S.ow / 2;
     p.P = S.pool ? 4 * (S.oh / 2) * (S.ow / 2) : S.oh * S.ow;
@@ -246,7 +250,7 @@ int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     }
     if (S.gap) {
         const int64_t n = (int64_t)rm.R * S.oc;
-        k_gap<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(gap_tmp, map_stride, mh * mw, S.oc, rm.R, y_out, y_stride);
+        k_gap<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tmp, map_stride, mh * mw, S.oc, rm.R, y_out, y_stride);
         ++launches;
     }
     return launches;

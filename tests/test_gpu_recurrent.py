@@ -74,6 +74,28 @@ def test_recurrent_network_matches_oracle(M, ctx, oracle_mod, size):
     assert np.array_equal(u["kill_bits"], r["kill_bits"])
 
 
+@pytest.mark.parametrize("n_in,per_layer", [(1, 4), (65, 7), (200, 40), (1500, 12)])
+def test_lstm_split_over_batches(M, ctx, oracle_mod, n_in, per_layer):
+    """The LSTM's rows per block, the waves of blocks and the sharing of the input sums follow the
+    batch: the same bits from one large batch, many small ones and vanilla; widths that are no
+    multiple of 4 and the 64-unit limit; logits against the oracle."""
+    model = wl.rnn(3, n_classes=5, vocab=40, dim=13, units=(64, 33), steps=5, name="rnn_odd")
+    X = wl.inputs(model, n_in, 2)
+    table = every_operator(model, per_layer, 90)
+    m = M.mure_model_load(ctx, model)
+    cache = M.mure_build_prefix_cache(m, X)
+    r = M.mure_eval_mutants(cache, table, logits=True)
+    for other in (M.mure_eval_mutants(cache, table, logits=True, workspace_bytes=1 << 20),
+                  M.mure_eval_mutants(cache, table, logits=True, skip_unchanged=True),
+                  M.mure_eval_vanilla(m, X, table, logits=True)):
+        assert np.array_equal(other["logits"].view(np.uint32), r["logits"].view(np.uint32))
+        assert np.array_equal(other["kill_bits"], r["kill_bits"])
+    some = np.unique(np.linspace(0, n_in - 1, 8).round().astype(np.int64))
+    ora = oracle_mod.vanilla(model, X[some], table)
+    ok, worst = logits_close(r["logits"][:, some], ora["logits"])
+    assert ok, worst
+
+
 def test_recurrent_identity_mutants_and_bad_ids(M, ctx):
     model = small_rnn()
     X = wl.inputs(model, 64, 1)
