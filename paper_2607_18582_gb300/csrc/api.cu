@@ -649,6 +649,7 @@ DevTable upload_table(mure_ctx *c, Scratch &sc, const mure_model *m, const mure_
         ea.patch = dt.patch;
         ea.perm = perm_len ? sc.get<int32_t>(perm_len) : nullptr;
         ea.ws_as_weights = ws_as_weights;
+        ea.bounds(jobs);
         dt.expand_launches = launch_expand(ea, c->stream);
         check_launch(c);
         if (patch_out) CK(c, cudaMemcpyAsync(patch_out, dt.patch, plen * 4, cudaMemcpyDeviceToHost, c->stream));

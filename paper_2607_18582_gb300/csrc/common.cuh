@@ -325,6 +325,14 @@ struct ExpandArgs {
     float *patch;
     int32_t *perm;              // WS permutation scratch
     int ws_as_weights;          // 1: WS patch holds the permuted weights (inspection)
+    int max_gf = 0, max_ws = 0; // largest fan-in among the GF / WS jobs (0: none)
+    void bounds(const std::vector<SlotJob> &all)
+    {
+        for (const SlotJob &j : all) {
+            int &m = j.op == MURE_OP_GF ? max_gf : max_ws;
+            if (j.F > m) m = j.F;
+        }
+    }
 };
 int launch_expand(const ExpandArgs &ea, cudaStream_t s);
 

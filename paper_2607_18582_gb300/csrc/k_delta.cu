@@ -10,60 +10,132 @@ namespace mure {
 
 // ------------------------------------------------------------------ expansion --
 
-// Box-Muller in fp64 on SplitMix64 draws: standard normal number f of a stream.
-__device__ double gauss_f64(uint64_t stream, int64_t f)
-{
-    const int64_t pr = f >> 1;
-    const double u1 = (double)((splitmix64(stream, (uint64_t)(2 * pr)) >> 11) + 1) * (1.0 / 9007199254740992.0);
-    const double u2 = (double)((splitmix64(stream, (uint64_t)(2 * pr + 1)) >> 11) + 1) * (1.0 / 9007199254740992.0);
-    const double r = sqrt(-2.0 * log(u1));
-    const double th = 6.283185307179586476925286766559 * u2;
-    return (f & 1) ? r * sin(th) : r * cos(th);
-}
+// GF: standard normals by Box-Muller in fp64 on SplitMix64 draws; normals 2p and 2p + 1 of a
+// stream share draws 2p and 2p + 1, so a thread makes both.  fp64 is what bounds it (two
+// operations per cycle and SM): a slot's fan-in is spread over blocks of 512 values (one block
+// per slot took 464 us for one embedding channel of 20,000 entries, now 14).
+constexpr int kExpandValues = 512;
 
-__global__ void k_expand(const ExpandArgs a)
+__global__ void __launch_bounds__(kExpandValues / 2) k_expand_gf(const ExpandArgs a)
 {
     const SlotJob jb = a.jobs[blockIdx.x];
+    if (jb.op != MURE_OP_GF) return;
+    const uint64_t stream = splitmix64(jb.seed, (uint64_t)jb.q);
+    const double sigma = (double)jb.param * a.sigma[jb.layer];
+    for (int64_t f = (int64_t)blockIdx.y * kExpandValues + 2 * threadIdx.x; f < jb.F; f += (int64_t)gridDim.y * kExpandValues) {
+        const double u1 = (double)((splitmix64(stream, (uint64_t)f) >> 11) + 1) * (1.0 / 9007199254740992.0);
+        const double u2 = (double)((splitmix64(stream, (uint64_t)f + 1) >> 11) + 1) * (1.0 / 9007199254740992.0);
+        const double r = sqrt(-2.0 * log(u1));
+        const double th = 6.283185307179586476925286766559 * u2;
+        float *out = a.patch + jb.out_off + f;
+        out[0] = (float)(sigma * (r * cos(th)));
+        if (f + 1 < jb.F) out[1] = (float)(sigma * (r * sin(th)));
+    }
+}
+
+// WS: Fisher-Yates from the last index down; step i swaps places i and j_i, draw F-1-i giving
+// j_i = floor(u (i+1)).
+__device__ __forceinline__ int shuffle_partner(uint64_t stream, int F, int i)
+{
+    const double u = (double)(splitmix64(stream, (uint64_t)(F - 1 - i)) >> 11) * (1.0 / 9007199254740992.0);
+    const int j = (int)(u * (double)(i + 1));
+    return j > i ? i : j;
+}
+
+// The same permutation without the serial chain of swaps.  Before step i, place p holds what
+// the last earlier step that swapped into p (the smallest e > i with j_e = p) found at its own
+// place e, or p itself if none did.  So with A(i) = the value at place i before step i:
+// A(i) = A(e), e the smallest e > i with j_e = i, or i; and the result at i is A(e), e the
+// smallest e > i with j_e = j_i, or j_i.  The steps into each place form short lists (their
+// expected length grows with log F), and A follows a short chain.  Lists and chains in
+// shared memory, 8 F bytes; above kShuffleMax places one thread swaps in global memory as
+// before.  The MLP's 784 inputs: 155 us with
+// one thread swapping, now 8.
+constexpr int kShuffleMax = 25000;
+
+__global__ void __launch_bounds__(1024) k_expand_ws(const ExpandArgs a)
+{
+    extern __shared__ int sh[];
+    const SlotJob jb = a.jobs[blockIdx.x];
+    if (jb.op != MURE_OP_WS) return;
     const uint64_t stream = splitmix64(jb.seed, (uint64_t)jb.q);
     float *out = a.patch + jb.out_off;
     const float *w = a.W[jb.layer] + (int64_t)jb.j * jb.F;
-    if (jb.op == MURE_OP_GF) {
-        const double sigma = (double)jb.param * a.sigma[jb.layer];
-        for (int f = threadIdx.x; f < jb.F; f += blockDim.x) out[f] = (float)(sigma * gauss_f64(stream, f));
+    int32_t *perm = a.perm + jb.perm_off;
+    const int F = jb.F, tid = threadIdx.x, nt = blockDim.x;
+    auto write = [&](int f, int v) {
+        const float wp = __ldg(w + v);
+        out[f] = a.ws_as_weights ? wp : wp - __ldg(w + f);
+    };
+    if (F > kShuffleMax) {
+        for (int f = tid; f < F; f += nt) perm[f] = f;
+        __syncthreads();
+        if (tid == 0) {
+            for (int i = F - 1; i >= 1; --i) {
+                const int j = shuffle_partner(stream, F, i);
+                const int32_t t = perm[i];
+                perm[i] = perm[j];
+                perm[j] = t;
+            }
+        }
+        __syncthreads();
+        for (int f = tid; f < F; f += nt) write(f, perm[f]);
         return;
     }
-    // WS: Fisher-Yates from the last index down, draw (F-1-i) picks j = floor(u (i+1))
-    int32_t *perm = a.perm + jb.perm_off;
-    for (int f = threadIdx.x; f < jb.F; f += blockDim.x) perm[f] = f;
+    int *head = sh, *link = sh + F;
+    for (int f = tid; f < F; f += nt) head[f] = -1;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = jb.F - 1; i >= 1; --i) {
-            const uint64_t x = splitmix64(stream, (uint64_t)(jb.F - 1 - i));
-            const double u = (double)(x >> 11) * (1.0 / 9007199254740992.0);
-            int jj = (int)(u * (double)(i + 1));
-            if (jj > i) jj = i;
-            const int32_t t = perm[i];
-            perm[i] = perm[jj];
-            perm[jj] = t;
+    for (int i = 1 + tid; i < F; i += nt) link[i] = atomicExch(head + shuffle_partner(stream, F, i), i);
+    __syncthreads();
+    // the smallest step above i into place p (-1: none)
+    auto next = [&](int p, int i) {
+        int best = -1;
+        for (int e = head[p]; e >= 0; e = link[e])
+            if (e > i && (best < 0 || e < best)) best = e;
+        return best;
+    };
+    // perm: A's chain; out (this thread's own places, as bits): the result's start, an index of
+    // A or ~value
+    for (int i = tid; i < F; i += nt) {
+        perm[i] = next(i, i);
+        int start = 0;
+        if (i > 0) {
+            const int j = shuffle_partner(stream, F, i), e = next(j, i);
+            start = e >= 0 ? e : ~j;
         }
+        out[i] = __int_as_float(start);
     }
     __syncthreads();
-    for (int f = threadIdx.x; f < jb.F; f += blockDim.x) {
-        const float wp = __ldg(w + perm[f]);
-        out[f] = a.ws_as_weights ? wp : wp - __ldg(w + f);
+    for (int f = tid; f < F; f += nt) head[f] = perm[f];
+    __syncthreads();
+    for (int f = tid; f < F; f += nt) {
+        const int start = __float_as_int(out[f]);
+        int v = ~start;
+        if (start >= 0)
+            for (v = start; head[v] >= 0;) v = head[v];
+        write(f, v);
     }
 }
 
 int launch_expand(const ExpandArgs &ea, cudaStream_t s)
 {
-    if (ea.n_jobs <= 0) return 0;
     int launches = 0;
+    const int f_ws = ea.max_ws <= kShuffleMax ? ea.max_ws : kShuffleMax;
     for (int64_t j0 = 0; j0 < ea.n_jobs; j0 += 65535) {
         ExpandArgs a = ea;
         a.jobs = ea.jobs + j0;
-        const int64_t n = ea.n_jobs - j0 < 65535 ? ea.n_jobs - j0 : 65535;
-        k_expand<<<(unsigned)n, 256, 0, s>>>(a);
-        ++launches;
+        const unsigned n = (unsigned)(ea.n_jobs - j0 < 65535 ? ea.n_jobs - j0 : 65535);
+        if (ea.max_gf > 0) {
+            const int chunks = (ea.max_gf - 1) / kExpandValues + 1;
+            k_expand_gf<<<dim3(n, (unsigned)std::min(chunks, 1024)), kExpandValues / 2, 0, s>>>(a);
+            ++launches;
+        }
+        if (ea.max_ws > 0) {
+            const int smem = 2 * f_ws * (int)sizeof(int);
+            cudaFuncSetAttribute(k_expand_ws, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            k_expand_ws<<<n, f_ws > 1024 ? 1024 : 256, smem, s>>>(a);
+            ++launches;
+        }
     }
     return launches;
 }

@@ -125,10 +125,11 @@ mure_status expand_noalloc(mure_ctx *c, mure_model *m, const mure_mutant *table,
     ea.sigma = m->sigma_dev;
     ea.W = reinterpret_cast<const float *const *>(scratch + o_w);
     ea.patch = out_dev;
-    // the kernel initialises every permutation entry it reads, so nothing in the
+    // the kernels initialise every permutation entry they read, so nothing in the
     // scratch has to start at zero or survives from an earlier call
     ea.perm = reinterpret_cast<int32_t *>(scratch + o_perm);
     ea.ws_as_weights = 1;
+    ea.bounds(jobs);
     c->launches += mure::launch_expand(ea, c->stream);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -164,6 +164,28 @@ def test_expanded_patches_bitexact(M, ctx, oracle_mod):
         assert mism <= max(1, total // 1_000_000), (mism, total)
 
 
+@pytest.mark.parametrize("fan", [1, 2, 33, 1025, 25000, 25001])
+def test_expansion_at_fan_in_edges(M, ctx, oracle_mod, fan):
+    """The shuffle without the chain of swaps (up to 25,000 weights, 256 or 1024 threads) and the
+    serial one above, and the noise's pairs and blocks, against the oracle."""
+    model = wl.mlp(4, (fan, 3, 2))
+    rows = [(0, "WS", [2, 0], 0.0, 77), (0, "GF", [1], 0.1, 78), (1, "WS", [1], 0.0, 79), (1, "GF", [0, 1], 0.1, 80)]
+    table = wl.table_from_rows(rows)
+    vals, offs = M.mure_expand_patches(M.mure_model_load(ctx, model), table)
+    for i, (l, op, ids, _, seed) in enumerate(rows):
+        nd = model.nodes[model.layers()[l]]
+        got = vals[offs[i]:offs[i] + len(ids) * nd.cin].reshape(len(ids), nd.cin)
+        if op == "WS":
+            Wm, _, _ = oracle_mod.mutant_layer(model, table, i)
+            assert np.array_equal(got, Wm.reshape(nd.cout, -1)[ids])
+        else:
+            sigma = float(np.float32(0.1)) * oracle_mod.layer_std(model, l)
+            exp = np.array([[np.float32(sigma * oracle_mod.gauss(oracle_mod.sm64(seed, q), f)) for f in range(nd.cin)]
+                            for q in range(len(ids))], np.float32)
+            # the fp64 results differ in their last bit at most, fp32 then in one unit at most
+            assert (got != exp).mean() <= 1e-3 and np.allclose(got, exp, rtol=2.0 ** -23, atol=0)
+
+
 @pytest.mark.parametrize("prec", PRECISIONS)
 def test_batch_invariance(M, ctx, prec):
     """Tiny workspaces force many batches (input tiles, mutant chunks): results are
