@@ -61,6 +61,28 @@ def test_depthwise_network_matches_oracle(M, ctx, case, prec):
     assert np.array_equal(u["logits"].view(np.uint32), r["logits"].view(np.uint32))
 
 
+@pytest.mark.parametrize("h,w,c,stride,pad,k", [(13, 11, 20, 1, 1, 3), (12, 9, 36, 2, 1, 3), (17, 16, 12, 2, 0, 3),
+                                                (16, 18, 8, 1, 2, 3), (6, 5, 8, 1, 1, 3), (14, 13, 18, 1, 1, 3),
+                                                (14, 13, 16, 1, 2, 5)])
+def test_depthwise_kernel_edges(M, ctx, oracle_mod, h, w, c, stride, pad, k):
+    """The 3 x 3 kernel of channels in fours (ragged output groups, both strides, every padding)
+    and the shapes that stay on the thread-per-output kernel, against the oracle and vanilla."""
+    b = wl._Builder("dw_edge", (h, w, 3), 5, 11)
+    x = b.conv(-1, c, 1)
+    x = b.dwconv(x, k, stride=stride, pad=pad)
+    x = b.gap(b.conv(x, 16, 1))
+    b.dense(x, 5, act="none")
+    X = wl.inputs(b.m, 67, 3)
+    table = wl.mutants(b.m, 16, seed=5, ratios=(0.1,), ops=("GF", "NS", "NAI", "WS"))
+    ora = oracle_mod.vanilla(b.m, X, table)
+    m = M.mure_model_load(ctx, b.m, precision="fp32")
+    r = M.mure_eval_mutants(M.mure_build_prefix_cache(m, X), table, logits=True)
+    ok, worst = logits_close(r["logits"], ora["logits"])
+    assert ok, worst
+    v = M.mure_eval_vanilla(m, X, table, logits=True)
+    assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
 def test_depthwise_identity_mutants(M, ctx):
     model = wl.mobilenetv2_tiny()
     X = wl.inputs(model, 64, 1)
