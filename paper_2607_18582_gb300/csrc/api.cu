@@ -685,7 +685,7 @@ struct Workspace {
     LstmWs lw;                 // a mutated LSTM layer's scratch (lw.proj = tmp)
     int64_t rows = 0;
     TcDeltaWs dw;              // tensor-core delta scratch (GF / WS slots of a batch)
-    // unchanged-row elimination: per-row flags, per-block counts, the compacted row
+    // unchanged-row elimination: per-row flags, counts per 32 rows, the compacted row
     // list and its length
     int32_t *uflags = nullptr, *ublk = nullptr, *lrow = nullptr, *ucount = nullptr;
 };
@@ -1215,7 +1215,7 @@ void evaluate(mure_ctx *c, const mure_model *m, const mure_cache *ca, const mure
         if (!vanilla && o->skip_unchanged) {
             ec.skip_unchanged = true;
             ws.uflags = sc.get<int32_t>(rows);
-            ws.ublk = sc.get<int32_t>(rows / 256 + 1);
+            ws.ublk = sc.get<int32_t>(rows / 32 + 1);
             ws.lrow = sc.get<int32_t>(rows);
             ws.ucount = sc.get<int32_t>(1);
             // compacted batches OR their kill bits in

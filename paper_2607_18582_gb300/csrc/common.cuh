@@ -345,7 +345,7 @@ int launch_layer_std(const float *const *W, const int64_t *n, int L, double *out
 // original forward pass, so its kill bit is 0 and its logits are the cached original
 // logits (written to logits_out when requested; its near tie is counted from them).
 // flags[r] = 1 for the rows still to run; lrow receives them in ascending order and
-// count their number.  Scratch: block_cnt of ceil(R / 256) ints.
+// count their number.  Scratch: group_cnt of ceil(R / 32) ints.
 struct UnchangedArgs {
     const float *patch;          // [R][kmax][cells] the delta's values
     int64_t row_stride;
@@ -360,7 +360,7 @@ struct UnchangedArgs {
     int C;
     FinalArgs fa;                // logits_out, near_ties, mutant ids, n_in
 };
-int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t *block_cnt, int32_t *lrow,
+int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t *group_cnt, int32_t *lrow,
                      int32_t *count, cudaStream_t s);
 
 // Score reduction: per mutant killed flag and |killingLabels|, summed.

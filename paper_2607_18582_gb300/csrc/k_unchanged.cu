@@ -14,20 +14,24 @@ namespace mure {
 
 namespace {
 
-constexpr int kRowsPerBlock = 256;   // 8 warps x 32 rows
+constexpr int kGroup = 32;   // rows per block of the flags kernel and per entry of the counts
 
-// One warp per row (32 rows per warp in turn): flags[r] = 1 for a row to run, 0 for
-// an unchanged row or a padding input; block_cnt[b] = the rows to run of block b.
+// One warp per row (4 rows per warp in turn): flags[r] = 1 for a row to run, 0 for an
+// unchanged row or a padding input; group_cnt[b] = the rows to run of block b.  Most rows
+// differ within the first cells, so the comparison stops at the first chunk that does; a chunk
+// keeps four loads of each side in flight per lane.  Few rows per block, since a batch has
+// only thousands of them (256 per block and whole channels compared: 183 us for 2,000 rows of
+// a 32 x 32 map, now 10).
 __global__ void __launch_bounds__(256) k_unchanged_flags(const UnchangedArgs ua, int64_t t0, int T, int R,
-                                                         int32_t *flags, int32_t *block_cnt)
+                                                         int32_t *flags, int32_t *group_cnt)
 {
     __shared__ int cnt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) cnt = 0;
     __syncthreads();
     int mine = 0;
-    for (int i = 0; i < 32; ++i) {
-        const int64_t r = (int64_t)blockIdx.x * kRowsPerBlock + warp * 32 + i;
+    for (int i = 0; i < kGroup / 8; ++i) {
+        const int64_t r = (int64_t)blockIdx.x * kGroup + warp * (kGroup / 8) + i;
         if (r >= R) break;
         const int g = (int)(r / T);
         const int64_t t = t0 + r % T;
@@ -40,10 +44,17 @@ __global__ void __launch_bounds__(256) k_unchanged_flags(const UnchangedArgs ua,
             bool same = true;
             for (int q = 0; q < k && same; ++q) {
                 const int j = ids[q];
-                for (int c = lane; c < ua.cells; c += 32)
-                    same &= __float_as_uint(__ldg(prow + (int64_t)q * ua.cells + c)) ==
-                            __float_as_uint(__ldg(orig + (int64_t)c * ua.ch + j));
-                same = __all_sync(0xffffffffu, same);
+                for (int c0 = 0; c0 < ua.cells && same; c0 += 128) {
+                    bool eq = true;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int c = c0 + 32 * u + lane;
+                        if (c < ua.cells)
+                            eq &= __float_as_uint(__ldg(prow + (int64_t)q * ua.cells + c)) ==
+                                  __float_as_uint(__ldg(orig + (int64_t)c * ua.ch + j));
+                    }
+                    same = __all_sync(0xffffffffu, eq);
+                }
             }
             run = same ? 0 : 1;
             if (same) {
@@ -65,63 +76,58 @@ __global__ void __launch_bounds__(256) k_unchanged_flags(const UnchangedArgs ua,
     }
     if (lane == 0 && mine) atomicAdd(&cnt, mine);
     __syncthreads();
-    if (threadIdx.x == 0) block_cnt[blockIdx.x] = cnt;
+    if (threadIdx.x == 0) group_cnt[blockIdx.x] = cnt;
 }
 
-// Exclusive scan of the block counts (one block); count = their sum.
-__global__ void __launch_bounds__(1024) k_unchanged_scan(int32_t *block_cnt, int nb, int32_t *count)
+// Exclusive scan of the group counts (one block); count = their sum.
+__global__ void __launch_bounds__(1024) k_unchanged_scan(int32_t *group_cnt, int ng, int32_t *count)
 {
-    __shared__ int32_t part[1024];
-    __shared__ int32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < nb; base += 1024) {
-        const int i = base + threadIdx.x;
-        const int32_t v = i < nb ? block_cnt[i] : 0;
-        part[threadIdx.x] = v;
-        __syncthreads();
-        // Hillis-Steele inclusive scan of the chunk
-        for (int off = 1; off < 1024; off <<= 1) {
-            const int32_t add = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-            __syncthreads();
-            part[threadIdx.x] += add;
-            __syncthreads();
+    __shared__ int32_t part[32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto warp_scan = [&](int32_t v) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t n = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += n;
         }
-        if (i < nb) block_cnt[i] = carry + part[threadIdx.x] - v;
+        return v;
+    };
+    int32_t carry = 0;
+    for (int base = 0; base < ng; base += 1024) {
+        const int i = base + threadIdx.x;
+        const int32_t v = i < ng ? group_cnt[i] : 0;
+        const int32_t incl = warp_scan(v);
+        if (lane == 31) part[warp] = incl;
         __syncthreads();
-        if (threadIdx.x == 1023) carry += part[1023];
+        if (warp == 0) part[lane] = warp_scan(part[lane]);
+        __syncthreads();
+        if (i < ng) group_cnt[i] = carry + (warp > 0 ? part[warp - 1] : 0) + incl - v;
+        carry += part[31];
         __syncthreads();
     }
     if (threadIdx.x == 0) *count = carry;
 }
 
-// lrow[offset of block b + rank of r among its block's rows to run] = r.
-__global__ void __launch_bounds__(256) k_unchanged_compact(const int32_t *flags, const int32_t *block_off, int R,
+// lrow[offset of r's group + rank of r among the group's rows to run] = r; a warp per group.
+__global__ void __launch_bounds__(256) k_unchanged_compact(const int32_t *flags, const int32_t *group_off, int R,
                                                            int32_t *lrow)
 {
-    __shared__ int32_t warp_cnt[8];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int32_t total = 0;
-    // rows of warp w: 32 consecutive groups of 32 rows? no: row = block * 256 + w * 32 + i
-    // (the flags kernel's order); each lane takes row i = lane
-    const int64_t r = (int64_t)blockIdx.x * kRowsPerBlock + warp * 32 + lane;
+    const int lane = threadIdx.x & 31;
+    const int64_t grp = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5), r = grp * kGroup + lane;
     const int f = r < R ? flags[r] : 0;
     const unsigned b = __ballot_sync(0xffffffffu, f);
-    if (lane == 0) warp_cnt[warp] = __popc(b);
-    __syncthreads();
-    for (int w = 0; w < warp; ++w) total += warp_cnt[w];
-    if (f) lrow[block_off[blockIdx.x] + total + __popc(b & ((1u << lane) - 1u))] = (int32_t)r;
+    if (f) lrow[group_off[grp] + __popc(b & ((1u << lane) - 1u))] = (int32_t)r;
 }
 
 }  // namespace
 
-int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t *block_cnt, int32_t *lrow,
+int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t *group_cnt, int32_t *lrow,
                      int32_t *count, cudaStream_t s)
 {
-    const int nb = (rm.R + kRowsPerBlock - 1) / kRowsPerBlock;
-    k_unchanged_flags<<<nb, 256, 0, s>>>(ua, rm.t0, rm.T, rm.R, flags, block_cnt);
-    k_unchanged_scan<<<1, 1024, 0, s>>>(block_cnt, nb, count);
-    k_unchanged_compact<<<nb, 256, 0, s>>>(flags, block_cnt, rm.R, lrow);
+    const int ng = (rm.R + kGroup - 1) / kGroup;
+    k_unchanged_flags<<<ng, 256, 0, s>>>(ua, rm.t0, rm.T, rm.R, flags, group_cnt);
+    k_unchanged_scan<<<1, 1024, 0, s>>>(group_cnt, ng, count);
+    k_unchanged_compact<<<(ng + 7) / 8, 256, 0, s>>>(flags, group_cnt, rm.R, lrow);
     return 3;
 }
 
