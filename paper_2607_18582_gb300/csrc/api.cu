@@ -1107,6 +1107,12 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
         timed(l + 1, 2 * Sn.macs * rm.R, [&] {
             return launch_conv_small(Sn, base, rm, nullptr, 0, ws.xb[l + 2], m->xd[l + 2].stride, s, &ov);
         });
+    } else if (!skip_reader && simt_overlay_inline(Sn, ov, base)) {
+        acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[l + 2].size * 4;
+        timed(l + 1, 2 * Sn.macs * rm.R, [&] {
+            return launch_stage_simt(Sn, base, rm, nullptr, 0, skip_of(Sn), ws.xb[l + 2], m->xd[l + 2].stride, ws.tmp, s,
+                                     &ov);
+        });
     } else {
         acct.bytes_gather += 2 * (int64_t)rm.R * m->xd[l + 1].size * 4;
         timed(C_DELTA, 0, [&] {

@@ -155,7 +155,9 @@ struct Overlay {
 // Stage v over R rows: z (optional) and y = post(act1(conv(x) + b)).  tmp: the stage's row
 // scratch (the map before global average pooling; an LSTM's input sums).
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip,
-                      float *y_out, int64_t y_stride, float *tmp, cudaStream_t s);
+                      float *y_out, int64_t y_stride, float *tmp, cudaStream_t s, const Overlay *ov = nullptr);
+// Whether the CUDA-core stage kernel applies the overlay as it fetches rows of x.
+int simt_overlay_inline(const Stage &S, const Overlay &ov, Src x);
 
 // The shared-memory direct convolution for small inputs (variant of a stage, 0 when
 // the geometry is not one it compiles) and its launcher.

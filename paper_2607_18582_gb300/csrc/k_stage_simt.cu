@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "device_util.cuh"
 #include "epilogue.cuh"
+#include "simt_tile.cuh"
 
 namespace mure {
 
@@ -28,129 +29,222 @@ struct StageParams {
     int P;   // GEMM rows per batch row: oh*ow, ordered (oy, ox), or with pooling
              // 4 * (oh/2) * (ow/2) ordered (py, px, dy, dx)
     int pw;  // pooled width
+    int n_tiles;   // column tiles (blockIdx.x: row tile * n_tiles + column tile)
+    int vec;       // 16-byte stores of y: channels in fours on 16-byte rows
+    Overlay ov;    // mutated channels of the input rows (ov.patch null: none)
 };
 
-template <int BN>
-__global__ void __launch_bounds__(256) k_stage_simt(const StageParams p)
+// Implicit-GEMM convolution / dense on the CUDA cores: BM rows (positions) x BN output
+// channels per block, TM x TN sums per thread (simt_tile.cuh), operand tiles
+// double-buffered in shared memory, the next pieces in flight while the current are used.  A4: the
+// input channels come in fours on 16-byte rows, so a thread fetches four k of its row at once.
+// OV (with A4 only): a fetched piece takes the mutated channels from the patch.
+template <int BM, int BN, int TM, int TN, bool A4, bool OV>
+__global__ void __launch_bounds__(BM / TM * (BN / TN), A4 && !OV && BN != 64 ? 4 : 3) k_stage_simt(const StageParams p)
 {
-    constexpr int BM = 4096 / BN, BK = 16;
-    constexpr int A_SPLIT = 256 / BM, A_PER = BK / A_SPLIT;
-    constexpr int B_SPLIT = 256 / BN, B_PER = BK / B_SPLIT;
-    __shared__ __align__(16) float As[BK][BM];
-    __shared__ __align__(16) float Bs[BK][BN];
-
+    constexpr int BK = 8, CT = BN / TN, RT = BM / TM, NT = CT * RT;
+    constexpr int RS = BM / (TM / 4), CS = BN / (TN / 4);
+    constexpr int A4N = BM * BK / 4 / NT, B4N = (BK * BN / 4 + NT - 1) / NT;
+    __shared__ __align__(16) float2 As[2][BK][BM];
+    __shared__ __align__(16) float Bs[2][BK][BN];
     const int tid = threadIdx.x;
-    const int tn = tid % (BN / 4), tm = tid / (BN / 4);
-    const int64_t M = (int64_t)p.R * p.P;
-    const int64_t m0 = (int64_t)blockIdx.x * BM;
-    const int n0 = blockIdx.y * BN;
-
-    // this thread's A-load row
-    const int m_l = tid % BM, kl0 = (tid / BM) * A_PER;
-    const int64_t m = m0 + m_l;
-    const bool valid_m = m < M;
-    int iy0 = 0, ix0 = 0;
-    const float *xrow = p.x;
-    if (valid_m) {
-        const int64_t row = m / p.P;
-        const int q = (int)(m % p.P);
-        int oy, ox;
+    constexpr int CL = CT < 8 ? CT : 8, RL = 32 / CL;
+    const int warp = tid >> 5, lane = tid & 31;
+    const int tn = (warp % (CT / CL)) * CL + lane % CL, tm = (warp / (CT / CL)) * RL + lane / CL;
+    const unsigned mt = blockIdx.x / (unsigned)p.n_tiles;
+    const int n0 = (int)(blockIdx.x - mt * p.n_tiles) * BN;
+    // the tile's first batch row and position
+    const int64_t m0 = (int64_t)mt * BM, row0 = m0 / p.P;
+    const unsigned q0 = (unsigned)(m0 - row0 * p.P);
+    auto place = [&](int i, int64_t &row, int &py, int &px, int &oy, int &ox) {
+        const unsigned qq = q0 + i, dr = qq / (unsigned)p.P, q = qq - dr * p.P;
+        row = row0 + dr;
         if (p.pool) {
-            const int w = q >> 2, sub = q & 3;
-            oy = 2 * (w / p.pw) + (sub >> 1);
-            ox = 2 * (w % p.pw) + (sub & 1);
+            const unsigned w = q >> 2, sub = q & 3;
+            py = w / (unsigned)p.pw;
+            px = w - py * p.pw;
+            oy = 2 * py + (sub >> 1);
+            ox = 2 * px + (sub & 1);
         } else {
-            oy = q / p.ow;
-            ox = q % p.ow;
+            py = px = 0;
+            oy = q / (unsigned)p.ow;
+            ox = q - oy * p.ow;
         }
-        iy0 = oy * p.stride - p.pad;
-        ix0 = ox * p.stride - p.pad;
-        xrow = p.x + (p.x_per_input ? (p.t0 + logical_row(p.lrow, row) % p.T) : row) * p.x_stride;
+    };
+    // this thread's A row: tid % BM
+    const float *xrow = nullptr, *ov_row = nullptr;
+    int iy0 = 0, ix0 = 0, ov_n = 0;
+    const int32_t *ov_ids = nullptr;
+    {
+        int64_t row;
+        int py, px, oy, ox;
+        place(tid % BM, row, py, px, oy, ox);
+        if (row < p.R) {
+            iy0 = oy * p.stride - p.pad;
+            ix0 = ox * p.stride - p.pad;
+            const int64_t lr = logical_row(p.lrow, row);
+            xrow = p.x + (p.x_per_input ? p.t0 + lr % p.T : row) * p.x_stride;
+            if (OV) {
+                const int g = (int)(lr / p.T);
+                ov_n = p.ov.n_neurons[g];
+                ov_ids = p.ov.ids + p.ov.neuron_off[g];
+                ov_row = p.ov.patch + lr * p.ov.row_stride;
+            }
+        }
     }
-    const int n_l = tid % BN, kb0 = (tid / BN) * B_PER;
-
-    float acc[4][4];
+    float4 ra[A4N], rb[B4N];
+    // where this thread's next A pieces stand in the fan-in: channel and tap, advanced by BK a
+    // tile (a division per piece and tile took longer than the tile's FMAs)
+    int ci[A4N] = {}, kx[A4N] = {}, ky[A4N] = {};
+    auto carry = [&](int i) {
+        while (ci[i] >= p.ic) {
+            ci[i] -= p.ic;
+            if (++kx[i] == p.kw) { kx[i] = 0; ++ky[i]; }
+        }
+    };
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < A4N; ++i) {
+        kx[i] = ky[i] = 0;
+        ci[i] = 4 * (tid / BM + i * (NT / BM));
+        carry(i);
+    }
+    auto load = [&](int k0) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-    for (int k0 = 0; k0 < p.K; k0 += BK) {
-        {
-            int k = k0 + kl0;
-            int ci = k % p.ic, t = k / p.ic, kx = t % p.kw, ky = t / p.kw;
+        for (int i = 0; i < A4N; ++i) {
+            float v[4] = {0.f, 0.f, 0.f, 0.f};
+            if (xrow && ky[i] < p.kh) {
+                if (A4) {
+                    const int iy = iy0 + ky[i], ix = ix0 + kx[i];
+                    if ((unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw) {
+                        const int e = (iy * p.iw + ix) * p.ic + ci[i];
+                        *reinterpret_cast<float4 *>(v) = __ldg(reinterpret_cast<const float4 *>(xrow + e));
+                        if (OV && ov_n > 0) {
+                            const int c = e / p.ov.ch, j = e - c * p.ov.ch;   // four channels of one cell
+                            for (int q = 0; q < ov_n; ++q) {
+                                const int d = __ldg(ov_ids + q) - j;
 #pragma unroll
-            for (int i = 0; i < A_PER; ++i) {
-                float v = 0.f;
-                if (valid_m && k + i < p.K) {
-                    const int iy = iy0 + ky, ix = ix0 + kx;
-                    if ((unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw)
-                        v = __ldg(xrow + ((int64_t)iy * p.iw + ix) * p.ic + ci);
+                                for (int u = 0; u < 4; ++u)
+                                    if (d == u) v[u] = __ldg(ov_row + q * p.ov.cells + c);
+                            }
+                        }
+                    }
+                } else {
+                    int c = ci[i], x = kx[i], y = ky[i];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int iy = iy0 + y, ix = ix0 + x;
+                        if (y < p.kh && (unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw)
+                            v[u] = __ldg(xrow + ((int64_t)iy * p.iw + ix) * p.ic + c);
+                        if (++c == p.ic) { c = 0; if (++x == p.kw) { x = 0; ++y; } }
+                    }
                 }
-                As[kl0 + i][m_l] = v;
-                if (++ci == p.ic) { ci = 0; if (++kx == p.kw) { kx = 0; ++ky; } }
+            }
+            ra[i] = make_float4(v[0], v[1], v[2], v[3]);
+            ci[i] += BK;
+            carry(i);
+        }
+#pragma unroll
+        for (int i = 0; i < B4N; ++i) {
+            const int e = tid + i * NT, k = k0 + e / (BN / 4), n = n0 + 4 * (e % (BN / 4));
+            rb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (e < BK * BN / 4 && k < p.K && n < p.oc) {
+                const float *w = p.Wt + (int64_t)k * p.oc + n;
+                if ((p.oc & 3) == 0) {
+                    rb[i] = __ldg(reinterpret_cast<const float4 *>(w));
+                } else {
+                    rb[i].x = __ldg(w);
+                    if (n + 1 < p.oc) rb[i].y = __ldg(w + 1);
+                    if (n + 2 < p.oc) rb[i].z = __ldg(w + 2);
+                    if (n + 3 < p.oc) rb[i].w = __ldg(w + 3);
+                }
             }
         }
+    };
+    auto store = [&](int s) {
 #pragma unroll
-        for (int i = 0; i < B_PER; ++i) {
-            const int k = k0 + kb0 + i, n = n0 + n_l;
-            Bs[kb0 + i][n_l] = (k < p.K && n < p.oc) ? __ldg(p.Wt + (int64_t)k * p.oc + n) : 0.f;
+        for (int i = 0; i < A4N; ++i) {
+            const int k = 4 * (tid / BM + i * (NT / BM)), r = tid % BM;
+            As[s][k][r] = make_float2(ra[i].x, ra[i].x);
+            As[s][k + 1][r] = make_float2(ra[i].y, ra[i].y);
+            As[s][k + 2][r] = make_float2(ra[i].z, ra[i].z);
+            As[s][k + 3][r] = make_float2(ra[i].w, ra[i].w);
         }
-        __syncthreads();
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            const float4 a = *reinterpret_cast<const float4 *>(&As[kk][tm * 4]);
-            const float4 b = *reinterpret_cast<const float4 *>(&Bs[kk][tn * 4]);
-            const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int i = 0; i < B4N; ++i) {
+            const int e = tid + i * NT;
+            if (e < BK * BN / 4) *reinterpret_cast<float4 *>(&Bs[s][e / (BN / 4)][4 * (e % (BN / 4))]) = rb[i];
         }
+    };
+    f32x2 acc[TM][TN / 2];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0;
+    load(0);
+    store(0);
+    __syncthreads();
+    int s = 0;
+    for (int k0 = 0; k0 < p.K; k0 += BK, s ^= 1) {
+        const bool more = k0 + BK < p.K;
+        if (more) load(k0 + BK);
+        simt_tile_fma<BK, BM, BN, TM, TN, RS, CS>(acc, &As[s][0][tm * 4], &Bs[s][0][tn * 4]);
+        if (more) store(s ^ 1);
         __syncthreads();
     }
-
-    // epilogue: bias, activation, skip, pooling
-    const int64_t mb = m0 + tm * 4;
+    // epilogue: bias, activation, skip, pooling; rows i .. i + 3 of a group of four are one
+    // pooling window
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int n = n0 + tn * 4 + j;
+    for (int jj = 0; jj < TN; jj += 4) {
+        const int n = n0 + (jj / 4) * CS + tn * 4;
         if (n >= p.oc) continue;
-        const float bias = __ldg(p.b + n);
-        float win[4];
-        int64_t row = 0;
-        int py = 0, px = 0;
+        float bias[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int64_t mm = mb + i;
-            win[i] = 0.f;
-            if (mm >= M) continue;
-            row = mm / p.P;
-            const int q = (int)(mm % p.P);
-            int oy, ox;
-            if (p.pool) {
-                const int w = q >> 2, sub = q & 3;
-                py = w / p.pw; px = w % p.pw;
-                oy = 2 * py + (sub >> 1);
-                ox = 2 * px + (sub & 1);
-            } else {
-                oy = q / p.ow;
-                ox = q % p.ow;
+        for (int e = 0; e < 4; ++e) bias[e] = n + e < p.oc ? __ldg(p.b + n + e) : 0.f;
+#pragma unroll
+        for (int ii = 0; ii < TM; ii += 4) {
+            float win[4][4];
+            float *yw = nullptr;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int64_t row;
+                int py, px, oy, ox;
+                place((ii / 4) * RS + tm * 4 + i, row, py, px, oy, ox);
+                if (row >= p.R) continue;
+                const float2 lo = unpack2(acc[ii + i][jj / 2]), hi = unpack2(acc[ii + i][jj / 2 + 1]);
+                float v[4] = {lo.x + bias[0], lo.y + bias[1], hi.x + bias[2], hi.y + bias[3]};
+                const float *sr = nullptr;
+                if (p.has_add)
+                    sr = p.skip + (p.skip_per_input ? p.t0 + logical_row(p.lrow, row) % p.T : row) * p.skip_stride +
+                         ((int64_t)oy * p.sk_stride * p.sk_w + ox * p.sk_stride) * p.sk_c + n;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (n + e >= p.oc) continue;
+                    if (p.z) p.z[row * p.z_stride + (int64_t)(n + e) * (p.oh * p.ow) + oy * p.ow + ox] = v[e];   // channel-major
+                    v[e] = act_apply(p.act1, v[e]);
+                    if (p.has_add) v[e] = act_apply(p.act2, v[e] + (n + e < p.sk_c ? __ldg(sr + e) : 0.f));
+                }
+                float *yr = p.y + row * p.y_stride + n;
+                if (p.pool) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) win[i][e] = v[e];
+                    yw = yr + ((int64_t)py * p.pw + px) * p.oc;
+                    continue;
+                }
+                yr += ((int64_t)oy * p.ow + ox) * p.oc;
+                if (p.vec) {
+                    *reinterpret_cast<float4 *>(yr) = make_float4(v[0], v[1], v[2], v[3]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (n + e < p.oc) yr[e] = v[e];
+                }
             }
-            const float z = acc[i][j] + bias;
-            if (p.z) p.z[row * p.z_stride + (int64_t)n * (p.oh * p.ow) + oy * p.ow + ox] = z;  // channel-major
-            float v = act_apply(p.act1, z);
-            if (p.has_add) {
-                const float *sr =
-                    p.skip + (p.skip_per_input ? (p.t0 + logical_row(p.lrow, row) % p.T) : row) * p.skip_stride;
-                const float s = n < p.sk_c ? sr[((int64_t)oy * p.sk_stride * p.sk_w + ox * p.sk_stride) * p.sk_c + n] : 0.f;
-                v = act_apply(p.act2, v + s);
+            if (p.pool && yw) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (n + e < p.oc) yw[e] = max4_first(win[0][e], win[1][e], win[2][e], win[3][e]);
             }
-            if (p.pool) win[i] = v;
-            else p.y[row * p.y_stride + ((int64_t)oy * p.ow + ox) * p.oc + n] = v;
         }
-        if (p.pool && mb < M)
-            p.y[row * p.y_stride + ((int64_t)py * p.pw + px) * p.oc + n] = max4_first(win[0], win[1], win[2], win[3]);
     }
 }
 
@@ -267,8 +361,30 @@ __global__ void __launch_bounds__(256) k_dwconv3(const StageParams p, int c4n, i
         }
 }
 
+namespace {
+
+bool aligned16(const void *q, int64_t stride) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0 && stride % 4 == 0; }
+
+template <int BM, int BN, int TM, int TN>
+void stage_tiles(StageParams p, bool a4, cudaStream_t s)
+{
+    p.n_tiles = (p.oc + BN - 1) / BN;
+    const int64_t tiles = ((int64_t)p.R * p.P + BM - 1) / BM * p.n_tiles;
+    if (p.ov.patch) k_stage_simt<BM, BN, TM, TN, true, true><<<(unsigned)tiles, BM / TM * (BN / TN), 0, s>>>(p);
+    else if (a4) k_stage_simt<BM, BN, TM, TN, true, false><<<(unsigned)tiles, BM / TM * (BN / TN), 0, s>>>(p);
+    else k_stage_simt<BM, BN, TM, TN, false, false><<<(unsigned)tiles, BM / TM * (BN / TN), 0, s>>>(p);
+}
+
+}  // namespace
+
+int simt_overlay_inline(const Stage &S, const Overlay &ov, Src x)
+{
+    return !S.tc && S.variant == 0 && (S.kind == MURE_NODE_CONV2D || S.kind == MURE_NODE_DENSE) && S.ic % 4 == 0 &&
+           ov.ch % 4 == 0 && aligned16(x.p, x.stride);
+}
+
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out,
-                      int64_t y_stride, float *tmp, cudaStream_t s)
+                      int64_t y_stride, float *tmp, cudaStream_t s, const Overlay *ov)
 {
     if (rm.R <= 0) return 0;
     if (S.tc) return launch_tc(S, x, rm, z_out, z_stride, skip, y_out, y_stride, tmp, s);
@@ -290,11 +406,10 @@ int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
         // 3 x 3 filters, channels in fours on 16-byte rows, and at least half a block of 2 x 4
         // output groups per row (a block takes one row's groups; with fewer most of its threads
         // would idle); else a thread per output
-        auto aligned = [](const void *q, int64_t stride) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0 && stride % 4 == 0; };
         const int gx = (S.ow + 3) / 4, c4n = S.oc / 4;
         const int64_t units = (int64_t)((S.oh + 1) / 2) * gx * c4n, bpr = (units + 255) / 256;
         if (S.kh == 3 && S.kw == 3 && (S.stride == 1 || S.stride == 2) && S.oc % 4 == 0 && units >= 128 &&
-            bpr * rm.R < INT32_MAX && aligned(x.p, x.stride) && aligned(y_out, y_stride) && aligned(S.Wt, 0) && aligned(S.b, 0)) {
+            bpr * rm.R < INT32_MAX && aligned16(x.p, x.stride) && aligned16(y_out, y_stride) && aligned16(S.Wt, 0) && aligned16(S.b, 0)) {
             auto go = [&](auto kern) { kern<<<(unsigned)(bpr * rm.R), 256, 0, s>>>(p, c4n, gx, (int)units, (int)bpr); };
             if (S.stride == 1) go(k_dwconv3<1>);
             else go(k_dwconv3<2>);
@@ -322,18 +437,15 @@ int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     p.y_stride = S.gap ? map_stride : y_stride;
     p.pw = S.ow / 2;
     p.P = S.pool ? 4 * (S.oh / 2) * (S.ow / 2) : S.oh * S.ow;
-    const int64_t M = (int64_t)rm.R * p.P;
+    p.vec = S.oc % 4 == 0 && aligned16(p.y, p.y_stride);
+    if (ov) p.ov = *ov;
+    const bool a4 = S.ic % 4 == 0 && aligned16(x.p, x.stride);
     int launches = 1;
-    if (S.oc <= 16) {
-        dim3 g((unsigned)((M + 255) / 256), (unsigned)((S.oc + 15) / 16));
-        k_stage_simt<16><<<g, 256, 0, s>>>(p);
-    } else if (S.oc <= 32) {
-        dim3 g((unsigned)((M + 127) / 128), (unsigned)((S.oc + 31) / 32));
-        k_stage_simt<32><<<g, 256, 0, s>>>(p);
-    } else {
-        dim3 g((unsigned)((M + 63) / 64), (unsigned)((S.oc + 63) / 64));
-        k_stage_simt<64><<<g, 256, 0, s>>>(p);
-    }
+    // the narrowest tile that holds the outputs: padded columns cost as much as real ones
+    if (S.oc <= 16) stage_tiles<128, 16, 4, 4>(p, a4, s);
+    else if (S.oc <= 32) stage_tiles<128, 32, 8, 4>(p, a4, s);
+    else if (S.oc <= 64) stage_tiles<128, 64, 8, 8>(p, a4, s);
+    else stage_tiles<64, 128, 8, 8>(p, a4, s);
     if (S.gap) {
         const int64_t n = (int64_t)rm.R * S.oc;
         k_gap<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tmp, map_stride, mh * mw, S.oc, rm.R, y_out, y_stride);
