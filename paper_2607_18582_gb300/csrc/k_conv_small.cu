@@ -1,7 +1,6 @@
 // Direct convolution for layers whose per-row input fits in shared memory (the
 // LeNet-5 convolutions): a block stages whole zero-padded input rows and the layer's
-// weights in shared memory, and each thread computes a 2x2 pooling window (or four
-// positions) for every output channel.  The receptive-field offsets are compile-time
+// weights in shared memory, and each thread computes whole 2x2 pooling windows.  The receptive-field offsets are compile-time
 // constants, so the inner loop is loads with immediate offsets and FMAs.
 //
 // Arithmetic: every output element is the same fp32 chain as in k_stage_simt, i.e.
@@ -24,14 +23,143 @@ struct ConvSmallParams {
     int act1;
     float *z; int64_t z_stride;
     float *y; int64_t y_stride;
-    int rows_per_block, cells;
     Overlay ov;       // mutated channels of the input rows (ov.patch null: none)
 };
 
-// KH x KW filter, IC input channels, OC output channels (OCT of them per thread),
-// WP / HP padded input width / height, PAD zero padding, POOL: 2x2 max pool after
-// the activation.
-template <int KH, int KW, int IC, int OC, int OCT, int WP, int HP, int PAD, bool POOL>
+// The row part of a block, shared by the kernels below: where each of its rows' inputs are and
+// whose mutant the row is.
+struct SmallRows {
+    const float *src[32];
+    int g[32];
+};
+
+__device__ __forceinline__ void small_rows(const ConvSmallParams &p, SmallRows &sr, int64_t row0, int nrows)
+{
+    if ((int)threadIdx.x < nrows) {
+        const int64_t row = row0 + threadIdx.x;
+        sr.src[threadIdx.x] = p.x + (p.x_per_input ? (p.t0 + row % p.T) : row) * p.x_stride;
+        sr.g[threadIdx.x] = (int)(row / p.T);
+    }
+    __syncthreads();
+}
+
+// The mutants' channels of the staged input rows (line floats per staged pixel row, IC per pixel,
+// the image at (oy0, ox0)).
+template <int IC>
+__device__ __forceinline__ void small_overlay(const ConvSmallParams &p, const SmallRows &sr, int64_t row0, int nrows,
+                                              float *xs, int tile, int line, int oy0, int ox0)
+{
+    const int per_row = p.ov.kmax * p.ov.cells;
+    for (int i = threadIdx.x; i < nrows * per_row; i += blockDim.x) {
+        const int rl = i / per_row, rem = i - rl * per_row, q = rem / p.ov.cells, c = rem - q * p.ov.cells;
+        const int g = sr.g[rl];
+        if (q >= p.ov.n_neurons[g]) continue;
+        const int j = p.ov.ids[p.ov.neuron_off[g] + q];
+        const int py = c / p.iw, px = c - py * p.iw;
+        xs[rl * tile + (py + oy0) * line + (px + ox0) * IC + j] = p.ov.patch[(row0 + rl) * p.ov.row_stride + q * p.ov.cells + c];
+    }
+    __syncthreads();
+}
+
+// 5 x 5, 1 -> 6 channels, pad 2, on 28 x 28, pooled (LeNet's first layer).  A thread takes two
+// neighbouring pooling windows: their 6 x 8 input field sits in registers (24 8-byte loads) and
+// each tap's six weights serve 48 FMAs (a window per thread, reading its inputs tap by tap, was
+// bound by its shared-memory loads, 10 for 24 FMAs: 1.08 ms for 109,000 rows, now 0.78).  16 rows of 98 pairs per block
+// of 224 threads, seven rounds each; the staged lines are 36 floats, the image from column 4,
+// so that rows are staged in 16-byte pieces.
+constexpr int kC1Rows = 16, kC1Threads = 224, kC1Line = 36, kC1Tile = 32 * kC1Line;
+
+__global__ void __launch_bounds__(kC1Threads, 2) k_conv1_pairs(const ConvSmallParams p)
+{
+    extern __shared__ __align__(16) float sm[];
+    float *ws = sm;              // [25][8]
+    float *xs = sm + 25 * 8;     // [rows][32][36]
+    __shared__ SmallRows sr;
+    const int tid = threadIdx.x;
+    const int64_t row0 = (int64_t)blockIdx.x * kC1Rows;
+    const int nrows = (int)(p.R - row0 < kC1Rows ? p.R - row0 : kC1Rows);
+    small_rows(p, sr, row0, nrows);
+    for (int i = tid; i < 200; i += kC1Threads) ws[i] = (i & 7) < 6 ? __ldg(p.Wt + (i >> 3) * 6 + (i & 7)) : 0.f;
+    // whole lines of nine 16-byte pieces: zero borders, the image's seven pieces between
+#pragma unroll 4
+    for (int i = tid; i < nrows * 288; i += kC1Threads) {
+        const int rl = i / 288, e = i - rl * 288, y = e / 9, c = e - y * 9;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (y >= 2 && y < 30 && c >= 1 && c < 8)
+            v = __ldg(reinterpret_cast<const float4 *>(sr.src[rl] + (y - 2) * 28) + c - 1);
+        reinterpret_cast<float4 *>(xs)[i] = v;
+    }
+    __syncthreads();
+    if (p.ov.patch) small_overlay<1>(p, sr, row0, nrows, xs, kC1Tile, kC1Line, 2, 4);
+    for (int pr = tid; pr < nrows * 98; pr += kC1Threads) {
+        const int rl = pr / 98, w = pr - rl * 98, py = w / 7, pp = w - py * 7;
+        // inputs (2 py - 2 .. + 3, 4 pp - 2 .. + 5), staged from column 4 pp + 2
+        const float *xt = xs + rl * kC1Tile + 2 * py * kC1Line + 4 * pp + 2;
+        float x[6][8];
+#pragma unroll
+        for (int i = 0; i < 6; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; j += 2) {
+                const float2 v = *reinterpret_cast<const float2 *>(xt + i * kC1Line + j);
+                x[i][j] = v.x;
+                x[i][j + 1] = v.y;
+            }
+        float acc[2][4][6];   // output row, column, channel
+#pragma unroll
+        for (int d = 0; d < 2; ++d)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+                for (int n = 0; n < 6; ++n) acc[d][c][n] = 0.f;
+#pragma unroll
+        for (int ky = 0; ky < 5; ++ky)
+#pragma unroll
+            for (int kx = 0; kx < 5; ++kx) {
+                const float4 wa = *reinterpret_cast<const float4 *>(ws + (ky * 5 + kx) * 8);
+                const float2 wb = *reinterpret_cast<const float2 *>(ws + (ky * 5 + kx) * 8 + 4);
+                const float wv[6] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y};
+#pragma unroll
+                for (int d = 0; d < 2; ++d)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int n = 0; n < 6; ++n) acc[d][c][n] = fmaf(x[ky + d][kx + c], wv[n], acc[d][c][n]);
+            }
+        const int64_t row = row0 + rl;
+        float out[2][6];
+#pragma unroll
+        for (int n = 0; n < 6; ++n) {
+            const float bias = __ldg(p.b + n);
+            float v[2][4];
+#pragma unroll
+            for (int d = 0; d < 2; ++d)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[d][c] = acc[d][c][n] + bias;
+            if (p.z) {
+#pragma unroll
+                for (int d = 0; d < 2; ++d)
+                    *reinterpret_cast<float4 *>(p.z + row * p.z_stride + n * 784 + (2 * py + d) * 28 + 4 * pp) =
+                        make_float4(v[d][0], v[d][1], v[d][2], v[d][3]);
+            }
+#pragma unroll
+            for (int d = 0; d < 2; ++d)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) v[d][c] = act_apply(p.act1, v[d][c]);
+            out[0][n] = max4_first(v[0][0], v[0][1], v[1][0], v[1][1]);
+            out[1][n] = max4_first(v[0][2], v[0][3], v[1][2], v[1][3]);
+        }
+        float4 *y = reinterpret_cast<float4 *>(p.y + row * p.y_stride + (py * 14 + 2 * pp) * 6);
+        y[0] = make_float4(out[0][0], out[0][1], out[0][2], out[0][3]);
+        y[1] = make_float4(out[0][4], out[0][5], out[1][0], out[1][1]);
+        y[2] = make_float4(out[1][2], out[1][3], out[1][4], out[1][5]);
+    }
+}
+
+// The other geometry (5 x 5, 6 -> 16 channels on 14 x 14, LeNet's second layer): KH x KW filter,
+// IC input channels, OC output channels (OCT of them per thread), WP / HP padded input width /
+// height, PAD zero padding, POOL: 2x2 max pool after the activation; ROWS rows of CELLS windows
+// (or groups of four positions) per block.
+template <int KH, int KW, int IC, int OC, int OCT, int WP, int HP, int PAD, bool POOL, int ROWS, int CELLS>
 __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
 {
     constexpr int K = KH * KW * IC;
@@ -40,18 +168,11 @@ __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
     extern __shared__ __align__(16) float sm[];
     float *ws = sm;              // [K][OC]
     float *xs = sm + K * OC;     // [rows_per_block][TILE]
-    __shared__ const float *src_row[32];
-    __shared__ int row_g[32];
+    __shared__ SmallRows sr;
     const int tid = threadIdx.x;
-    const int64_t row0 = (int64_t)blockIdx.x * p.rows_per_block;
-    const int nrows = (int)(p.R - row0 < p.rows_per_block ? p.R - row0 : p.rows_per_block);
-    if (tid < nrows) {
-        const int64_t row = row0 + tid;
-        src_row[tid] = p.x + (p.x_per_input ? (p.t0 + row % p.T) : row) * p.x_stride;
-        row_g[tid] = (int)(row / p.T);
-    }
-    __syncthreads();
-
+    const int64_t row0 = (int64_t)blockIdx.x * ROWS;
+    const int nrows = (int)(p.R - row0 < ROWS ? p.R - row0 : ROWS);
+    small_rows(p, sr, row0, nrows);
     for (int i = tid; i < K * OC; i += blockDim.x) ws[i] = __ldg(p.Wt + i);
     if (PAD == 0 && TILE % 4 == 0 && p.x_stride % 4 == 0) {
         // the padded tile is the row itself: 16-byte copies, several in flight
@@ -59,7 +180,7 @@ __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
 #pragma unroll 4
         for (int i = tid; i < nrows * T4; i += blockDim.x) {
             const int rl = i / T4, e = i - rl * T4;
-            reinterpret_cast<float4 *>(xs)[i] = __ldg(reinterpret_cast<const float4 *>(src_row[rl]) + e);
+            reinterpret_cast<float4 *>(xs)[i] = __ldg(reinterpret_cast<const float4 *>(sr.src[rl]) + e);
         }
     } else {
 #pragma unroll 4
@@ -69,27 +190,14 @@ __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
             const int iy = py - PAD, ix = px - PAD;
             float v = 0.f;
             if ((unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw)
-                v = __ldg(src_row[rl] + (iy * p.iw + ix) * IC + ci);
+                v = __ldg(sr.src[rl] + (iy * p.iw + ix) * IC + ci);
             xs[i] = v;
         }
     }
     __syncthreads();
-    if (p.ov.patch) {
-        // the mutant's channels of each input row, written over the staged tile
-        const int per_row = p.ov.kmax * p.ov.cells;
-        for (int i = tid; i < nrows * per_row; i += blockDim.x) {
-            const int rl = i / per_row, rem = i - rl * per_row, q = rem / p.ov.cells, c = rem - q * p.ov.cells;
-            const int g = row_g[rl];
-            if (q >= p.ov.n_neurons[g]) continue;
-            const int j = p.ov.ids[p.ov.neuron_off[g] + q];
-            const int py = c / p.iw, px = c - py * p.iw;
-            xs[rl * TILE + ((py + PAD) * WP + px + PAD) * IC + j] =
-                p.ov.patch[(row0 + rl) * p.ov.row_stride + q * p.ov.cells + c];
-        }
-        __syncthreads();
-    }
+    if (p.ov.patch) small_overlay<IC>(p, sr, row0, nrows, xs, TILE, WP * IC, PAD, PAD);
 
-    const int per_row = p.cells * NSPLIT;
+    const int per_row = CELLS * NSPLIT;
     const int rl = tid / per_row, cell = (tid % per_row) / NSPLIT, n0 = (tid % NSPLIT) * OCT;
     if (rl >= nrows) return;
     const int64_t row = row0 + rl;
@@ -153,34 +261,6 @@ __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
     }
 }
 
-namespace {
-
-template <int KH, int KW, int IC, int OC, int OCT, int WP, int HP, int PAD, bool POOL>
-int launch_small(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, float *y_out, int64_t y_stride,
-                 cudaStream_t s, const Overlay *ov)
-{
-    ConvSmallParams p{};
-    if (ov) p.ov = *ov;
-    p.x = x.p; p.x_stride = x.stride; p.x_per_input = x.per_input;
-    p.t0 = rm.t0; p.T = rm.T; p.R = rm.R;
-    p.ih = S.ih; p.iw = S.iw; p.oh = S.oh; p.ow = S.ow;
-    p.Wt = S.Wt; p.b = S.b; p.act1 = S.act1;
-    p.z = z_out; p.z_stride = z_stride;
-    p.y = y_out; p.y_stride = y_stride;
-    p.cells = POOL ? (S.oh / 2) * (S.ow / 2) : S.oh * S.ow / 4;
-    p.rows_per_block = std::min(32, 256 / (p.cells * (OC / OCT)));
-    const size_t smem = ((size_t)KH * KW * IC * OC + (size_t)p.rows_per_block * HP * WP * IC) * sizeof(float);
-    // per device, cheap: allow more than the default 48 KiB of dynamic shared memory
-    cudaFuncSetAttribute(k_conv_small<KH, KW, IC, OC, OCT, WP, HP, PAD, POOL>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int64_t blocks = (rm.R + p.rows_per_block - 1) / p.rows_per_block;
-    k_conv_small<KH, KW, IC, OC, OCT, WP, HP, PAD, POOL>
-        <<<(unsigned)blocks, p.rows_per_block * p.cells * (OC / OCT), smem, s>>>(p);
-    return 1;
-}
-
-}  // namespace
-
 // Which layers the shared-memory kernel takes: stride 1, no residual add or GAP, and
 // one of the compiled geometries.
 int conv_small_variant(const Stage &S)
@@ -195,11 +275,22 @@ int launch_conv_small(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
                       int64_t y_stride, cudaStream_t s, const Overlay *ov)
 {
     if (rm.R <= 0) return 0;
-    switch (S.variant) {
-    case 1: return launch_small<5, 5, 6, 16, 4, 14, 14, 0, true>(S, x, rm, z_out, z_stride, y_out, y_stride, s, ov);
-    case 2: return launch_small<5, 5, 1, 6, 6, 32, 32, 2, true>(S, x, rm, z_out, z_stride, y_out, y_stride, s, ov);
-    }
-    return 0;
+    ConvSmallParams p{};
+    if (ov) p.ov = *ov;
+    p.x = x.p; p.x_stride = x.stride; p.x_per_input = x.per_input;
+    p.t0 = rm.t0; p.T = rm.T; p.R = rm.R;
+    p.ih = S.ih; p.iw = S.iw; p.oh = S.oh; p.ow = S.ow;
+    p.Wt = S.Wt; p.b = S.b; p.act1 = S.act1;
+    p.z = z_out; p.z_stride = z_stride;
+    p.y = y_out; p.y_stride = y_stride;
+    auto go = [&](auto kern, int rows, int threads, int floats) {
+        const int smem = floats * (int)sizeof(float);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        kern<<<(unsigned)((rm.R + rows - 1) / rows), threads, smem, s>>>(p);
+    };
+    if (S.variant == 1) go(k_conv_small<5, 5, 6, 16, 4, 14, 14, 0, true, 2, 25>, 2, 200, 150 * 16 + 2 * 14 * 14 * 6);
+    else go(k_conv1_pairs, kC1Rows, kC1Threads, 25 * 8 + kC1Rows * kC1Tile);
+    return 1;
 }
 
 }  // namespace mure
