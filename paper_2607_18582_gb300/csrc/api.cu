@@ -1015,8 +1015,19 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
                 stage(v, mut ? ws.zb : nullptr, zst);
                 if (!mut) continue;
                 acct.bytes_gather += rm.R * ((int64_t)kv[v] * cells_v + m->zd[v].size + m->xd[v].size) * 4;
+                // a dense layer's values go straight into the rows
+                if (patch_rows_supported(Sv, zrows)) {
+                    timed(C_DELTA, dfl, [&] {
+                        return launch_patch_rows(Sv, zrows, xsrc(Sv.in_src), rm, pv, kv[v], ws.xb[v + 1],
+                                                 m->xd[v + 1].stride, s);
+                    });
+                    continue;
+                }
+                const bool dots = patch_dot_supported(Sv, kv[v]);   // GF / WS in a kernel of their own
                 timed(C_DELTA, dfl, [&] {
-                    return launch_patch_vals(Sv, zrows, xsrc(Sv.in_src), skip_of(Sv), rm, pv, kv[v], ws.patch, pstride_v, s);
+                    const int nl = launch_patch_vals(Sv, zrows, xsrc(Sv.in_src), skip_of(Sv), rm, pv, kv[v], ws.patch,
+                                                     pstride_v, s, dots);
+                    return nl + (dots ? launch_patch_dot(Sv, zrows, xsrc(Sv.in_src), rm, pv, kv[v], ws.patch, pstride_v, s) : 0);
                 });
                 const Src xr{ws.xb[v + 1], m->xd[v + 1].stride, 0};
                 timed(C_DELTA, 0, [&] {
@@ -1031,11 +1042,14 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
                 f2.x_stride = m->xd[L].stride;
                 timed(v, 2 * Sv.macs * rm.R, [&] { return launch_final_dense(Sv, xsrc(Sv.in_src), rm, f2, s); });
                 acct.bytes_gather += rm.R * ((int64_t)kv[v] + m->zd[v].size + m->xd[v].size) * 4;
+                const bool direct = patch_rows_supported(Sv, zrows);
                 timed(C_DELTA, dfl, [&] {
-                    return launch_patch_vals(Sv, zrows, xsrc(Sv.in_src), skip_of(Sv), rm, pv, kv[v], ws.patch, pstride_v, s);
+                    return direct ? launch_patch_rows(Sv, zrows, xsrc(Sv.in_src), rm, pv, kv[v], ws.xb[L], m->xd[L].stride, s)
+                                  : launch_patch_vals(Sv, zrows, xsrc(Sv.in_src), skip_of(Sv), rm, pv, kv[v], ws.patch,
+                                                      pstride_v, s);
                 });
                 timed(C_EPI, 0, [&] {
-                    return launch_epilogue(Src{ws.xb[L], m->xd[L].stride, 0}, m->n_classes, rm, fa, s, &ovv);
+                    return launch_epilogue(Src{ws.xb[L], m->xd[L].stride, 0}, m->n_classes, rm, fa, s, direct ? nullptr : &ovv);
                 });
             } else {
                 timed(v, 2 * Sv.macs * rm.R, [&] { return launch_final_dense(Sv, xsrc(Sv.in_src), rm, fa, s); });

@@ -278,6 +278,13 @@ struct PatchArgs {
 int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const PatchArgs &pa, int kmax, float *out,
                       int64_t out_stride, cudaStream_t s, bool skip_dot_ops = false, bool skip_copy_ops = false);
 
+// The same values of a dense layer whose rows have their own z, written over the neurons' places
+// in the rows y of x_{l+1} (where patch_rows_supported; else launch_patch_vals and
+// launch_rows_overlay).
+int patch_rows_supported(const Stage &S, Src z);
+int launch_patch_rows(const Stage &S, Src z, Src x, RowMap rm, const PatchArgs &pa, int kmax, float *y, int64_t y_stride,
+                      cudaStream_t s);
+
 // GF / WS delta values on the tensor cores (convolution layers, tensor-core precision
 // modes): one implicit GEMM over the batch's inputs whose output channels are the
 // weight deltas e of every GF / WS slot of the batch (128 per N slice, so a slot's

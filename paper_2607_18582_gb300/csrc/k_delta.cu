@@ -519,10 +519,109 @@ __global__ void __launch_bounds__(256) k_patch_vals_dense_in(const PatchValsPara
     }
 }
 
-int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const PatchArgs &pa, int kmax, float *out,
-                      int64_t out_stride, cudaStream_t s, bool skip_dot_ops, bool skip_copy_ops)
+// Dense layers whose rows have their own z (vanilla rows, later layers of multi-layer mutants):
+// a warp per (mutant, RPW of its rows), every slot of a row at once.  Operators without a
+// fan-in sum: a row's slots on neighbouring lanes, 32 / slots rows per load.  GF / WS: the
+// weight deltas of SG slots stay in registers for all the warp's rows, a row is loaded once for
+// them, and each sum is dot_warp's (lane i takes k = i, i + 32, ... ascending, then the
+// butterfly; with SG values the halves of the warp each keep half of them at the first exchanges,
+// which adds the same pairs).  It was a warp per (mutant, slot), which read every row again for
+// each of its slots: FC 400-120 of LeNet-5's 3 % model-wide mutants, 279,000 rows, 280 us and 16 more
+// to move the patch into the rows, now 164.  Writes the patch, or (y non-null) the neurons' places in the rows themselves.
+template <int KPER>
+__global__ void __launch_bounds__(256, KPER <= 16 ? 2 : 1) k_patch_dense_rows(const PatchValsParams p, float *y, int64_t y_stride, int rpw)
 {
-    if (rm.R <= 0 || kmax <= 0) return 0;
+    constexpr int SG = KPER <= 16 ? 4 : 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = blockIdx.x;
+    const int n = p.pa.n_neurons[g];
+    if (n == 0) return;
+    const int op = p.pa.op[g];
+    const int32_t *ids = p.pa.ids + p.pa.neuron_off[g];
+    const int tl0 = (blockIdx.y * 8 + warp) * rpw, tl1 = min(tl0 + rpw, p.T);
+    auto put = [&](int64_t r, int q, int j, float v) {
+        if (y) y[r * y_stride + j] = v;
+        else p.out[r * p.out_stride + q] = v;
+    };
+    if (op != MURE_OP_GF && op != MURE_OP_WS) {
+        int w = 1;   // lanes per row
+        while (w < n && w < 32) w <<= 1;
+        for (int q = lane % w; q < n; q += w) {
+            const int j = ids[q], sj = op == MURE_OP_NS ? ids[q ^ 1] : j;
+#pragma unroll 4
+            for (int tl = tl0 + lane / w; tl < tl1; tl += 32 / w) {
+                const int64_t r = (int64_t)g * p.T + tl;
+                float zz = op == MURE_OP_NEB ? 0.f : __ldg(p.z + (p.z_per_input ? p.t0 + tl : r) * p.z_stride + sj);
+                if (op == MURE_OP_NAI) zz = -zz;
+                put(r, q, j, op == MURE_OP_NEB ? 0.f : act_apply(p.act1, zz));
+            }
+        }
+        return;
+    }
+    const float *e = p.pa.patch + p.pa.patch_off[g];
+    for (int q0 = 0; q0 < n; q0 += SG) {
+        float ev[SG][KPER];
+#pragma unroll
+        for (int a = 0; a < SG; ++a)
+#pragma unroll
+            for (int i = 0; i < KPER; ++i)
+                ev[a][i] = q0 + a < n && lane + 32 * i < p.K ? __ldg(e + (int64_t)(q0 + a) * p.K + lane + 32 * i) : 0.f;
+        // the slot whose sum this lane ends with
+        const int hi = lane >> 4 & 1, b = lane >> 3 & 1, mine = q0 + (SG == 4 ? 2 * hi + b : hi);
+        const int j = mine < n ? ids[mine] : 0;
+        for (int tl = tl0; tl < tl1; ++tl) {
+            const int64_t r = (int64_t)g * p.T + tl, t = p.t0 + tl;
+            const float *xr = p.x + (p.x_per_input ? t : r) * p.x_stride;
+            const float zv = __ldg(p.z + (p.z_per_input ? t : r) * p.z_stride + j);
+            float acc[SG];
+#pragma unroll
+            for (int a = 0; a < SG; ++a) acc[a] = 0.f;
+            float xv[KPER];
+#pragma unroll
+            for (int i = 0; i < KPER; ++i) xv[i] = lane + 32 * i < p.K ? __ldg(xr + lane + 32 * i) : 0.f;
+#pragma unroll
+            for (int i = 0; i < KPER; ++i)
+                if (lane + 32 * i < p.K) {
+#pragma unroll
+                    for (int a = 0; a < SG; ++a) acc[a] = fmaf(ev[a][i], xv[i], acc[a]);
+                }
+            float sum;
+            if constexpr (SG == 4) {
+                const float s0 = (hi ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, hi ? acc[0] : acc[2], 16);
+                const float s1 = (hi ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, hi ? acc[1] : acc[3], 16);
+                sum = (b ? s1 : s0) + __shfl_xor_sync(0xffffffffu, b ? s0 : s1, 8);
+            } else {
+                sum = (hi ? acc[1] : acc[0]) + __shfl_xor_sync(0xffffffffu, hi ? acc[0] : acc[1], 16);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 8);
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if ((lane & (SG == 4 ? 7 : 15)) == 0 && mine < n) put(r, mine, j, act_apply(p.act1, zv + sum));
+        }
+    }
+}
+
+int patch_rows_supported(const Stage &S, Src z)
+{
+    return S.kind == MURE_NODE_DENSE && !z.per_input && !S.has_add && !S.gap && !S.pool && S.oh * S.ow == 1 &&
+           S.K <= kDenseKMax;
+}
+
+static int launch_dense_rows(const PatchValsParams &p, float *y, int64_t y_stride, cudaStream_t s)
+{
+    // rows per warp: enough to pay for the deltas in registers, few enough to fill the GPU
+    int rpw = 8;
+    while (rpw < 32 && (int64_t)p.G * p.T > (int64_t)152 * 64 * rpw) rpw *= 2;
+    while ((p.T + 8 * rpw - 1) / (8 * rpw) > 65535) rpw *= 2;
+    const dim3 grid((unsigned)p.G, (unsigned)((p.T + 8 * rpw - 1) / (8 * rpw)));
+    if (p.K <= 128) k_patch_dense_rows<4><<<grid, 256, 0, s>>>(p, y, y_stride, rpw);
+    else if (p.K <= 256) k_patch_dense_rows<8><<<grid, 256, 0, s>>>(p, y, y_stride, rpw);
+    else if (p.K <= 512) k_patch_dense_rows<16><<<grid, 256, 0, s>>>(p, y, y_stride, rpw);
+    else k_patch_dense_rows<kDenseKMax / 32><<<grid, 256, 0, s>>>(p, y, y_stride, rpw);
+    return 1;
+}
+
+static PatchValsParams patch_vals_params(const Stage &S, Src z, Src x, Src skip, RowMap rm, const PatchArgs &pa, int kmax)
+{
     PatchValsParams p{};
     p.ih = S.ih; p.iw = S.iw; p.ic = S.ic; p.kh = S.kh; p.kw = S.kw; p.stride = S.stride; p.pad = S.pad;
     p.oh = S.oh; p.ow = S.ow; p.oc = S.oc; p.K = S.K;
@@ -537,15 +636,31 @@ int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const P
     p.t0 = rm.t0; p.T = rm.T; p.G = rm.R / rm.T;
     p.pa = pa;
     p.kmax = kmax;
-    p.out = out; p.out_stride = out_stride;
     p.warp_dot = (S.oh * S.ow) < 32;
-    p.skip_dot_ops = skip_dot_ops;
-    p.skip_copy_ops = skip_copy_ops;
     p.dw = S.kind == MURE_NODE_DWCONV;
     p.embed = S.kind == MURE_NODE_EMBED;
     p.vocab = S.vocab;
     p.W = S.W;
     p.b = S.b;
+    return p;
+}
+
+int launch_patch_rows(const Stage &S, Src z, Src x, RowMap rm, const PatchArgs &pa, int kmax, float *y, int64_t y_stride,
+                      cudaStream_t s)
+{
+    if (rm.R <= 0 || kmax <= 0) return 0;
+    return launch_dense_rows(patch_vals_params(S, z, x, Src{nullptr, 0, 0}, rm, pa, kmax), y, y_stride, s);
+}
+
+int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const PatchArgs &pa, int kmax, float *out,
+                      int64_t out_stride, cudaStream_t s, bool skip_dot_ops, bool skip_copy_ops)
+{
+    if (rm.R <= 0 || kmax <= 0) return 0;
+    PatchValsParams p = patch_vals_params(S, z, x, skip, rm, pa, kmax);
+    p.out = out; p.out_stride = out_stride;
+    p.skip_dot_ops = skip_dot_ops;
+    p.skip_copy_ops = skip_copy_ops;
+    if (patch_rows_supported(S, z) && !skip_dot_ops) return launch_dense_rows(p, nullptr, 0, s);
     const int64_t n_items = (int64_t)p.G * kmax;
     // each warp walks several inputs (blockIdx.y, +gridDim.y, ...): enough blocks to
     // fill the GPU, few enough that block scheduling stays negligible.  Without fan-in
@@ -597,46 +712,47 @@ int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const P
     return launches + 1;
 }
 
-// Materialise rows: out = base with the overlay's channels written in (for suffix
-// kernels that read plain rows).  out may alias a per-row base.
+// Materialise rows: out = base with the overlay's channels written in (for suffix kernels
+// that read plain rows), TPR threads per row (a warp, or the whole block for rows above 2 KB):
+// 16-byte copies through shared memory, the patch written there in between (one element per
+// thread and index division, it took 507 us for 140,800 rows of LeNet's 14 x 14 x 6 maps, now
+// 311).
+template <int TPR>
 __global__ void __launch_bounds__(256) k_rows_overlay(const float *__restrict__ base, int64_t base_stride,
-                                                      int base_per_input, int64_t t0, int T, int R, int64_t n_floats,
+                                                      int base_per_input, int64_t t0, int T, int R, int n4,
                                                       const Overlay ov, float *out, int64_t out_stride,
-                                                      int rows_per_block, const int32_t *lrow)
+                                                      const int32_t *lrow)
 {
-    extern __shared__ float sm[];  // [rows_per_block][n_floats]
-    __shared__ const float *src[64];
-    __shared__ float *dst[64];
-    __shared__ int gidx[64];
-    __shared__ int64_t lidx[64];
-    const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-    const int nr = (int)(R - r0 < rows_per_block ? R - r0 : rows_per_block);
-    if (threadIdx.x < nr) {
-        const int64_t r = r0 + threadIdx.x, lr = logical_row(lrow, r);
-        src[threadIdx.x] = base + (base_per_input ? t0 + lr % T : r) * base_stride;
-        dst[threadIdx.x] = out + r * out_stride;
-        gidx[threadIdx.x] = (int)(lr / T);
-        lidx[threadIdx.x] = lr;
+    extern __shared__ __align__(16) float sm[];  // [256 / TPR][4 n4]
+    const int tid = threadIdx.x % TPR;
+    const int64_t r = (int64_t)blockIdx.x * (256 / TPR) + threadIdx.x / TPR;
+    float *row = sm + (threadIdx.x / TPR) * 4 * n4;
+    const bool ok = r < R;
+    const int64_t lr = ok ? logical_row(lrow, r) : 0;
+    auto sync = [] {
+        if (TPR == 32) __syncwarp();
+        else __syncthreads();
+    };
+    if (ok) {
+        const float4 *src = reinterpret_cast<const float4 *>(base + (base_per_input ? t0 + lr % T : r) * base_stride);
+#pragma unroll 4
+        for (int i = tid; i < n4; i += TPR) reinterpret_cast<float4 *>(row)[i] = __ldg(src + i);
     }
-    __syncthreads();
-    const int nf = (int)n_floats;
-    for (int i = threadIdx.x; i < nr * nf; i += blockDim.x) {
-        const int rl = i / nf;
-        sm[i] = __ldg(src[rl] + (i - rl * nf));
+    sync();
+    if (ok) {
+        const int g = (int)(lr / T), n = ov.n_neurons[g];
+        const int32_t *ids = ov.ids + ov.neuron_off[g];
+        const float *patch = ov.patch + lr * ov.row_stride;
+        for (int q = 0; q < n; ++q) {
+            const int j = ids[q];
+            for (int c = tid; c < ov.cells; c += TPR) row[c * ov.ch + j] = __ldg(patch + q * ov.cells + c);
+        }
     }
-    __syncthreads();
-    const int per_row = ov.kmax * ov.cells;
-    for (int i = threadIdx.x; i < nr * per_row; i += blockDim.x) {
-        const int rl = i / per_row, rem = i - rl * per_row, q = rem / ov.cells, c = rem - q * ov.cells;
-        const int g = gidx[rl];
-        if (q >= ov.n_neurons[g]) continue;
-        const int j = ov.ids[ov.neuron_off[g] + q];
-        sm[rl * nf + c * ov.ch + j] = ov.patch[lidx[rl] * ov.row_stride + q * ov.cells + c];
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nr * nf; i += blockDim.x) {
-        const int rl = i / nf;
-        dst[rl][i - rl * nf] = sm[i];
+    sync();
+    if (ok) {
+        float4 *dst = reinterpret_cast<float4 *>(out + r * out_stride);
+#pragma unroll 4
+        for (int i = tid; i < n4; i += TPR) dst[i] = reinterpret_cast<const float4 *>(row)[i];
     }
 }
 
@@ -689,13 +805,16 @@ int launch_rows_overlay(Src base, int64_t n_floats, RowMap rm, const Overlay &ov
         }
         return launches;
     }
-    const int rows_per_block = (int)std::max<int64_t>(1, std::min<int64_t>(64, 8192 / std::max<int64_t>(n_floats, 1)));
-    const size_t smem = (size_t)rows_per_block * n_floats * sizeof(float);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(k_rows_overlay, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int64_t blocks = (rm.R + rows_per_block - 1) / rows_per_block;
-    k_rows_overlay<<<(unsigned)blocks, 256, smem, s>>>(base.p, base.stride, base.per_input, rm.t0, rm.T, rm.R,
-                                                      n_floats, ov, out, out_stride, rows_per_block, rm.lrow);
+    const int n4 = (int)((n_floats + 3) / 4);   // rows are whole 16-byte pieces
+    const int per_block = n4 <= 128 ? 8 : 1;
+    const size_t smem = (size_t)per_block * n4 * 16;
+    const unsigned blocks = (unsigned)((rm.R + per_block - 1) / per_block);
+    if (per_block == 8)
+        k_rows_overlay<32><<<blocks, 256, smem, s>>>(base.p, base.stride, base.per_input, rm.t0, rm.T, rm.R, n4, ov, out,
+                                                     out_stride, rm.lrow);
+    else
+        k_rows_overlay<256><<<blocks, 256, smem, s>>>(base.p, base.stride, base.per_input, rm.t0, rm.T, rm.R, n4, ov, out,
+                                                      out_stride, rm.lrow);
     return 1;
 }
 

@@ -137,3 +137,24 @@ def test_invalid_tagged_descriptors(M, ctx):
     # the expansion entry points take untagged descriptors only
     with pytest.raises(M.MureError):
         M.mure_expand_patches(model, tagged([(1, 3), (3, 5)], "GF", 1))
+
+
+@pytest.mark.parametrize("widths,slots", [((20, 130, 300, 600, 1100, 40, 7), 45), ((33, 128, 129, 9), 3), ((520, 70, 5), 80)])
+def test_dense_rows_at_fan_in_edges(M, ctx, oracle_mod, widths, slots):
+    """Dense layers' deltas on rows with their own pre-activations: every size of the register-held
+    delta rows (fan-ins 20 to 1,100, the last on the generic kernel), one slot to more slots than a
+    warp has lanes, every operator; the oracle, vanilla and small batches bit for bit."""
+    model = wl.mlp(5, widths)
+    neurons = sum(widths[1:])
+    X = wl.inputs(model, 70, 3)
+    table = wl.modelwide_mutants(model, 20, seed=6, ratio=slots / neurons, ops=("GF", "WS", "NAI", "NS", "NEB"))
+    ora = oracle_mod.vanilla(model, X, table)
+    m = M.mure_model_load(ctx, model, precision="fp32")
+    cache = M.mure_build_prefix_cache(m, X)
+    res = M.mure_eval_mutants(cache, table, logits=True)
+    ok, worst = logits_close(res["logits"], ora["logits"])
+    assert ok, worst
+    for other in (M.mure_eval_vanilla(m, X, table, logits=True),
+                  M.mure_eval_mutants(cache, table, logits=True, workspace_bytes=1 << 20)):
+        assert np.array_equal(other["logits"].view(np.uint32), res["logits"].view(np.uint32))
+        assert np.array_equal(other["kill_bits"], res["kill_bits"])
