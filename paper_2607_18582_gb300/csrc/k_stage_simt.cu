@@ -8,6 +8,8 @@
 // contribute x = 0), then z = acc + b[n].  Nothing depends on the batch size, the
 // tile a row lands in or the number of mutants, so one row gives the same bits in
 // the cache build, in a vanilla prefix and in a memoized suffix.
+#include <algorithm>
+
 #include "common.cuh"
 #include "device_util.cuh"
 #include "epilogue.cuh"
@@ -38,7 +40,10 @@ struct StageParams {
 // channels per block, TM x TN sums per thread (simt_tile.cuh), operand tiles
 // double-buffered in shared memory, the next pieces in flight while the current are used.  A4: the
 // input channels come in fours on 16-byte rows, so a thread fetches four k of its row at once.
-// OV (with A4 only): a fetched piece takes the mutated channels from the patch.
+// OV (with A4 only): a fetched piece takes the mutated channels from the patch.  Measured on
+// LeNet-5 in fp32 (1,500 x 150, FC 400-120 and 120-84): 0.88 ms with 4 x 4 sums per thread and
+// rows materialised first, 0.69 now; what bounds it is the latency of a tile's loads (few tiles
+// per SM at these sizes) and 84 or 120 outputs in 128 columns.
 template <int BM, int BN, int TM, int TN, bool A4, bool OV>
 __global__ void __launch_bounds__(BM / TM * (BN / TN), A4 && !OV && BN != 64 ? 4 : 3) k_stage_simt(const StageParams p)
 {
@@ -709,45 +714,20 @@ __global__ void __launch_bounds__(128) k_final_dense_w(const FinalParams p)
 // The weights come from the input-major copy Wt [F][C] with 16-byte loads all in flight;
 // each warp copies the rows' next 32 inputs (16-byte loads) into its own tile of 36-float
 // lines (16-byte stores and loads without bank conflicts) while it runs the FMAs of the
-// current 32; the warps' sums meet in shared memory and warp 0 runs the epilogue.  Needs
-// F a multiple of 4 and 16-byte aligned rows; dynamic shared memory [F][4][4] (class c at
+// current 32; the warps' sums meet in shared memory and one warp runs the epilogue.  A block
+// stays and takes many tiles of 32 rows, its weights placed once (a block per tile: 100 us for
+// 279,000 rows of 84 inputs, now 76).  Needs F a multiple of 4 and 16-byte aligned rows;
+// dynamic shared memory [F][4][4] (class c at
 // [f][c mod 4][c / 4]).
 constexpr int kSplitLine = 36;
 
-__global__ void __launch_bounds__(128) k_final_dense_split(const FinalParams p)
+__global__ void __launch_bounds__(128, 4) k_final_dense_split(const FinalParams p, int tiles)
 {
     extern __shared__ __align__(16) float wsm[];   // [F][4][4]
     __shared__ __align__(16) float xs[4][32][kSplitLine];
-    __shared__ float sums[32][13];
+    __shared__ float sums[2][32][13];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < p.F * 16; i += 128) wsm[i] = 0.f;
-    const int64_t row0 = (int64_t)blockIdx.x * 32;
-    const int64_t row = row0 + lane;
-    const bool in_range = row < p.R;
-    int ov_k = 0;
-    const int32_t *ov_ids = nullptr;
-    const int64_t lrow = in_range ? logical_row(p.lrow, row) : row;
-    if (p.ov.patch && in_range) {
-        const int g = (int)(lrow / p.T);
-        ov_k = p.ov.n_neurons[g];
-        ov_ids = p.ov.ids + p.ov.neuron_off[g];
-    }
-    // this lane copies 16 bytes (inputs 4 (lane mod 8) .. +3) of rows 4i + lane / 8
-    const int fq = 4 * (lane & 7);
-    const float *src[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int64_t r = row0 + 4 * i + (lane >> 3);
-        src[i] = r < p.R ? p.x + (p.x_per_input ? (p.t0 + logical_row(p.lrow, r) % p.T) : r) * p.x_stride : nullptr;
-    }
-    auto load = [&](int f0, float4 (&v)[8]) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            v[i] = (src[i] && f0 + fq < p.F) ? __ldg(reinterpret_cast<const float4 *>(src[i] + f0 + fq))
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-    };
-    float4 cur[8];
-    load(0, cur);
     __syncthreads();   // padding zeroed before the weights are placed
     {
         const int n4 = p.F * p.C / 4;
@@ -774,76 +754,108 @@ __global__ void __launch_bounds__(128) k_final_dense_split(const FinalParams p)
         }
     }
     __syncthreads();   // the weights
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f;
     const float *wq = wsm + 4 * warp;
     const float *xr = &xs[warp][lane][0];
-    for (int f0 = 0; f0 < p.F; f0 += 32) {
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 8; ++i) *reinterpret_cast<float4 *>(&xs[warp][4 * i + (lane >> 3)][fq]) = cur[i];
-        if (f0 + 32 < p.F) load(f0 + 32, cur);
-        __syncwarp();
-        const int fe = min(32, p.F - f0);
-        // overlay on this lane's own row (no other lane reads it)
-        for (int q = 0; q < ov_k; ++q) {
-            const int j = ov_ids[q];
-            const int cfirst = f0 - j <= 0 ? 0 : (f0 - j + p.ov.ch - 1) / p.ov.ch;
-            for (int c = cfirst; c < p.ov.cells && c * p.ov.ch + j < f0 + fe; ++c)
-                xs[warp][lane][c * p.ov.ch + j - f0] = p.ov.patch[lrow * p.ov.row_stride + q * p.ov.cells + c];
+    const int fq = 4 * (lane & 7);
+    int it = 0;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++it) {
+        const int buf = it & 1;
+        const int64_t row0 = (int64_t)tile * 32;
+        const int64_t row = row0 + lane;
+        const bool in_range = row < p.R;
+        int ov_k = 0;
+        const int32_t *ov_ids = nullptr;
+        const int64_t lrow = in_range ? logical_row(p.lrow, row) : row;
+        if (p.ov.patch && in_range) {
+            const int g = (int)(lrow / p.T);
+            ov_k = p.ov.n_neurons[g];
+            ov_ids = p.ov.ids + p.ov.neuron_off[g];
         }
-        if (fe == 32) {
+        // this lane copies 16 bytes (inputs 4 (lane mod 8) .. +3) of rows 4i + lane / 8
+        const float *src[8];
 #pragma unroll
-            for (int f4 = 0; f4 < 32; f4 += 4) {
-                const float4 x4 = *reinterpret_cast<const float4 *>(xr + f4);
-                const float xq[4] = {x4.x, x4.y, x4.z, x4.w};
+        for (int i = 0; i < 8; ++i) {
+            const int64_t r = row0 + 4 * i + (lane >> 3);
+            src[i] = r < p.R ? p.x + (p.x_per_input ? (p.t0 + logical_row(p.lrow, r) % p.T) : r) * p.x_stride : nullptr;
+        }
+        auto load = [&](int f0, float4 (&v)[8]) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float4 w4 = *reinterpret_cast<const float4 *>(wq + (f0 + f4 + e) * 16);
-                    a0 = fmaf(xq[e], w4.x, a0);
-                    a1 = fmaf(xq[e], w4.y, a1);
-                    a2 = fmaf(xq[e], w4.z, a2);
+            for (int i = 0; i < 8; ++i)
+                v[i] = (src[i] && f0 + fq < p.F) ? __ldg(reinterpret_cast<const float4 *>(src[i] + f0 + fq))
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        float4 cur[8];
+        load(0, cur);
+        float a0 = 0.f, a1 = 0.f, a2 = 0.f;
+        for (int f0 = 0; f0 < p.F; f0 += 32) {
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) *reinterpret_cast<float4 *>(&xs[warp][4 * i + (lane >> 3)][fq]) = cur[i];
+            if (f0 + 32 < p.F) load(f0 + 32, cur);
+            __syncwarp();
+            const int fe = min(32, p.F - f0);
+            // overlay on this lane's own row (no other lane reads it)
+            for (int q = 0; q < ov_k; ++q) {
+                const int j = ov_ids[q];
+                const int cfirst = f0 - j <= 0 ? 0 : (f0 - j + p.ov.ch - 1) / p.ov.ch;
+                for (int c = cfirst; c < p.ov.cells && c * p.ov.ch + j < f0 + fe; ++c)
+                    xs[warp][lane][c * p.ov.ch + j - f0] = p.ov.patch[lrow * p.ov.row_stride + q * p.ov.cells + c];
+            }
+            if (fe == 32) {
+#pragma unroll
+                for (int f4 = 0; f4 < 32; f4 += 4) {
+                    const float4 x4 = *reinterpret_cast<const float4 *>(xr + f4);
+                    const float xq[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float4 w4 = *reinterpret_cast<const float4 *>(wq + (f0 + f4 + e) * 16);
+                        a0 = fmaf(xq[e], w4.x, a0);
+                        a1 = fmaf(xq[e], w4.y, a1);
+                        a2 = fmaf(xq[e], w4.z, a2);
+                    }
+                }
+            } else {
+                for (int fl = 0; fl < fe; ++fl) {
+                    const float xv = xr[fl];
+                    const float4 w4 = *reinterpret_cast<const float4 *>(wq + (f0 + fl) * 16);
+                    a0 = fmaf(xv, w4.x, a0);
+                    a1 = fmaf(xv, w4.y, a1);
+                    a2 = fmaf(xv, w4.z, a2);
                 }
             }
-        } else {
-            for (int fl = 0; fl < fe; ++fl) {
-                const float xv = xr[fl];
-                const float4 w4 = *reinterpret_cast<const float4 *>(wq + (f0 + fl) * 16);
-                a0 = fmaf(xv, w4.x, a0);
-                a1 = fmaf(xv, w4.y, a1);
-                a2 = fmaf(xv, w4.z, a2);
+        }
+        sums[buf][lane][warp] = a0;
+        sums[buf][lane][warp + 4] = a1;
+        sums[buf][lane][warp + 8] = a2;
+        // one barrier per tile: the other warps go on to the next tile, whose sums go to the other
+        // buffer; they write this one again only after every warp has come to the next barrier.
+        // The warps take the epilogue in turn
+        __syncthreads();
+        if (warp != (it & 3)) continue;
+        float v[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const float z = c < p.C ? sums[buf][lane][c] + __ldg(p.b + c) : 0.f;
+            if (in_range && c < p.C && p.fa.z_out) p.fa.z_out[row * p.fa.z_stride + c] = z;
+            v[c] = act_apply(p.act, z);
+        }
+        if (p.fa.mode == 1) {  // cache build: logits rows and original predictions
+            if (in_range) {
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    if (c < p.C) p.fa.x_out[row * p.fa.x_stride + c] = v[c];
+                p.fa.pred_out[row] = argmax_reg<12>(v, p.C);
             }
+        } else if (p.fa.mode == 2) {  // per-row logits for a following delta + epilogue
+            if (in_range) {
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    if (c < p.C) p.fa.logits_rows[row * p.fa.x_stride + c] = v[c];
+            }
+        } else {
+            epilogue_reg<12>(p.fa, p.t0, p.T, row, in_range, v, p.C);
         }
     }
-    sums[lane][warp] = a0;
-    sums[lane][warp + 4] = a1;
-    sums[lane][warp + 8] = a2;
-    __syncthreads();
-    if (warp != 0) return;
-    float v[12];
-#pragma unroll
-    for (int c = 0; c < 12; ++c) {
-        const float z = c < p.C ? sums[lane][c] + __ldg(p.b + c) : 0.f;
-        if (in_range && c < p.C && p.fa.z_out) p.fa.z_out[row * p.fa.z_stride + c] = z;
-        v[c] = act_apply(p.act, z);
-    }
-    if (p.fa.mode == 1) {  // cache build: logits rows and original predictions
-        if (in_range) {
-#pragma unroll
-            for (int c = 0; c < 12; ++c)
-                if (c < p.C) p.fa.x_out[row * p.fa.x_stride + c] = v[c];
-            p.fa.pred_out[row] = argmax_reg<12>(v, p.C);
-        }
-        return;
-    }
-    if (p.fa.mode == 2) {  // per-row logits for a following delta + epilogue
-        if (in_range) {
-#pragma unroll
-            for (int c = 0; c < 12; ++c)
-                if (c < p.C) p.fa.logits_rows[row * p.fa.x_stride + c] = v[c];
-        }
-        return;
-    }
-    epilogue_reg<12>(p.fa, p.t0, p.T, row, in_range, v, p.C);
 }
 
 __global__ void __launch_bounds__(128) k_epilogue(const float *__restrict__ lg, int64_t stride, int per_input, int C,
@@ -983,7 +995,10 @@ int launch_final_dense(const Stage &S, Src x, RowMap rm, const FinalArgs &fa, cu
             // 9 to 12 classes: a block's 32 rows shared by four warps
             const size_t sbytes = (size_t)p.F * 16 * sizeof(float);
             cudaFuncSetAttribute(k_final_dense_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes);
-            k_final_dense_split<<<(unsigned)((rm.R + 31) / 32), 128, sbytes, s>>>(p);
+            // blocks that stay (four per SM) and take several tiles: the weights are placed once
+            // per block, not once per 32 rows
+            const int tiles = (rm.R + 31) / 32;
+            k_final_dense_split<<<(unsigned)std::min(tiles, 4 * 152), 128, sbytes, s>>>(p, tiles);
         }
         return 1;
     }
