@@ -84,24 +84,43 @@ void *dalloc(mure_ctx *c, size_t bytes)
     return p;
 }
 
-void dfree(mure_ctx *c, void *p)
+void dfree(mure_ctx *c, const void *cp)
 {
+    void *p = const_cast<void *>(cp);
     if (!p) return;
     if (c->has_alloc) c->alloc.free(p, (void *)c->stream, c->alloc.user);
     else cudaFreeAsync(p, c->stream);
 }
 
-// Device allocations owned by one call (freed on every exit path).
+// Device allocations owned by one call (freed on every exit path).  Small ones share blocks of
+// kBlock bytes: an allocation through a caller's allocator costs microseconds of host time, and
+// a small call asks for a dozen.
 struct Scratch {
+    static constexpr size_t kBlock = 1 << 20, kAlign = 512;
     mure_ctx *c;
     std::vector<void *> ptrs;
+    char *block = nullptr;
+    size_t left = 0;
     explicit Scratch(mure_ctx *ctx) : c(ctx) {}
     template <class T>
     T *get(size_t n)
     {
-        void *p = dalloc(c, n * sizeof(T));
-        ptrs.push_back(p);
+        const size_t bytes = (std::max<size_t>(n * sizeof(T), 16) + kAlign - 1) / kAlign * kAlign;
+        if (bytes > kBlock / 2) return static_cast<T *>(own(bytes));
+        if (bytes > left) {
+            block = static_cast<char *>(own(kBlock));
+            left = kBlock;
+        }
+        void *p = block;
+        block += bytes;
+        left -= bytes;
         return static_cast<T *>(p);
+    }
+    void *own(size_t bytes)
+    {
+        void *p = dalloc(c, bytes);
+        ptrs.push_back(p);
+        return p;
     }
     ~Scratch()
     {
@@ -110,6 +129,41 @@ struct Scratch {
 };
 
 int64_t round_up(int64_t n, int64_t a) { return (n + a - 1) / a * a; }
+
+// A call's results on their way to the host: small ones through the context's pinned memory,
+// queued without waiting and handed over by finish() after one synchronisation (a copy into
+// pageable memory waits for the stream by itself, each of them); larger ones, and those of a
+// call that finds another thread's call holding the memory, straight.
+struct Results {
+    static constexpr size_t kPinned = 1 << 20;
+    mure_ctx *c;
+    size_t used = 0;
+    struct Item {
+        void *dst;
+        size_t off, bytes;
+    };
+    std::vector<Item> items;
+    std::unique_lock<std::mutex> lock;
+    explicit Results(mure_ctx *ctx) : c(ctx), lock(ctx->pinned_mu, std::try_to_lock) {}
+    void add(void *dst, const void *dev, size_t bytes)
+    {
+        const size_t need = round_up(bytes, 16);
+        if (lock.owns_lock() && c->pinned && used + need <= kPinned) {
+            CK(c, cudaMemcpyAsync(c->pinned + used, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
+            items.push_back({dst, used, bytes});
+            used += need;
+        } else {
+            CK(c, cudaMemcpyAsync(dst, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
+        }
+    }
+    void finish()
+    {
+        CK(c, cudaStreamSynchronize(c->stream));
+        for (const Item &i : items) memcpy(i.dst, c->pinned + i.off, i.bytes);
+        items.clear();
+        used = 0;
+    }
+};
 
 template <class F>
 mure_status run(mure_ctx *c, F &&fn)
@@ -637,15 +691,11 @@ DevTable upload_table(mure_ctx *c, Scratch &sc, const mure_model *m, const mure_
     }
     dt.patch = plen ? sc.get<float>(plen) : nullptr;
     if (!jobs.empty()) {
-        std::vector<const float *> Wp(m->L);
-        for (int l = 0; l < m->L; ++l) Wp[l] = m->st[l].W;
-        const float **Wd = sc.get<const float *>(m->L);
-        CK(c, cudaMemcpyAsync(Wd, Wp.data(), m->L * sizeof(float *), cudaMemcpyHostToDevice, c->stream));
         ExpandArgs ea{};
         ea.jobs = (const SlotJob *)(dev + o_jobs);
         ea.n_jobs = dt.n_jobs;
         ea.sigma = m->sigma_dev;
-        ea.W = Wd;
+        ea.W = m->W_dev;
         ea.patch = dt.patch;
         ea.perm = perm_len ? sc.get<int32_t>(perm_len) : nullptr;
         ea.ws_as_weights = ws_as_weights;
@@ -1268,17 +1318,16 @@ void evaluate(mure_ctx *c, const mure_model *m, const mure_cache *ca, const mure
         check_launch(c);
         CK(c, cudaEventRecord(c->ev[3], s));
         unsigned long long host_cnt[4];
-        CK(c, cudaMemcpyAsync(host_cnt, ec.counters, sizeof host_cnt, cudaMemcpyDeviceToHost, s));
         int dev_err = 0;
-        CK(c, cudaMemcpyAsync(&dev_err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
+        Results res(c);
+        res.add(host_cnt, ec.counters, sizeof host_cnt);
+        res.add(&dev_err, c->err_dev, sizeof(int));
         if (!o->outputs_on_device) {
-            CK(c, cudaMemcpyAsync(out.kill_bits, ec.kill32, (size_t)n * words32 * 4, cudaMemcpyDeviceToHost, s));
-            if (o->logits_out)
-                CK(c, cudaMemcpyAsync(o->logits_out, lg_dev, (size_t)n * ca->n_in * m->n_classes * 4,
-                                      cudaMemcpyDeviceToHost, s));
+            res.add(out.kill_bits, ec.kill32, (size_t)n * words32 * 4);
+            if (o->logits_out) res.add(o->logits_out, lg_dev, (size_t)n * ca->n_in * m->n_classes * 4);
         }
         CK(c, cudaEventRecord(c->ev[4], s));
-        CK(c, cudaStreamSynchronize(s));
+        res.finish();
         CK(c, cudaGetLastError());
         if (dev_err) {
             CK(c, cudaMemset(c->err_dev, 0, sizeof(int)));
@@ -1330,15 +1379,13 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
     FAILIF(n_in < 0, c, MURE_ERR_INVALID_ARG, "n_inputs < 0");
     FAILIF(n_in > 0 && !X, c, MURE_ERR_INVALID_ARG, "NULL X");
     FAILIF(n_in > ((int64_t)1 << 30), c, MURE_ERR_UNSUPPORTED, "more than 2^30 inputs");
-    std::vector<int32_t> lab_host;
-    if (labels && n_in > 0) {
-        lab_host.resize(n_in);
-        if (on_dev) CK(c, cudaMemcpy(lab_host.data(), labels, n_in * 4, cudaMemcpyDeviceToHost));
-        else memcpy(lab_host.data(), labels, n_in * 4);
+    auto check_labels = [&](const int32_t *lab) {
         for (int64_t t = 0; t < n_in; ++t)
-            FAILIF(lab_host[t] < 0 || lab_host[t] >= m->n_classes, c, MURE_ERR_INVALID_ARG, "label %d of input %lld",
-                   lab_host[t], (long long)t);
-    }
+            FAILIF(lab[t] < 0 || lab[t] >= m->n_classes, c, MURE_ERR_INVALID_ARG, "label %d of input %lld", lab[t],
+                   (long long)t);
+    };
+    // labels on the device are counted there (k_label_set, below)
+    if (labels && !on_dev) check_labels(labels);
     cudaStream_t s = c->stream;
     auto *ca = new mure_cache();
     ca->model = m;
@@ -1357,22 +1404,41 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         }
     } cl{ca};
     const int64_t np = std::max<int64_t>(ca->n_pad, kInputAlign);
-    for (int s2 = 0; s2 <= L; ++s2) {
-        ca->x[s2] = (float *)dalloc(c, np * m->xd[s2].stride * 4);
-        CK(c, cudaMemsetAsync(ca->x[s2], 0, np * m->xd[s2].stride * 4, s));
+    {
+        // one block; every row of every tensor is written below but the padding inputs of x_0
+        // and the padding at the end of rows whose size is no multiple of 4: only those are zeroed
+        size_t off = 0;
+        auto place = [&](int64_t floats) {
+            const size_t o = off;
+            off += round_up(np * floats * 4, 512);
+            return o;
+        };
+        std::vector<size_t> ox(L + 1), oz(L);
+        for (int s2 = 0; s2 <= L; ++s2) ox[s2] = place(m->xd[s2].stride);
+        for (int v = 0; v < L; ++v) oz[v] = place(m->zd[v].stride);
+        const size_t op = place(1), ol = place(1);
+        ca->mem = (char *)dalloc(c, off);
+        auto tensor = [&](size_t o, const TensorDim &d) {
+            float *p = (float *)(ca->mem + o);
+            if (d.stride != d.size || n_in == 0) CK(c, cudaMemsetAsync(p, 0, np * d.stride * 4, s));
+            return p;
+        };
+        for (int s2 = 0; s2 <= L; ++s2) ca->x[s2] = tensor(ox[s2], m->xd[s2]);
+        for (int v = 0; v < L; ++v) ca->z[v] = tensor(oz[v], m->zd[v]);
+        if (np > n_in)
+            CK(c, cudaMemsetAsync(ca->x[0] + n_in * m->xd[0].stride, 0, (np - n_in) * m->xd[0].stride * 4, s));
+        ca->pred0 = (int32_t *)(ca->mem + op);
+        ca->label = (int32_t *)(ca->mem + ol);
+        CK(c, cudaMemsetAsync(ca->pred0, 0, np * 4, s));
+        CK(c, cudaMemsetAsync(ca->label, 0, np * 4, s));
     }
-    for (int v = 0; v < L; ++v) {
-        ca->z[v] = (float *)dalloc(c, np * m->zd[v].stride * 4);
-        CK(c, cudaMemsetAsync(ca->z[v], 0, np * m->zd[v].stride * 4, s));
-    }
-    ca->pred0 = (int32_t *)dalloc(c, np * 4);
-    ca->label = (int32_t *)dalloc(c, np * 4);
-    CK(c, cudaMemsetAsync(ca->pred0, 0, np * 4, s));
-    CK(c, cudaMemsetAsync(ca->label, 0, np * 4, s));
     if (n_in > 0) {
         const int64_t sz = m->xd[0].size, str = m->xd[0].stride;
-        CK(c, cudaMemcpy2DAsync(ca->x[0], str * 4, X, sz * 4, sz * 4, n_in,
-                                on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        if (sz == str)
+            CK(c, cudaMemcpyAsync(ca->x[0], X, n_in * sz * 4, on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        else
+            CK(c, cudaMemcpy2DAsync(ca->x[0], str * 4, X, sz * 4, sz * 4, n_in,
+                                    on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
         Scratch sc(c);
         int64_t g = 0;
         for (int v = 0; v < L; ++v) g = std::max(g, stage_scratch(m->st[v]));
@@ -1399,17 +1465,30 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         fa.pred_out = ca->pred0;
         c->launches += launch_final_dense(m->st[L - 1], Src{xs[L - 1], m->xd[L - 1].stride, 0}, rm, fa, s);
         check_launch(c);
-        if (labels) CK(c, cudaMemcpyAsync(ca->label, lab_host.data(), n_in * 4, cudaMemcpyHostToDevice, s));
-        else CK(c, cudaMemcpyAsync(ca->label, ca->pred0, n_in * 4, cudaMemcpyDeviceToDevice, s));
-        uint32_t *mask = sc.get<uint32_t>(kLabelWords);
-        CK(c, cudaMemsetAsync(mask, 0, 4 * kLabelWords, s));
-        c->launches += launch_label_set(ca->label, n_in, mask, s);
+        if (labels && on_dev && s && s != cudaStreamLegacy) {
+            // labels written on the default stream are waited for whatever the context's stream
+            CK(c, cudaEventRecord(c->ev[7], cudaStreamLegacy));
+            CK(c, cudaStreamWaitEvent(s, c->ev[7], 0));
+        }
+        CK(c, cudaMemcpyAsync(ca->label, labels ? labels : ca->pred0, n_in * 4,
+                              labels && !on_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
+        uint32_t *mask = sc.get<uint32_t>(kLabelWords + 1);
+        CK(c, cudaMemsetAsync(mask, 0, 4 * (kLabelWords + 1), s));
+        c->launches += launch_label_set(ca->label, n_in, m->n_classes, mask, s);
         check_launch(c);
-        uint32_t hm[kLabelWords] = {};
-        CK(c, cudaMemcpyAsync(hm, mask, 4 * kLabelWords, cudaMemcpyDeviceToHost, s));
+        uint32_t hm[kLabelWords + 1] = {};
         int dev_err = 0;
-        CK(c, cudaMemcpyAsync(&dev_err, c->err_dev, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CK(c, cudaStreamSynchronize(s));
+        Results res(c);
+        res.add(hm, mask, sizeof hm);
+        res.add(&dev_err, c->err_dev, sizeof(int));
+        res.finish();
+        if (hm[kLabelWords]) {
+            // the first bad label, as for labels on the host
+            std::vector<int32_t> lab(n_in);
+            CK(c, cudaMemcpy(lab.data(), ca->label, n_in * 4, cudaMemcpyDeviceToHost));
+            if (dev_err) CK(c, cudaMemset(c->err_dev, 0, sizeof(int)));
+            check_labels(lab.data());
+        }
         ca->n_label_values = 0;
         for (int k = 0; k < kLabelWords; ++k) ca->n_label_values += __builtin_popcount(hm[k]);
         if (dev_err) {
@@ -1424,7 +1503,7 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
                                                      : "wait limit");
         }
     }
-    CK(c, cudaStreamSynchronize(s));
+    if (n_in == 0) CK(c, cudaStreamSynchronize(s));
     cl.ok = true;
     return ca;
 }
@@ -1466,6 +1545,10 @@ mure_status mure_create(int device, void *cuda_stream, const mure_allocator *all
         for (auto &e : c->ev) CK(c, cudaEventCreate(&e));
         CK(c, cudaMalloc(&c->err_dev, sizeof(int)));
         CK(c, cudaMemset(c->err_dev, 0, sizeof(int)));
+        if (cudaMallocHost(&c->pinned, Results::kPinned) != cudaSuccess) {
+            cudaGetLastError();
+            c->pinned = nullptr;
+        }
     });
     if (st != MURE_OK) {
         mure_destroy(c);
@@ -1482,6 +1565,7 @@ void mure_destroy(mure_ctx *ctx)
         if (e) cudaEventDestroy(e);
     for (auto &e : ctx->evpool) cudaEventDestroy(e);
     if (ctx->err_dev) cudaFree(ctx->err_dev);
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
     delete ctx;
 }
 
@@ -1591,12 +1675,12 @@ mure_status mure_model_load(mure_ctx *c, const mure_model_desc *d, mure_model **
             std::vector<const float *> Wp(m->L);
             std::vector<int64_t> cnt(m->L);
             for (int l = 0; l < m->L; ++l) { Wp[l] = m->st[l].W; cnt[l] = (int64_t)m->st[l].oc * m->st[l].K; }
-            const float **Wd = sc.get<const float *>(m->L);
+            m->W_dev = (const float **)dalloc(c, m->L * sizeof(float *));
             int64_t *nd = sc.get<int64_t>(m->L);
             m->sigma_dev = (double *)dalloc(c, m->L * 8);
-            CK(c, cudaMemcpyAsync(Wd, Wp.data(), m->L * sizeof(float *), cudaMemcpyHostToDevice, c->stream));
+            CK(c, cudaMemcpyAsync(m->W_dev, Wp.data(), m->L * sizeof(float *), cudaMemcpyHostToDevice, c->stream));
             CK(c, cudaMemcpyAsync(nd, cnt.data(), m->L * 8, cudaMemcpyHostToDevice, c->stream));
-            c->launches += launch_layer_std(Wd, nd, m->L, m->sigma_dev, c->stream);
+            c->launches += launch_layer_std(m->W_dev, nd, m->L, m->sigma_dev, c->stream);
             check_launch(c);
             m->sigma_host.resize(m->L);
             CK(c, cudaMemcpyAsync(m->sigma_host.data(), m->sigma_dev, m->L * 8, cudaMemcpyDeviceToHost, c->stream));
@@ -1617,6 +1701,7 @@ void mure_model_free(mure_model *m)
         dfree(m->ctx, S.b);
         dfree(m->ctx, S.Wtc);
     }
+    dfree(m->ctx, m->W_dev);
     dfree(m->ctx, m->sigma_dev);
     cudaStreamSynchronize(m->ctx->stream);
     delete m;
@@ -1674,10 +1759,7 @@ void mure_cache_free(mure_cache *ca)
 {
     if (!ca) return;
     mure_ctx *c = ca->model->ctx;
-    for (float *p : ca->x) dfree(c, p);
-    for (float *p : ca->z) dfree(c, p);
-    dfree(c, ca->pred0);
-    dfree(c, ca->label);
+    dfree(c, ca->mem);
     cudaStreamSynchronize(c->stream);
     delete ca;
 }
@@ -1689,11 +1771,22 @@ mure_status mure_cache_outputs(mure_cache *ca, float *logits, int32_t *pred)
     return run(c, [&] {
         const mure_model *m = ca->model;
         if (ca->n_in == 0) return;
-        if (logits)
-            CK(c, cudaMemcpy2DAsync(logits, m->n_classes * 4, ca->x[m->L], m->xd[m->L].stride * 4, m->n_classes * 4,
-                                    ca->n_in, cudaMemcpyDeviceToHost, c->stream));
-        if (pred) CK(c, cudaMemcpyAsync(pred, ca->pred0, ca->n_in * 4, cudaMemcpyDeviceToHost, c->stream));
-        CK(c, cudaStreamSynchronize(c->stream));
+        Scratch sc(c);
+        Results res(c);
+        if (logits) {
+            // packed on the device: a strided copy to the host goes row by row
+            const int64_t str = m->xd[m->L].stride;
+            const float *src = ca->x[m->L];
+            if (str != m->n_classes) {
+                float *dense = sc.get<float>(ca->n_in * m->n_classes);
+                c->launches += launch_pack_rows(src, str, m->n_classes, ca->n_in, dense, c->stream);
+                check_launch(c);
+                src = dense;
+            }
+            res.add(logits, src, ca->n_in * m->n_classes * 4);
+        }
+        if (pred) res.add(pred, ca->pred0, ca->n_in * 4);
+        res.finish();
     });
 }
 

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -76,6 +77,10 @@ struct mure_ctx {
     int64_t launches = 0;             // kernels launched since creation
     int *err_dev = nullptr;           // device error word written by bounded waits
     int64_t wait_limit = 0;           // limit of the device-side waits in SM cycles (0 = default)
+    // pinned host memory for a call's small results (created with the context, freed with it):
+    // copies into it are queued without waiting, one synchronisation then covers all of them
+    char *pinned = nullptr;           // null: not available, results are copied straight
+    std::mutex pinned_mu;             // held from a call's first copy to its hand-over
 };
 
 struct mure_model {
@@ -86,6 +91,7 @@ struct mure_model {
     std::vector<mure::Stage> st;      // L stages
     std::vector<mure::TensorDim> xd;  // L + 1 stage inputs
     std::vector<mure::TensorDim> zd;  // L pre-activations
+    const float **W_dev = nullptr;    // device [L] the layers' weight pointers
     double *sigma_dev = nullptr;      // device [L] population std of each layer's W (fp64)
     std::vector<double> sigma_host;
 };
@@ -93,6 +99,7 @@ struct mure_model {
 struct mure_cache {
     mure_model *model = nullptr;
     int64_t n_in = 0, n_pad = 0;
+    char *mem = nullptr;              // one allocation for all of the below
     std::vector<float *> x;           // x[s], s = 0..L: [n_pad][xd[s].stride]
     std::vector<float *> z;           // z[v], v = 0..L-1: [n_pad][zd[v].stride]
     int32_t *pred0 = nullptr;         // [n_pad]
@@ -376,7 +383,11 @@ int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t
 int launch_scores(const uint32_t *kill32, int64_t n_mut, int64_t words32, const int32_t *label, int n_classes,
                   unsigned long long *totals /* [2]: killed, sum of label counts */, cudaStream_t s);
 
-// Distinct labels among n inputs (bitset of kLabelWords words; mask zeroed by the caller).
-int launch_label_set(const int32_t *label, int64_t n, uint32_t *mask, cudaStream_t s);
+// Distinct labels among n inputs: a bitset of kLabelWords words, then the number of labels
+// outside [0, n_classes) (all zeroed by the caller).
+int launch_label_set(const int32_t *label, int64_t n, int n_classes, uint32_t *mask, cudaStream_t s);
+
+// Rows of n floats without their padding: out [R][n].
+int launch_pack_rows(const float *in, int64_t in_stride, int n, int64_t R, float *out, cudaStream_t s);
 
 }  // namespace mure

@@ -139,7 +139,7 @@ def test_invalid_tagged_descriptors(M, ctx):
         M.mure_expand_patches(model, tagged([(1, 3), (3, 5)], "GF", 1))
 
 
-@pytest.mark.parametrize("widths,slots", [((20, 130, 300, 600, 1100, 40, 7), 45), ((33, 128, 129, 9), 3), ((520, 70, 5), 80)])
+@pytest.mark.parametrize("widths,slots", [((20, 130, 300, 600, 1100, 40, 7), 45), ((33, 128, 129, 9), 3), ((520, 70, 5), 50)])
 def test_dense_rows_at_fan_in_edges(M, ctx, oracle_mod, widths, slots):
     """Dense layers' deltas on rows with their own pre-activations: every size of the register-held
     delta rows (fan-ins 20 to 1,100, the last on the generic kernel), one slot to more slots than a

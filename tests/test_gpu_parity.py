@@ -433,3 +433,23 @@ def test_gather_mode_convolutions_match_oracle(M, ctx, oracle_runs, monkeypatch,
         assert bad == 0
         v = M.mure_eval_vanilla(model, w.X, table, logits=True)
         assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
+@pytest.mark.parametrize("on_device", [False, True])
+def test_bad_labels_are_refused(M, ctx, on_device):
+    """A label outside the classes: INVALID_ARG naming the first one, from host and device arrays
+    alike; the context stays usable and good labels reach the kill rule."""
+    import torch
+    w = wl.workload("mlp", 70, 8)
+    model = M.mure_model_load(ctx, w.model)
+    good = np.arange(70, dtype=np.int32) % 10
+    put = (lambda a: torch.from_numpy(a).cuda()) if on_device else (lambda a: a)
+    for bad_value in (10, -1, 97, -(2 ** 31)):
+        bad = good.copy()
+        bad[[41, 60]] = bad_value
+        with pytest.raises(M.MureError, match=f"label {bad_value} of input 41") as ei:
+            M.mure_build_prefix_cache(model, put(w.X), put(bad))
+        assert ei.value.status == 1
+    a = M.mure_eval_mutants(M.mure_build_prefix_cache(model, put(w.X), put(good)), w.table)
+    b = M.mure_eval_mutants(M.mure_build_prefix_cache(model, w.X, good), w.table)
+    assert np.array_equal(a["kill_bits"], b["kill_bits"]) and a["scoreB"] == b["scoreB"]
