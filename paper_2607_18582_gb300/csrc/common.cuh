@@ -44,6 +44,8 @@ struct Stage {
     int tc_wide = 0;          // tc_conv: all 256 outputs in one CTA (one N = 256 MMA per K8 step)
     int tc_win = 0;           // tc_conv: a GEMM row per 2x2 output window (16-channel 3x3 layers:
                               // N = 4 positions x 16 outputs over a 4x4 field of 16 channels)
+    int c11 = 0;              // the 1 x 1 kernel of few channels (tc is then 0; the tc_ fields
+                              // still say how its delta's GEMM runs)
     float *Wtc = nullptr;     // tc: TF32 halves of W in the tensor-core operand layout
     int *err = nullptr;       // device error word of the context (bounded waits)
     const int64_t *wait_limit = nullptr;   // host: the context's wait limit (0 = default)
@@ -163,7 +165,12 @@ struct Overlay {
 // scratch (the map before global average pooling; an LSTM's input sums).
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip,
                       float *y_out, int64_t y_stride, float *tmp, cudaStream_t s, const Overlay *ov = nullptr);
-// Whether the CUDA-core stage kernel applies the overlay as it fetches rows of x.
+// 1 x 1 convolutions of few channels in fp32: which layers, and the launcher (the map before
+// global average pooling goes to y).
+int conv1x1_geometry(const Stage &S);
+int launch_conv1x1(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out, int64_t y_stride,
+                   cudaStream_t s, const Overlay *ov);
+// Whether the CUDA-core stage kernels apply the overlay as they fetch rows of x.
 int simt_overlay_inline(const Stage &S, const Overlay &ov, Src x);
 
 // The shared-memory direct convolution for small inputs (variant of a stage, 0 when

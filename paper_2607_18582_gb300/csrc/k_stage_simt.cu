@@ -446,6 +446,8 @@ int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     if (ov) p.ov = *ov;
     const bool a4 = S.ic % 4 == 0 && aligned16(x.p, x.stride);
     int launches = 1;
+    if (S.c11 && a4 && p.vec) launch_conv1x1(S, x, rm, z_out, z_stride, skip, p.y, p.y_stride, s, ov);
+    else
     // the narrowest tile that holds the outputs: padded columns cost as much as real ones
     if (S.oc <= 16) stage_tiles<128, 16, 4, 4>(p, a4, s);
     else if (S.oc <= 32) stage_tiles<128, 32, 8, 4>(p, a4, s);
