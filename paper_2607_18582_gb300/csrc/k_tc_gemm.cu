@@ -15,10 +15,10 @@
 //              splits them into TF32 halves and stores the halves into a tensor-memory
 //              A stage (tcgen05.st); the MMA reads A from tensor memory, so the
 //              operand never goes through shared memory a second time;
-//   warps 8-10 MMA issue (kind::tf32, M=128, K=8): one thread issues an MMA only about
-//              every 120 cycles, whatever N is, so where tensor memory allows, a
+//   warps 8-10 MMA issue (kind::tf32, M=128, K=8): where tensor memory allows, a
 //              K-step's MMAs are dealt to up to three warps, each accumulating into its
-//              own partial accumulator; the epilogue adds the partials in a fixed order;
+//              own partial accumulator (the epilogue adds the partials in a fixed order), or
+//              two take turns on one accumulator;
 //   warp 11    one thread moves the weights: pre-split, pre-swizzled K-step chunks
 //              (one bulk copy each), or the whole slice once when it fits;
 //   warps 4-7  epilogue: two accumulator sets alternate, so the bias / activation /
@@ -30,6 +30,7 @@
 // role, lets its own copies and MMAs drain (bounded), frees its tensor memory and
 // returns.
 #include <algorithm>
+#include <type_traits>
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -169,6 +170,21 @@ __device__ __forceinline__ void wait_phase_drain(uint32_t a, uint32_t parity)
     const long long t0 = clock64();
     while (!mbar_try(a, parity))
         if (clock64() - t0 > kSpin) return;
+}
+
+// One lane of a converged warp (the same one every time).  The tensor-core and bulk-copy
+// instructions take their operands from uniform registers; in a branch on the lane number the
+// compiler cannot know that a single lane runs it.  So the issuing warps run their loops whole,
+// with warp-uniform operands, and elect a lane around the instructions themselves, and the copying
+// warps elect the lane that copies.  Measured (lane-number branches before): the window GEMM of
+// LeNet's second convolution 8.93 -> 8.32 ms (1,000 mutants x 10,000 inputs), VGG's staged
+// convolutions 122.3 -> 117.8 ms (250 x 1,000), ResNet-20's 19.2 -> 18.5 ms (60 x 600); dense
+// layers unchanged.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+    return ok != 0;
 }
 
 // A from tensor memory, B from shared memory.
@@ -1341,7 +1357,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
         }
     } else if (DENSE && warp == 10 && p.a_tma) {
         // ------------------------------------------------------ A tiles by TMA --
-        if (lane == 0) {
+        if (elect_one()) {
             const uint64_t tmap = reinterpret_cast<uint64_t>(&p.tmap_a);
             int slot_i = 0, kt = 0;
             uint32_t slot_wraps = 0;
@@ -1497,7 +1513,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
                     return false;
                 }
             }
-            if (lane == 0) issue(issued);
+            if (elect_one()) issue(issued);
             __syncwarp();
             ++issued;
             return true;
@@ -1553,27 +1569,28 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
     } else if (warp < 11) {
         // ------------------------------------------------------------------ MMA --
         // The K-steps of a tile are dealt to the n_mma issuing warps by their index
-        // (kt mod n_mma = w), each warp into its own partial accumulator.  One thread
-        // issues an MMA only about every 60 cycles and then waits for its next stage,
-        // so while one warp waits the others keep the tensor pipe busy.  The split
-        // depends on kt alone: a row's partial sums never depend on its place in the
+        // (kt mod n_mma = w), each warp into its own partial accumulator: a split that
+        // depends on kt alone, so a row's partial sums never depend on its place in the
         // batch.  With mma_chain the warps share one accumulator and take the K-steps
         // in turn: a warp issues K-step g only once the warp before it has issued g - 1
         // (an arrival on the turn barrier), so the MMAs reach the tensor pipe in K-step
         // order, as from one warp, while each warp's barrier waits and commits overlap
         // the other's issue.  (A barrier is never two phases ahead of its waiter: the
-        // other warp's next turn waits for this warp's arrival.)
+        // other warp's next turn waits for this warp's arrival.)  The turns stay on one
+        // lane's slower issue: electing there let a turn's first MMA pass the one before
+        // (sums in another order), and one elected warp instead of two in turn is 4 %
+        // (staged convolutions) to 20 % (dense) slower.
         const int w = warp - 8;
         if (pair) {
             // tile pairs: warp w issues tile w of each unit into its own accumulator, both
             // warps side by side from the same A and weight stages (each stage is released
             // by the commits of both)
-            if (lane == 0 && w < 2) {
+            if (w < 2) {
                 constexpr int Q = THREE ? 12 : 4;
                 const uint32_t id = idesc_tf32(kTileM, Nt), id2 = idesc_tf32(kTileM, 2 * Nt);
                 const bool merged = THREE && p.merge_lo;
                 bool ok = true;
-                if (p.b_resident) ok = wait_phase<32>(smem_u32(&bar_bfull[0]), 0, abort_flag);
+                if (p.b_resident) ok = warp_wait_phase<32>(smem_u32(&bar_bfull[0]), 0, abort_flag);
                 const uint64_t desc_b0 = sw128_desc(b_region);
                 const uint32_t b_step16 = b_step >> 4, lo16 = (uint32_t)Nt * 128 >> 4;
                 int t = 0, sb = 0;
@@ -1581,97 +1598,127 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
                 for (int64_t i = 0; ok && i < my_tiles; ++i) {
                     const int a = p.n_acc == 2 ? (int)(i & 1) : 0;
                     const int64_t use = p.n_acc == 2 ? (i >> 1) : i;
-                    if (use >= 1 && !wait_phase<32>(smem_u32(&bar_accempty[a]), (uint32_t)((use - 1) & 1), abort_flag)) break;
+                    if (use >= 1 && !warp_wait_phase<32>(smem_u32(&bar_accempty[a]), (uint32_t)((use - 1) & 1), abort_flag)) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint32_t d = tmem + (uint32_t)((a * 2 + w) * p.acc_cols);
                     for (int kt = 0; kt < nK; ++kt) {
-                        if (!wait_phase<32>(smem_u32(&bar_afull[t]), t_wraps & 1, abort_flag)) { ok = false; break; }
+                        if (!warp_wait_phase<32>(smem_u32(&bar_afull[t]), t_wraps & 1, abort_flag)) { ok = false; break; }
                         if (!p.b_resident &&
-                            !wait_phase<32>(smem_u32(&bar_bfull[sb]), b_wraps & 1, abort_flag)) { ok = false; break; }
+                            !warp_wait_phase<32>(smem_u32(&bar_bfull[sb]), b_wraps & 1, abort_flag)) { ok = false; break; }
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint64_t dh = desc_b0 + (uint64_t)((p.b_resident ? kt : sb) * b_step16), dl = dh + lo16;
                         const uint32_t ta = tmem + p.a_col + (uint32_t)(t * 2 + w) * kAColsPerStage;
                         const uint32_t acc0 = kt > 0 ? 1u : 0u;   // K-step 0 of the tile overwrites
-                        if (merged) mma_block_merged(d, ta, dh, id2, id, acc0);
-                        else mma_block<THREE, 0, Q>(d, ta, dh, dl, id, acc0);
-                        mma_commit(smem_u32(&bar_aempty[t]));
-                        if (!p.b_resident) mma_commit(smem_u32(&bar_bempty[sb]));
+                        if (elect_one()) {
+                            if (merged) mma_block_merged(d, ta, dh, id2, id, acc0);
+                            else mma_block<THREE, 0, Q>(d, ta, dh, dl, id, acc0);
+                            mma_commit(smem_u32(&bar_aempty[t]));
+                            if (!p.b_resident) mma_commit(smem_u32(&bar_bempty[sb]));
+                        }
+                        __syncwarp();
                         if (++t == p.n_stages) { t = 0; ++t_wraps; }
                         if (!p.b_resident && ++sb == p.nb) { sb = 0; ++b_wraps; }
                     }
                     if (!ok) break;
-                    mma_commit(smem_u32(&bar_accfull[a]));
+                    if (elect_one()) mma_commit(smem_u32(&bar_accfull[a]));
+                    __syncwarp();
                 }
                 // every MMA of both issuing warps has finished before the teardown
-                mma_commit(smem_u32(&bar_drain));
+                if (elect_one()) mma_commit(smem_u32(&bar_drain));
+                __syncwarp();
                 wait_phase_drain(smem_u32(&bar_drain), 0);
             }
-        } else if (lane == 0 && w < p.n_mma) {
+        } else if (w < p.n_mma) {
             const int nmma = p.n_mma, nacc = p.n_acc;
             constexpr int Q = THREE ? 12 : 4;
             const uint32_t id = idesc_tf32(kTileM, Nt), id2 = idesc_tf32(kTileM, 2 * Nt);
             // (the window GEMM never takes these paths: compiled out of its latency-bound
             // issuing loop)
             const bool merged = MODE == 3 && THREE && p.merge_lo;
-            bool ok = true;
-            if (p.b_resident) ok = wait_phase<32>(smem_u32(&bar_bfull[0]), 0, abort_flag);
-            const uint64_t desc_b0 = sw128_desc(b_region);
-            const uint32_t b_step16 = b_step >> 4, lo16 = (uint32_t)Nt * 128 >> 4;
-            int t = 0, sb = 0;                  // ring slots of K-step kt (every warp tracks every step)
-            uint32_t t_wraps = 0, b_wraps = 0;
-            for (int64_t i = 0; ok && i < my_tiles; ++i) {
-                const int a = nacc == 2 ? (int)(i & 1) : 0;
-                const int64_t use = nacc == 2 ? (i >> 1) : i;
-                if (use >= 1 && !wait_phase<32>(smem_u32(&bar_accempty[a]), (uint32_t)((use - 1) & 1), abort_flag)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const bool chain = MODE != 2 && p.mma_chain != 0;
-                const uint32_t d = tmem + (uint32_t)((a * p.n_part + (chain ? 0 : w)) * p.acc_cols);
-                // two warps keep dealing across tiles (an odd nK alternates which warp
-                // takes the extra K-step); the epilogue's p0 + p1 is commutative, so a
-                // row's sum does not depend on which partial holds which K-steps
-                int own = nmma == 2 ? (int)((i * nK) & 1) : 0;
-                bool first = true;              // the warp's first K-step of the tile overwrites
-                for (int kt = 0; kt < nK; ++kt) {
-                    if (own == w) {
-                        if (!wait_phase<32>(smem_u32(&bar_afull[t]), t_wraps & 1, abort_flag)) { ok = false; break; }
-                        if (!p.b_resident &&
-                            !wait_phase<32>(smem_u32(&bar_bfull[sb]), b_wraps & 1, abort_flag)) { ok = false; break; }
-                        const uint32_t g = (uint32_t)(i * nK + kt);
-                        // K-step g goes to warp g mod 2; it waits for the other warp's
-                        // arrival after K-step g - 1, the ((g + w) / 2)-th on its barrier
-                        if (chain && g > 0 &&
-                            !wait_phase<0>(smem_u32(&bar_turn[w]), (((g + (uint32_t)w) >> 1) + 1) & 1, abort_flag)) {
-                            ok = false;
-                            break;
+            // WHOLE: the warp runs the loop, a lane elected around the instructions; else
+            // (turns) one lane runs it
+            auto issue_tiles = [&](auto whole) {
+                constexpr bool WHOLE = decltype(whole)::value, chain = !WHOLE;
+                auto wait = [&](uint64_t *bar, uint32_t parity) {
+                    if constexpr (WHOLE) return warp_wait_phase<32>(smem_u32(bar), parity, abort_flag);
+                    else return wait_phase<32>(smem_u32(bar), parity, abort_flag);
+                };
+                auto leads = [&] {
+                    if constexpr (WHOLE) return elect_one();
+                    else return true;
+                };
+                auto join = [&] {
+                    if constexpr (WHOLE) __syncwarp();
+                };
+                bool ok = true;
+                if (p.b_resident) ok = wait(&bar_bfull[0], 0);
+                const uint64_t desc_b0 = sw128_desc(b_region);
+                const uint32_t b_step16 = b_step >> 4, lo16 = (uint32_t)Nt * 128 >> 4;
+                int t = 0, sb = 0;                  // ring slots of K-step kt (every warp tracks every step)
+                uint32_t t_wraps = 0, b_wraps = 0;
+                for (int64_t i = 0; ok && i < my_tiles; ++i) {
+                    const int a = nacc == 2 ? (int)(i & 1) : 0;
+                    const int64_t use = nacc == 2 ? (i >> 1) : i;
+                    if (use >= 1 && !wait(&bar_accempty[a], (uint32_t)((use - 1) & 1))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t d = tmem + (uint32_t)((a * p.n_part + (chain ? 0 : w)) * p.acc_cols);
+                    // two warps keep dealing across tiles (an odd nK alternates which warp
+                    // takes the extra K-step); the epilogue's p0 + p1 is commutative, so a
+                    // row's sum does not depend on which partial holds which K-steps
+                    int own = nmma == 2 ? (int)((i * nK) & 1) : 0;
+                    bool first = true;              // the warp's first K-step of the tile overwrites
+                    for (int kt = 0; kt < nK; ++kt) {
+                        if (own == w) {
+                            if (!wait(&bar_afull[t], t_wraps & 1)) { ok = false; break; }
+                            if (!p.b_resident && !wait(&bar_bfull[sb], b_wraps & 1)) { ok = false; break; }
+                            const uint32_t g = (uint32_t)(i * nK + kt);
+                            // K-step g goes to warp g mod 2; it waits for the other warp's
+                            // arrival after K-step g - 1, the ((g + w) / 2)-th on its barrier
+                            if (chain && g > 0 &&
+                                !wait_phase<0>(smem_u32(&bar_turn[w]), (((g + (uint32_t)w) >> 1) + 1) & 1, abort_flag)) {
+                                ok = false;
+                                break;
+                            }
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint64_t dh = desc_b0 + (uint64_t)((p.b_resident ? kt : sb) * b_step16), dl = dh + lo16;
+                            // shared accumulator: K-step 0 of the tile overwrites
+                            const uint32_t acc0 = chain ? (kt > 0 ? 1u : 0u) : (first ? 0u : 1u);
+                            if (leads()) {
+                                if (merged) mma_block_merged(d, tmem + p.a_col + t * kAColsPerStage, dh, id2, id, acc0);
+                                else mma_block<THREE, 0, Q>(d, tmem + p.a_col + t * kAColsPerStage, dh, dl, id, acc0);
+                                if (chain) {
+                                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                                    mbar_arrive(smem_u32(&bar_turn[1 - w]));
+                                }
+                                mma_commit(smem_u32(&bar_aempty[t]));
+                                if (!p.b_resident) mma_commit(smem_u32(&bar_bempty[sb]));
+                            }
+                            join();
+                            first = false;
                         }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint64_t dh = desc_b0 + (uint64_t)((p.b_resident ? kt : sb) * b_step16), dl = dh + lo16;
-                        // shared accumulator: K-step 0 of the tile overwrites
-                        const uint32_t acc0 = chain ? (kt > 0 ? 1u : 0u) : (first ? 0u : 1u);
-                        if (merged) mma_block_merged(d, tmem + p.a_col + t * kAColsPerStage, dh, id2, id, acc0);
-                        else mma_block<THREE, 0, Q>(d, tmem + p.a_col + t * kAColsPerStage, dh, dl, id, acc0);
-                        first = false;
-                        if (chain) {
-                            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                            mbar_arrive(smem_u32(&bar_turn[1 - w]));
-                        }
-                        mma_commit(smem_u32(&bar_aempty[t]));
-                        if (!p.b_resident) mma_commit(smem_u32(&bar_bempty[sb]));
+                        if (++own == nmma) own = 0;
+                        if (++t == p.n_stages) { t = 0; ++t_wraps; }
+                        if (!p.b_resident && ++sb == p.nb) { sb = 0; ++b_wraps; }
                     }
-                    if (++own == nmma) own = 0;
-                    if (++t == p.n_stages) { t = 0; ++t_wraps; }
-                    if (!p.b_resident && ++sb == p.nb) { sb = 0; ++b_wraps; }
+                    if (!ok) break;
+                    if (leads()) mma_commit(smem_u32(&bar_accfull[a]));
+                    join();
                 }
-                if (!ok) break;
-                mma_commit(smem_u32(&bar_accfull[a]));
+                // every MMA of every issuing warp has finished before the teardown
+                if (leads()) mma_commit(smem_u32(&bar_drain));
+                join();
+                wait_phase_drain(smem_u32(&bar_drain), 0);
+            };
+            if (MODE != 2 && p.mma_chain) {
+                if (lane == 0) issue_tiles(std::false_type());
+            } else {
+                issue_tiles(std::true_type());
             }
-            // every MMA of every issuing warp has finished before the teardown
-            mma_commit(smem_u32(&bar_drain));
-            wait_phase_drain(smem_u32(&bar_drain), 0);
         }
     } else {
         // -------------------------------------------------------------- weights --
-        if (MODE == 3 && lane == 0) {
+        const bool leader = elect_one();
+        if (MODE == 3 && leader) {
             // the weight K-steps, each copy as soon as the MMAs have released its slot (the
             // staged input rows come from warp 10)
             const int64_t n_b = p.b_resident ? 0 : total;
@@ -1694,7 +1741,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
             // the copies still in flight land before the shared memory is released
             for (int64_t jj = jb > p.nb ? jb - p.nb : 0; jj < jb; ++jj)
                 wait_phase_drain(smem_u32(&bar_bfull[(int)(jj % p.nb)]), (uint32_t)((jj / p.nb) & 1));
-        } else if (lane == 0) {
+        } else if (leader) {
             if (p.b_resident) {
                 const uint32_t bytes = (uint32_t)nK * b_step;
                 mbar_expect_tx(smem_u32(&bar_bfull[0]), bytes);
@@ -1999,6 +2046,7 @@ static void tc_config(TcParams &p, int nt_max, bool three, bool chain)
         p.mma_chain = 1;
     }
 }
+
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to libcuda).
 static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
