@@ -333,12 +333,12 @@ __device__ __forceinline__ f32x2 tanh2(f32x2 v)
 
 // A block of 128 threads runs up to p.bm rows of one mutant through every step.  Thread 2u
 // holds the recurrent weights of unit u's gates i and f, thread 2u + 1 those of g and o, in
-// registers (64 x 2) for all steps: no weight is loaded again.  (With the weights in shared
-// memory every group of rows re-read all 64 KB per step, and that, not the FMAs, bound the
-// kernel: 4.1k cycles per step before any row.)  What bounds it now is the return path of the
-// shared-memory loads of h, 128 bytes per cycle: 1.2k cycles per four rows on an SM, one or two
-// blocks there alike, against 512 of FMAs.  Rows go four at a time: a 16-byte uniform load brings h of four units of a row for
-// 8 FMAs per thread.  The two threads of a unit then swap half of their sums, so that each
+// registers (64 x 2) for all steps: no weight is loaded again.  (A version with the weights in
+// shared memory took 6.2k cycles per step of 8 rows and 8.2k of 16.)  What bounds it now is issue:
+// 1.3k cycles per four rows and step with one block on an SM, 1.2k per block with two; ncu shows
+// an instruction per warp every 1.9 cycles, the rest fixed latencies and dispatch stalls (an FMA
+// with three registers of its own issues at two thirds of the rate).  Rows go four at a time: a
+// 16-byte uniform load brings h of four units of a row for 8 FMAs per thread.  The two threads of a unit then swap half of their sums, so that each
 // finishes two rows' cells.  h (double-buffered: one barrier per step) and c live in shared
 // memory; the next rows' stored sums are fetched while the current ones run.
 constexpr int kRecThreads = 2 * kMaxUnits;
