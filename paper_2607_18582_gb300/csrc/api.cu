@@ -881,6 +881,33 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
     const int64_t G = rm.R / rm.T;
     const int64_t delta_flops =
         (dt.dot_prefix[g0 + G] - dt.dot_prefix[g0]) * rm.T * 2 * (int64_t)Sl.oh * Sl.ow * Sl.K;
+    // an LSTM on the embedding, by token: its rows' sums come from the tokens' rows (the batch's
+    // tile must hold at least two positions per token of the whole cache: past that the rows
+    // themselves are as few)
+    const bool by_token = !vanilla && !ec.skip_unchanged && l <= 1 && L > 2 && ca->tok_n > 0 &&
+                          2 * (int64_t)ca->tok_n <= (int64_t)rm.T * m->st[1].iw;
+    LstmTokens tk;
+    if (by_token) {
+        tk.tok = ca->tok;
+        tk.id = ca->tok_id;
+        tk.n = ca->tok_n;
+        tk.rows = m->st[0].Wt;
+    }
+    if (by_token && l == 0) {
+        // a mutant of the embedding: the tokens' rows as it has them, no row materialised
+        acct.bytes_gather += G * (int64_t)tk.n * Sl.oc * 4;
+        timed(C_DELTA, delta_flops, [&] { return launch_embed_tokens(Sl, pa, (int)G, tk, ws.xb[1], s); });
+        tk.rows = ws.xb[1];
+        tk.rows_g = 1;
+        acct.bytes_rows += 2 * (int64_t)rm.R * m->xd[2].size * 4;
+        timed(1, 2 * m->st[1].macs * rm.R, [&] {
+            return launch_lstm(m->st[1], Src{nullptr, 0, 0}, rm, nullptr, 0, ws.xb[2], m->xd[2].stride, nullptr, ws.lw, s, &tk);
+        });
+        for (int v = 2; v < L - 1; ++v) stage(v, nullptr, 0);
+        const Stage &SLe = m->st[L - 1];
+        timed(L - 1, 2 * SLe.macs * rm.R, [&] { return launch_final_dense(SLe, xsrc(SLe.in_src), rm, fa, s); });
+        return launches;
+    }
     if (Sl.kind == MURE_NODE_LSTM) {
         // a mutated LSTM layer: its recurrence spreads one unit's change to every unit
         // from the first step on, so the layer itself is recomputed for every row from
@@ -892,7 +919,8 @@ int run_batch(mure_ctx *c, const mure_model *m, const mure_cache *ca, const DevT
         timed(l, 2 * Sl.macs * rm.R, [&] {
             LstmWs lw = ws.lw;
             lw.kmax = dt.kmax_layer[l];
-            return launch_lstm(Sl, xsrc(Sl.in_src), rm, nullptr, 0, ws.xb[l + 1], m->xd[l + 1].stride, &pa, lw, s);
+            return launch_lstm(Sl, xsrc(Sl.in_src), rm, nullptr, 0, ws.xb[l + 1], m->xd[l + 1].stride, &pa, lw, s,
+                               by_token ? &tk : nullptr);
         });
         for (int v = l + 1; v < L - 1; ++v) stage(v, nullptr, 0);
         const Stage &SLr = m->st[L - 1];
@@ -1417,7 +1445,19 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         for (int s2 = 0; s2 <= L; ++s2) ox[s2] = place(m->xd[s2].stride);
         for (int v = 0; v < L; ++v) oz[v] = place(m->zd[v].stride);
         const size_t op = place(1), ol = place(1);
+        // an embedding that an LSTM reads, and it alone: the positions' token numbers and the
+        // tokens' ids
+        const Stage &S0 = m->st[0];
+        bool tokens = full && n_in > 0 && L > 2 && S0.kind == MURE_NODE_EMBED && !S0.act1 && !S0.act2 && !S0.has_add &&
+                      m->st[1].kind == MURE_NODE_LSTM && m->st[1].in_src == 1;
+        for (int v = 2; v < L; ++v) tokens = tokens && m->st[v].in_src != 1 && !(m->st[v].has_add && m->st[v].skip_src == 1);
+        const int64_t steps = S0.iw, most = std::min<int64_t>(S0.vocab, np * steps);
+        const size_t ot = tokens ? place(steps) : 0, oi = tokens ? place((most + np - 1) / np) : 0;
         ca->mem = (char *)dalloc(c, off);
+        if (tokens) {
+            ca->tok = (int32_t *)(ca->mem + ot);
+            ca->tok_id = (int32_t *)(ca->mem + oi);
+        }
         auto tensor = [&](size_t o, const TensorDim &d) {
             float *p = (float *)(ca->mem + o);
             if (d.stride != d.size || n_in == 0) CK(c, cudaMemsetAsync(p, 0, np * d.stride * 4, s));
@@ -1449,8 +1489,32 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         for (int s2 = 0; s2 <= L; ++s2) xs[s2] = ca->x[s2];
         for (int v = 0; v < L; ++v) zs[v] = ca->z[v];
         const RowMap rm{0, (int)ca->n_pad, (int)ca->n_pad};
+        int32_t *tok_count = nullptr;
+        LstmTokens tk;
+        if (ca->tok) {
+            const int vocab = m->st[0].vocab, steps = m->st[0].iw;
+            int32_t *seen = sc.get<int32_t>(vocab + 1), *slot = sc.get<int32_t>(vocab);
+            tok_count = seen + vocab;
+            CK(c, cudaMemsetAsync(seen, 0, ((size_t)vocab + 1) * 4, s));
+            c->launches += launch_tokens(Src{ca->x[0], m->xd[0].stride, 0}, ca->n_pad, steps, vocab, seen, slot, ca->tok_id,
+                                         tok_count, ca->tok, s);
+            check_launch(c);
+            tk.tok = ca->tok;
+            tk.id = ca->tok_id;
+            tk.n_dev = tok_count;
+            tk.n = (int)std::min<int64_t>(vocab, ca->n_pad * steps);
+            tk.rows = m->st[0].Wt;
+        }
         for (int v = 0; v < L - 1; ++v) {
             const Stage &S = m->st[v];
+            if (v == 1 && ca->tok && tk.n <= ca->n_pad * S.iw) {
+                LstmWs lw;
+                lw.proj = tmp;
+                c->launches += launch_lstm(S, Src{nullptr, 0, 0}, rm, zs[1], m->zd[1].stride, xs[2], m->xd[2].stride, nullptr,
+                                           lw, s, &tk);
+                check_launch(c);
+                continue;
+            }
             const Src skip = S.has_add ? Src{xs[S.skip_src], m->xd[S.skip_src].stride, 0} : Src{nullptr, 0, 0};
             c->launches += launch_stage_simt(S, Src{xs[S.in_src], m->xd[S.in_src].stride, 0}, rm, zs[v], m->zd[v].stride, skip,
                                              xs[v + 1], m->xd[v + 1].stride, tmp, s);
@@ -1481,6 +1545,7 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         Results res(c);
         res.add(hm, mask, sizeof hm);
         res.add(&dev_err, c->err_dev, sizeof(int));
+        if (tok_count) res.add(&ca->tok_n, tok_count, sizeof(int));
         res.finish();
         if (hm[kLabelWords]) {
             // the first bad label, as for labels on the host

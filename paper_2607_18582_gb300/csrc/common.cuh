@@ -104,6 +104,9 @@ struct mure_cache {
     char *mem = nullptr;              // one allocation for all of the below
     std::vector<float *> x;           // x[s], s = 0..L: [n_pad][xd[s].stride]
     std::vector<float *> z;           // z[v], v = 0..L-1: [n_pad][zd[v].stride]
+    // an embedding followed by an LSTM: each position's token number, the tokens' ids, their count
+    int32_t *tok = nullptr, *tok_id = nullptr;
+    int tok_n = 0;
     int32_t *pred0 = nullptr;         // [n_pad]
     int32_t *label = nullptr;         // [n_pad]
     int n_label_values = 0;           // |L|: distinct labels among the inputs
@@ -232,8 +235,19 @@ struct LstmWs {
     int kmax = 0;
 };
 int64_t lstm_proj_floats(const Stage &S);   // proj floats per row (0: not an LSTM layer)
+// The inputs of an LSTM that follows an embedding, by distinct token: tok [input][step] numbers
+// them, id their entries in the table.  rows: the table [vocab][dim], or (rows_g) every mutant's
+// rows [mutant][token][dim].  n_dev: the device's count where the host has only a bound n.
+struct LstmTokens {
+    const int32_t *tok = nullptr, *id = nullptr, *n_dev = nullptr;
+    int n = 0, rows_g = 0;
+    const float *rows = nullptr;
+};
+int launch_tokens(const Src &x, int64_t rows, int steps, int vocab, int32_t *seen, int32_t *slot, int32_t *tok_id, int32_t *count,
+                  int32_t *tok, cudaStream_t s);
+int launch_embed_tokens(const Stage &S, const PatchArgs &pa, int G, const LstmTokens &tk, float *out, cudaStream_t s);
 int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, float *y_out, int64_t y_stride,
-                const PatchArgs *pa, const LstmWs &lw, cudaStream_t s);
+                const PatchArgs *pa, const LstmWs &lw, cudaStream_t s, const LstmTokens *tk = nullptr);
 
 // Global average pooling of R rows of a [P][C] map.
 int launch_gap(const float *in, int64_t in_stride, int P, int C, int R, float *y, int64_t y_stride, cudaStream_t s);

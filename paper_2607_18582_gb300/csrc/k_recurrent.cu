@@ -53,6 +53,57 @@ __global__ void __launch_bounds__(256) k_embed(const EmbedParams p)
     p.y[row * p.y_stride + (int64_t)t * p.dim + j] = v;
 }
 
+// A text repeats its words: the first LSTM's input sums depend on a position's token alone, so
+// they are needed once per distinct token of the inputs (2,010 among 40,000 positions of 500
+// synthetic reviews), not once per position.  k_tokens numbers the distinct ids (in no particular
+// order), k_token_map gives every position its token's number.
+__global__ void __launch_bounds__(256) k_tokens(const float *x, int64_t x_stride, int steps, int64_t n, int vocab,
+                                                int32_t *seen, int32_t *slot, int32_t *tok_id, int32_t *count)
+{
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const float idf = __ldg(x + i / steps * x_stride + i % steps);
+    const int id = idf >= 0.f && idf < (float)vocab ? (int)idf : 0;   // (k_embed refuses the others)
+    if (__ldcg(seen + id) == 0 && atomicExch(seen + id, 1) == 0) {   // (a seen id, the usual one, needs no atomic)
+        const int k = atomicAdd(count, 1);
+        tok_id[k] = id;
+        slot[id] = k;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_token_map(const float *x, int64_t x_stride, int steps, int64_t n, int vocab,
+                                                   const int32_t *slot, int32_t *tok)
+{
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    const float idf = __ldg(x + i / steps * x_stride + i % steps);
+    tok[i] = slot[idf >= 0.f && idf < (float)vocab ? (int)idf : 0];
+}
+
+// The embedding rows of the tokens as each mutant of the embedding has them: out[g][token][dim],
+// a mutated channel's entry with the delta's arithmetic (its sum over the one-hot input is
+// 0 + e[id]).
+__global__ void __launch_bounds__(256) k_embed_tokens(const PatchArgs pa, const float *__restrict__ Wt,
+                                                      const int32_t *__restrict__ tok_id,
+                                                      int n_tok, int dim, int vocab, float *__restrict__ out)
+{
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x, per_g = (int64_t)n_tok * dim;
+    const int g = blockIdx.y;
+    if (i >= per_g) return;
+    const int k = (int)(i / dim), j = (int)(i - (int64_t)k * dim), id = __ldg(tok_id + k);
+    float v = __ldg(Wt + (int64_t)id * dim + j);
+    const int n = pa.n_neurons[g], op = pa.op[g];
+    const int32_t *ids = pa.ids + pa.neuron_off[g];
+    for (int q = 0; q < n; ++q) {
+        if (ids[q] != j) continue;
+        if (op == MURE_OP_NEB) v = 0.f;
+        else if (op == MURE_OP_NAI) v = -v;
+        else if (op == MURE_OP_NS) v = __ldg(Wt + (int64_t)id * dim + ids[q ^ 1]);
+        else v = v + (0.f + __ldg(pa.patch + pa.patch_off[g] + (int64_t)q * vocab + id));
+    }
+    out[g * per_g + i] = v;
+}
+
 // --------------------------------------------------------------------- LSTM --
 //
 // A gate's pre-activation at step t is one fp32 FMA chain from +0: its input weights on x_t
@@ -64,11 +115,13 @@ __global__ void __launch_bounds__(256) k_embed(const EmbedParams p)
 //                memory for all steps), the bias and the cell.
 // A stored partial sum is exact, so the result is that of the uncut chain.  Measured on the
 // IMDB-sized model (500 inputs x 40 mutants): 62.3 ms in one kernel that read a weight from
-// global memory per FMA -> 1.1 (proj, 60 TFLOP/s, 0.86 of cuBLAS fp32) + 2.0 ms (rec).  The part on x_t
+// global memory per FMA -> 1.2 (proj, 60 TFLOP/s, 0.86 of cuBLAS fp32) + 2.0 ms (rec).  The part on x_t
 // depends on the row's input alone but for a mutant's own units: where the rows read cached
 // inputs, one product per input serves all mutants of a batch (it is two thirds of the
 // 128-input layer's work), and each mutant adds the columns of its mutated units
-// (k_lstm_cols, k_lstm_proj with the mutant as grid z).
+// (k_lstm_cols, k_lstm_proj with the mutant as grid z).  Behind an embedding the products take a
+// row per distinct token instead (k_tokens): proj 1.2 -> 0.65 ms; the recurrence looks the rows
+// up, two groups ahead.
 
 constexpr int kMaxUnits = 64;   // units per layer
 constexpr int kMaxIn = 128;     // input width
@@ -120,6 +173,8 @@ __global__ void __launch_bounds__(128) k_lstm_cols(const PatchArgs pa, const flo
 }
 
 struct ProjParams {
+    const int32_t *tok_id;  // rows of x are this list's entries (tokens; steps = 1), else null
+    const int32_t *m_dev;   // GEMM rows counted on the device (M is then their bound), else null
     const float *x; int64_t x_stride; int x_per_input;
     int64_t t0; int T;
     const int32_t *lrow;
@@ -149,10 +204,12 @@ __global__ void __launch_bounds__(256, VEC ? 2 : 1) k_lstm_proj(const ProjParams
     const int tn = (warp % (CT / CL)) * CL + lane % CL, tm = (warp / (CT / CL)) * RL + lane / CL;
     const int mt = (int)(blockIdx.x / p.n_tiles), n0 = (int)(blockIdx.x - mt * p.n_tiles) * BN;
     const float *B = p.B + z * p.b_stride;
+    const int64_t M = p.m_dev ? (int64_t)*p.m_dev : p.M;
+    if ((int64_t)mt * BM >= M) return;
     // this thread's A pieces: four k of row tid % BM
     const float *xr = nullptr;
-    if (const int64_t m = (int64_t)mt * BM + tid % BM; m < p.M) {
-        const int64_t row = m / p.steps + z * p.z_rows;
+    if (const int64_t m = (int64_t)mt * BM + tid % BM; m < M) {
+        const int64_t row = p.tok_id ? p.tok_id[m] : m / p.steps + z * p.z_rows;
         const int t = (int)(m % p.steps);
         xr = p.x + (p.x_per_input ? p.t0 + logical_row(p.lrow, row) % p.T : row) * p.x_stride + (int64_t)t * p.cin;
     }
@@ -215,7 +272,7 @@ __global__ void __launch_bounds__(256, VEC ? 2 : 1) k_lstm_proj(const ProjParams
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int64_t mm = (int64_t)mt * BM + (i / 4) * RS + tm * 4 + (i & 3);
-        if (mm >= p.M) continue;
+        if (mm >= M) continue;
 #pragma unroll
         for (int j = 0; j < TN; j += 4) {
             const int n = n0 + (j / 4) * CS + tn * 4;
@@ -228,8 +285,10 @@ __global__ void __launch_bounds__(256, VEC ? 2 : 1) k_lstm_proj(const ProjParams
 
 struct LstmParams {
     const float *proj; int proj_shared;   // [row][steps][4H]; shared: rows are the tile's inputs
-    const float *projx;                   // mutated units: slot q of mutant g at g px_g + row px_row + step px_step + 4 q
-    int64_t px_g, px_row; int px_step;
+    const int32_t *tok; int64_t t0;       // sums per token: of input t0 + row at step t, number tok[..] (else null)
+    int64_t proj_g;                       // floats between the mutants' sums (tokens of each mutant)
+    const float *projx;                   // mutated units: slot q of mutant g at g px_g + (row steps + step, or token) px_step + 4 q
+    int64_t px_g; int px_step;
     int rows_per_g, bm, blocks_per_g;     // rows of a mutant (or all rows); rows per block
     int steps, cin, H, seq;
     const float *W;       // [H][4][cin + H]
@@ -360,8 +419,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_lstm_rec(const LstmParams p)
     LstmSlot sl;
     sl.unit = sl.partner = live ? u : 0;
     bool changed = false, blocked = false;
-    const float *pp = p.proj + ((p.proj_shared ? first : row0) * p.steps) * N + 2 * tid;
-    int64_t p_row = (int64_t)p.steps * N;
+    const float *pp = p.proj + (p.tok ? g * p.proj_g : ((p.proj_shared ? first : row0) * p.steps) * N) + 2 * tid;
     int p_step = N;
     if (p.mutated && live)
         for (int q = 0; q < p.pa.n_neurons[g]; ++q) {
@@ -371,8 +429,7 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_lstm_rec(const LstmParams p)
             changed = true;
             blocked = c.op == MURE_OP_NEB;
             p_step = p.px_step;
-            p_row = p.px_row;
-            pp = p.projx + g * p.px_g + first * p_row + 4 * q + 2 * hi;
+            pp = p.projx + g * p.px_g + (p.tok ? 0 : (int64_t)first * p.steps * p_step) + 4 * q + 2 * hi;
         }
     float w0[kMaxUnits], w1[kMaxUnits];
 #pragma unroll
@@ -388,13 +445,24 @@ __global__ void __launch_bounds__(kRecThreads, 2) k_lstm_rec(const LstmParams p)
     const float b0 = lstm_bias(sl, p.b, 2 * hi), b1 = lstm_bias(sl, p.b, 2 * hi + 1);
     for (int i = tid; i < 2 * p.bm * kRecLine; i += kRecThreads) hs[i] = 0.f;
     for (int i = tid; i < p.bm * kMaxUnits; i += kRecThreads) cs[i] = 0.f;
+    // the stored sums of rows r0 .. r0 + 3 at step t, one group of rows ahead of their use; where
+    // they go by token, the numbers of the tokens two groups ahead
     float2 pre[4];
+    int32_t tk[4];
+    const int32_t *tok = p.tok ? p.tok + (p.t0 + first) * p.steps : nullptr;
+    auto number = [&](int r0, int t) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tk[i] = tok && r0 + i < nr && t < p.steps ? __ldg(tok + (int64_t)(r0 + i) * p.steps + t) : 0;
+    };
     auto fetch = [&](int r0, int t) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            pre[i] = live && r0 + i < nr ? __ldg(reinterpret_cast<const float2 *>(pp + (r0 + i) * p_row + (int64_t)t * p_step))
-                                         : make_float2(0.f, 0.f);
+        for (int i = 0; i < 4; ++i) {
+            const int64_t at = tok ? (int64_t)tk[i] : (int64_t)(r0 + i) * p.steps + t;
+            pre[i] = live && r0 + i < nr ? __ldg(reinterpret_cast<const float2 *>(pp + at * p_step)) : make_float2(0.f, 0.f);
+        }
+        if (tok) number(r0 + 4 < nr ? r0 + 4 : 0, r0 + 4 < nr ? t : t + 1);
     };
+    if (tok) number(0, 0);
     fetch(0, 0);
     __syncthreads();
     for (int t = 0; t < p.steps; ++t) {
@@ -495,6 +563,30 @@ int launch_embed(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_strid
     return 1;
 }
 
+int launch_tokens(const Src &x, int64_t rows, int steps, int vocab, int32_t *seen, int32_t *slot, int32_t *tok_id, int32_t *count,
+                  int32_t *tok, cudaStream_t s)
+{
+    const int64_t n = rows * steps;
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    k_tokens<<<blocks, 256, 0, s>>>(x.p, x.stride, steps, n, vocab, seen, slot, tok_id, count);
+    k_token_map<<<blocks, 256, 0, s>>>(x.p, x.stride, steps, n, vocab, slot, tok);
+    return 2;
+}
+
+int launch_embed_tokens(const Stage &S, const PatchArgs &pa, int G, const LstmTokens &tk, float *out, cudaStream_t s)
+{
+    const int64_t per_g = (int64_t)tk.n * S.oc;
+    PatchArgs a = pa;
+    int launches = 0;
+    for (int g0 = 0; g0 < G; g0 += 65535, ++launches) {   // the grid's y limit
+        const int gn = G - g0 < 65535 ? G - g0 : 65535;
+        k_embed_tokens<<<dim3((unsigned)((per_g + 255) / 256), (unsigned)gn), 256, 0, s>>>(a, S.Wt, tk.id, tk.n, S.oc,
+                                                                                         S.vocab, out + g0 * per_g);
+        a.op += gn; a.n_neurons += gn; a.neuron_off += gn; a.patch_off += gn;
+    }
+    return launches;
+}
+
 int64_t lstm_proj_floats(const Stage &S) { return S.kind == MURE_NODE_LSTM ? (int64_t)S.iw * 4 * S.oc : 0; }
 
 namespace {
@@ -515,13 +607,13 @@ void proj(ProjParams q, int nz, cudaStream_t s)
 }  // namespace
 
 int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, float *y_out, int64_t y_stride,
-                const PatchArgs *pa, const LstmWs &lw, cudaStream_t s)
+                const PatchArgs *pa, const LstmWs &lw, cudaStream_t s, const LstmTokens *tk)
 {
     if (rm.R <= 0) return 0;
     int launches = 0;
     // rows that read cached inputs share their inputs' sums (not in a compacted batch, whose
     // rows are any inputs in any order)
-    const bool shared = x.per_input && !rm.lrow;
+    const bool shared = (x.per_input && !rm.lrow) || (tk && !tk->rows_g);
     ProjParams q{};
     q.x = x.p; q.x_stride = x.stride; q.x_per_input = x.per_input;
     q.t0 = rm.t0; q.T = rm.T; q.lrow = rm.lrow;
@@ -529,12 +621,23 @@ int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride
     q.M = (int64_t)(shared ? rm.T : rm.R) * S.iw;
     q.B = S.Wt;
     q.out = lw.proj;
+    LstmParams p{};
+    if (tk) {
+        // a GEMM row per token: entries of the embedding's table, or each mutant's rows of it
+        q.x = tk->rows; q.x_stride = S.ic; q.x_per_input = 0;
+        q.steps = 1;
+        q.tok_id = tk->rows_g ? nullptr : tk->id;
+        q.m_dev = tk->rows_g ? nullptr : tk->n_dev;
+        q.M = tk->rows_g ? (int64_t)tk->n * (rm.R / rm.T) : tk->n;
+        p.tok = tk->tok;
+        p.t0 = rm.t0;
+        p.proj_g = tk->rows_g ? (int64_t)tk->n * q.N : 0;
+    }
     proj<128, 128, 8, 8, 8>(q, 1, s);
     ++launches;
-    LstmParams p{};
     if (pa && lw.kmax > 0) {
         const int G = rm.R / rm.T, cols = 4 * lw.kmax;
-        q.M = (int64_t)rm.T * S.iw;
+        if (!tk) q.M = (int64_t)rm.T * S.iw;
         q.B = lw.cols;
         q.out = lw.projx;
         p.projx = lw.projx;
@@ -563,12 +666,11 @@ int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride
                 ++launches;
             }
         }
-        p.px_row = (int64_t)S.iw * p.px_step;
         ++launches;
     }
     p.proj = lw.proj; p.proj_shared = shared;
     // blocks of one mutant's rows (or one input tile's, where its sums are shared)
-    const int rows_per_g = pa || shared ? rm.T : rm.R, G = rm.R / rows_per_g;
+    const int rows_per_g = pa || shared || tk ? rm.T : rm.R, G = rm.R / rows_per_g;
     p.rows_per_g = rows_per_g;
     p.steps = S.iw; p.cin = S.ic; p.H = S.oc; p.seq = S.kh;
     p.W = S.W; p.Wt = S.Wt; p.b = S.b;

@@ -96,6 +96,23 @@ def test_lstm_split_over_batches(M, ctx, oracle_mod, n_in, per_layer):
     assert ok, worst
 
 
+@pytest.mark.parametrize("n_in,vocab", [(1, 2), (70, 129), (300, 129), (300, 700), (70, 4000)])
+def test_lstm_sums_by_token(M, ctx, n_in, vocab):
+    """The first LSTM's input sums per distinct token (few tokens) or per position (many, or a
+    small tile of inputs): the bits of vanilla, which always takes the positions; token counts
+    at the edges of a product's 128 rows, every operator on the embedding and the first LSTM."""
+    model = wl.rnn(4, n_classes=3, vocab=vocab, dim=13, units=(9, 6), steps=5, name="rnn_tokens")
+    X = wl.inputs(model, n_in, 5)
+    table = wl.concat([wl.mutants(model, 12, seed=30 + l, ratios=(0.3,), ops=wl.OPS, layers=[l]) for l in (0, 1)])
+    m = M.mure_model_load(ctx, model)
+    cache = M.mure_build_prefix_cache(m, X)
+    v = M.mure_eval_vanilla(m, X, table, logits=True)
+    for r in (M.mure_eval_mutants(cache, table, logits=True),
+              M.mure_eval_mutants(cache, table, logits=True, workspace_bytes=1 << 19)):
+        assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+        assert np.array_equal(v["kill_bits"], r["kill_bits"])
+
+
 def test_recurrent_identity_mutants_and_bad_ids(M, ctx):
     model = small_rnn()
     X = wl.inputs(model, 64, 1)
