@@ -306,10 +306,13 @@ struct LstmParams {
 // sigmoid = 1 / (1 + exp(-v)), 0 below -87; |tanh| = 1 - 2 e / (1 + e) with e = exp(-2 |v|), and
 // below 0.6, where that cancels, the odd polynomial x + x^3 P(x^2) (minimax fit in x^2,
 // relative error 3e-9).  The arguments are clamped to where the result is already 0 or 1 (a NaN
-// passes).  Against 64 bits over [-100, 100], worst and rms relative error: sigmoid 1.9e-7 and
-// 3.7e-8 (1 / (1 + expf(-v)): 2.1e-7 and 4.2e-8), tanh 1.8e-7 and 1.6e-8 (tanhf: 2.0e-7 and
-// 2.1e-8).  With those functions, scalar, a step of 4 rows took 0.86 us, now 0.66.
-constexpr float kLog2e = 1.44269502f, kLog2eTail = 1.92596303e-8f, kLn2 = 0.693147182f;
+// passes).  Against 64 bits over [-100, 100], worst and rms relative error: sigmoid 1.6e-7 and
+// 3.3e-8 (1 / (1 + expf(-v)): 2.1e-7 and 4.2e-8), tanh 1.6e-7 and 1.5e-8 (tanhf: 2.0e-7 and
+// 2.1e-8).  The mean error matters more than the rms, since a recurrence adds it up: without the
+// term for ex2's own (kEx2Lean) sigmoid leant by 3e-8 and the logits of the Reuters-sized model
+// were 1.87e-7 off (relative, over 6 tables), with it 1.69e-7; with the functions named, 1.83e-7.
+// Those, scalar, took 0.86 us for a step of 4 rows, these 0.66.
+constexpr float kLog2e = 1.44269502f, kLog2eTail = 1.92596303e-8f, kLn2 = 0.693147182f, kEx2Lean = 5.96046448e-8f;
 
 __device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
 
@@ -350,7 +353,14 @@ __device__ __forceinline__ f32x2 exp_neg2(f32x2 a, f32x2 &ec)
     const f32x2 e = pack2(ex2_approx(t.x), ex2_approx(t.y));
     f32x2 d = fma2(a, both(S * kLog2e), nt);                           // what the rounding lost
     d = fma2(a, both(S * kLog2eTail), d);
-    ec = mul2(mul2(d, both(-kLn2)), e);
+    if (S == 1) {
+        // ex2 reads high by 2^-24 of the exponent above 1, low below -1, in between less (measured)
+        d = fma2(pack2(min_nan(max_nan(t.x, -1.f), 1.f), min_nan(max_nan(t.y, -1.f), 1.f)), both(kEx2Lean), d);
+        d = mul2(d, both(-kLn2));
+    } else {
+        d = fma2(d, both(-kLn2), both(kLn2 * kEx2Lean));              // used below -1 only
+    }
+    ec = mul2(d, e);
     return e;
 }
 
