@@ -629,13 +629,24 @@ struct SmallSteps {
     }
 };
 
+// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; with the output layer in the
+// epilogue (FCP > 0) a second set of epilogue warps, since there the epilogue bounds the layer:
+// a row costs F x 12 FMAs and as many weight words from shared memory.  LeNet-5's 120 -> 84 -> 10
+// over 904,000 rows: 275 us with one set that tested each input's index, 208 without the tests
+// (the weights' loads then run ahead of the sums), 162 with two sets.
+template <int FCP>
+constexpr int tc_threads()
+{
+    return FCP > 0 ? kThreads + 128 : kThreads;
+}
+
 // MODE 0: dense layer (one GEMM row per batch row); 1: implicit-GEMM convolution; 2:
 // the small-image convolution; 3: the staged convolution (see TcParams).  THREE: 3xTF32 (else one TF32 product).  FCP > 0
 // (dense, one N slice): the output layer, with up to FCP classes, is computed from
 // each row's outputs in the epilogue, followed by the kill epilogue, and the rows
 // themselves are not stored.
 template <int MODE, bool THREE, int FCP = 0>
-__global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__ TcParams p)
+__global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_constant__ TcParams p)
 {
     static_assert(FCP == 0 || (MODE == 0 && FCP % 4 == 0) || (MODE == 3 && FCP == -1),
                   "the output layer is fused into dense layers only; -1: the staged mode's slot GEMM with a residual add");
@@ -689,13 +700,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if constexpr (FCP > 0) {
-        for (int i = threadIdx.x; i < p.ff.F * FCP; i += kThreads) {
+        for (int i = threadIdx.x; i < p.ff.F * FCP; i += tc_threads<FCP>()) {
             const int f = i / FCP, c = i % FCP;
             const float wv = c < p.ff.C ? p.ff.W[(int64_t)c * p.ff.F + f] : 0.f;
             asm volatile("st.shared.f32 [%0], %1;" ::"r"(fw_region + 4 * i), "f"(wv) : "memory");
         }
     }
-    for (int n = threadIdx.x; n < kSliceMax; n += kThreads) {
+    for (int n = threadIdx.x; n < kSliceMax; n += tc_threads<FCP>()) {
         if (MODE == 2) bias_sh[n] = n < SmallConv::N ? p.b[n % SmallConv::OC] : 0.f;
         else bias_sh[n] = n_base + n < p.N ? p.b[n_base + n] : 0.f;
     }
@@ -1040,11 +1051,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
             }
             cp_async_wait<0>();
         }
-    } else if (warp < 8) {
+    } else if (warp < 8 || (FCP > 0 && warp >= 12)) {
         // ------------------------------------------------------------- epilogue --
         const int qd = warp & 3;
         const uint32_t lane_off = (uint32_t)(qd * 32) << 16;
-        for (int64_t i = 0; i < my_tiles; ++i) {
+        // with the output layer in the epilogue two sets of warps take the tiles in turn, a set
+        // to an accumulator (with one accumulator the second set has nothing to do)
+        const int sets = FCP > 0 && p.n_acc == 2 ? 2 : 1;
+        for (int64_t i = warp >= 12 ? (sets == 2 ? 1 : my_tiles) : 0; i < my_tiles; i += sets) {
             const int a = p.n_acc == 2 ? (int)(i & 1) : 0;
             const int64_t use = p.n_acc == 2 ? (i >> 1) : i;
             if (!warp_wait_phase<64>(smem_u32(&bar_accfull[a]), (uint32_t)(use & 1), abort_flag)) break;
@@ -1164,7 +1178,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
             // covers 4 rows x 128 bytes instead of 32 rows x 16 bytes
             float *stage = epi_stage[qd];
             const bool vec = DENSE || (p.N & 3) == 0;
-            if (!(!DENSE && p.pool))
+            if (FCP <= 0 && !(!DENSE && p.pool))
                 epi_ptr[qd][lane] = ri.ok ? yrow + (DENSE ? 0 : ((int64_t)ri.oy * p.ow + ri.ox) * p.N) : nullptr;
             float facc[FCP > 0 ? FCP : 1];
 #pragma unroll
@@ -1215,21 +1229,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_gemm(const __grid_constant__
                         for (int e = 0; e < 16; ++e) vh[e] = act_apply(p.act1, vh[e]);
                     }
                     if constexpr (FCP > 0) {
-                        // the output layer: fp32 FMAs over the inputs f in ascending
-                        // order, as the output-layer kernel does
+                        // the output layer: fp32 FMAs over the inputs f in ascending order, as
+                        // the output-layer kernel does (a whole block of 16 without a test per
+                        // input, so that the weights' loads run ahead of the sums)
+                        auto input = [&](int e) {
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const int f = n0 + h + e;
-                            if (f < p.N) {
-#pragma unroll
-                                for (int c4 = 0; c4 < FCP; c4 += 4) {
-                                    const float4 w4 = fw4[(f * FCP + c4) >> 2];
-                                    facc[c4] = fmaf(vh[e], w4.x, facc[c4]);
-                                    facc[c4 + 1] = fmaf(vh[e], w4.y, facc[c4 + 1]);
-                                    facc[c4 + 2] = fmaf(vh[e], w4.z, facc[c4 + 2]);
-                                    facc[c4 + 3] = fmaf(vh[e], w4.w, facc[c4 + 3]);
-                                }
+                            for (int c4 = 0; c4 < FCP; c4 += 4) {
+                                const float4 w4 = fw4[((n0 + h + e) * FCP + c4) >> 2];
+                                facc[c4] = fmaf(vh[e], w4.x, facc[c4]);
+                                facc[c4 + 1] = fmaf(vh[e], w4.y, facc[c4 + 1]);
+                                facc[c4 + 2] = fmaf(vh[e], w4.z, facc[c4 + 2]);
+                                facc[c4 + 3] = fmaf(vh[e], w4.w, facc[c4 + 3]);
                             }
+                        };
+                        if (n0 + h + 16 <= p.N) {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) input(e);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 16; ++e)
+                                if (n0 + h + e < p.N) input(e);
                         }
                     }
                     if (!DENSE && p.has_add && ri.ok) {
@@ -2272,7 +2291,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, kThreads, smem, s>>>(p);
+        kern<<<grid, dense && ff ? tc_threads<kFuseClasses>() : kThreads, smem, s>>>(p);
     };
     if (dense && ff) { if (three) go(k_tc_gemm<0, true, kFuseClasses>); else go(k_tc_gemm<0, false, kFuseClasses>); }
     else if (dense) { if (three) go(k_tc_gemm<0, true>); else go(k_tc_gemm<0, false>); }
