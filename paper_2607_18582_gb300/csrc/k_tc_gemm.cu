@@ -450,6 +450,62 @@ __device__ __forceinline__ void chunk_cursor(const TcParams &p, LoadRows &lr)
     lr.ky = t / p.kw;
 }
 
+// An entry of a row's overlay in a ring slot: the value at `src` for position pos of the K-step.
+__device__ __forceinline__ void ov_entry(const TcParams &p, int r, uint32_t ov, int &cnt, int pos, const float *src)
+{
+    if (cnt < kOvMax) {
+        cp_async4(ov + (uint32_t)(cnt * kTileM + r) * 4, src, 4);
+        asm volatile("st.shared.u8 [%0], %1;" ::"r"(ov + kTileM * kOvMax * 4 + cnt * kTileM + r), "r"(pos));
+    } else {
+        atomicExch(p.err, MURE_ERR_UNSUPPORTED);   // the host keeps the entry count in range
+    }
+    ++cnt;
+}
+
+__device__ __forceinline__ void ov_count(int r, uint32_t ov, int cnt)
+{
+    asm volatile("st.shared.u8 [%0], %1;" ::"r"(ov + kTileM * kOvMax * 5 + r), "r"(min(cnt, kOvMax)));
+}
+
+// A dense row's overlay entries of K-step k0 .. k0+31: positions are c * ch + j (cell c of
+// mutated channel j); the K-steps of a row come in ascending k, so each slot keeps a cursor.
+// entry(position in the K-step, index into the row's patch); returns their number.
+template <class F>
+__device__ __forceinline__ int dense_overlay(const TcParams &p, RowInfo &pf, int k0, F &&entry)
+{
+    int cnt = 0;
+    const int nq = min(pf.ov_k, 4);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (q >= nq) break;
+        while (pf.ov_c[q] < p.ov.cells && pf.ov_pos[q] < k0 + kTileK) {
+            if (pf.ov_pos[q] < k0) {   // (of a K-step that the other set takes)
+                pf.ov_pos[q] += p.ov.ch;
+                ++pf.ov_c[q];
+                continue;
+            }
+            entry(pf.ov_pos[q] - k0, q * p.ov.cells + pf.ov_c[q]);
+            ++cnt;
+            pf.ov_pos[q] += p.ov.ch;
+            ++pf.ov_c[q];
+        }
+    }
+    return cnt;
+}
+
+// The row's overlay entries of a K-step, written over its landed values.
+__device__ __forceinline__ void overlay_apply(uint32_t slot, uint32_t ov, int r)
+{
+    uint32_t n;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(n) : "r"(ov + kTileM * kOvMax * 5 + r));
+    for (uint32_t e = 0; e < n; ++e) {
+        uint32_t pos, val;
+        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(pos) : "r"(ov + kTileM * kOvMax * 4 + e * kTileM + r));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(val) : "r"(ov + (e * kTileM + r) * 4));
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(slot + sw128_off(r, pos >> 2) + 4 * (pos & 3)), "r"(val) : "memory");
+    }
+}
+
 // Queue the cp.async copies of K-step k0 .. k0+31 of the warp's 32 GEMM rows into
 // their 128-byte rows of `slot` (swizzled like the MMA operand layout, so that each
 // thread's read-back of its own row is free of bank conflicts).  Values past the
@@ -464,15 +520,7 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
     const float *dummy = p.b;   // a valid address for zero-byte copies
     const int lane = r & 31, wbase = r & ~31, ch = lane & 7;
     int cnt = 0;
-    auto entry = [&](int pos, const float *src) {
-        if (cnt < kOvMax) {
-            cp_async4(ov + (uint32_t)(cnt * kTileM + r) * 4, src, 4);
-            asm volatile("st.shared.u8 [%0], %1;" ::"r"(ov + kTileM * kOvMax * 4 + cnt * kTileM + r), "r"(pos));
-        } else {
-            atomicExch(p.err, MURE_ERR_UNSUPPORTED);   // the host keeps the entry count in range
-        }
-        ++cnt;
-    };
+    auto entry = [&](int pos, const float *src) { ov_entry(p, r, ov, cnt, pos, src); };
     if (DENSE) {
         const int kk = k0 + 4 * ch;
         const int nbk = max(0, min(16, (p.K - kk) * 4));
@@ -482,18 +530,7 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
             const int nb = lr.xrow[c] ? nbk : 0;
             cp_async16(slot + sw128_off(row, ch), nb ? (const void *)(lr.xrow[c] + kk) : (const void *)dummy, nb);
         }
-        // overlay positions are c * ch + j (cell c of mutated channel j); the K-steps of a
-        // row come in ascending k, so each slot keeps a cursor
-        const int nq = min(pf.ov_k, 4);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            if (q >= nq) break;
-            while (pf.ov_c[q] < p.ov.cells && pf.ov_pos[q] < k0 + kTileK) {
-                entry(pf.ov_pos[q] - k0, pf.ov_patch + q * p.ov.cells + pf.ov_c[q]);
-                pf.ov_pos[q] += p.ov.ch;
-                ++pf.ov_c[q];
-            }
-        }
+        dense_overlay(p, pf, k0, [&](int pos, int at) { entry(pos, pf.ov_patch + at); });
     } else if ((p.ic & 3) == 0) {
         // 16-byte chunks: 4 channels of one input pixel; this lane's chunk has the same
         // (ky, kx, ci) in all its rows
@@ -545,7 +582,7 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
             if (++ci == p.ic) { ci = 0; if (++kx == p.kw) { kx = 0; ++ky; } }
         }
     }
-    if (p.ov.patch) asm volatile("st.shared.u8 [%0], %1;" ::"r"(ov + kTileM * kOvMax * 5 + r), "r"(min(cnt, kOvMax)));
+    if (p.ov.patch) ov_count(r, ov, cnt);
 }
 
 // The small-image convolution mode: 5x5 filters over a 14 x 14 x 6 map, stride 1, no
@@ -629,15 +666,21 @@ struct SmallSteps {
     }
 };
 
-// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; with the output layer in the
-// epilogue (FCP > 0) a second set of epilogue warps, since there the epilogue bounds the layer:
+// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; for dense layers another 4.
+// Without the output layer in the epilogue (FCP = 0) they are a second set of producers, which
+// take the K-steps in turn: a K-step's way through a producer (wait, read, split, store to tensor
+// memory) is a chain, and writing the overlay's values over the row makes it longer.  LeNet-5's
+// 400 -> 120 over 904,000 rows of cached inputs with 25 overlay values each: 510 us with rows and
+// values by cp.async, 445 with rows by tensor-map copies and values in registers, 318 with two
+// sets of producers (290, the memory bandwidth, for rows of their own without an overlay).
+// With the output layer (FCP > 0) they are a second set of epilogue warps, since there that bounds it:
 // a row costs F x 12 FMAs and as many weight words from shared memory.  LeNet-5's 120 -> 84 -> 10
 // over 904,000 rows: 275 us with one set that tested each input's index, 208 without the tests
 // (the weights' loads then run ahead of the sums), 162 with two sets.
-template <int FCP>
+template <int MODE, int FCP>
 constexpr int tc_threads()
 {
-    return FCP > 0 ? kThreads + 128 : kThreads;
+    return MODE == 0 ? kThreads + 128 : kThreads;
 }
 
 // MODE 0: dense layer (one GEMM row per batch row); 1: implicit-GEMM convolution; 2:
@@ -646,7 +689,7 @@ constexpr int tc_threads()
 // each row's outputs in the epilogue, followed by the kill epilogue, and the rows
 // themselves are not stored.
 template <int MODE, bool THREE, int FCP = 0>
-__global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_constant__ TcParams p)
+__global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __grid_constant__ TcParams p)
 {
     static_assert(FCP == 0 || (MODE == 0 && FCP % 4 == 0) || (MODE == 3 && FCP == -1),
                   "the output layer is fused into dense layers only; -1: the staged mode's slot GEMM with a residual add");
@@ -700,13 +743,13 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if constexpr (FCP > 0) {
-        for (int i = threadIdx.x; i < p.ff.F * FCP; i += tc_threads<FCP>()) {
+        for (int i = threadIdx.x; i < p.ff.F * FCP; i += tc_threads<MODE, FCP>()) {
             const int f = i / FCP, c = i % FCP;
             const float wv = c < p.ff.C ? p.ff.W[(int64_t)c * p.ff.F + f] : 0.f;
             asm volatile("st.shared.f32 [%0], %1;" ::"r"(fw_region + 4 * i), "f"(wv) : "memory");
         }
     }
-    for (int n = threadIdx.x; n < kSliceMax; n += tc_threads<FCP>()) {
+    for (int n = threadIdx.x; n < kSliceMax; n += tc_threads<MODE, FCP>()) {
         if (MODE == 2) bias_sh[n] = n < SmallConv::N ? p.b[n % SmallConv::OC] : 0.f;
         else bias_sh[n] = n_base + n < p.N ? p.b[n_base + n] : 0.f;
     }
@@ -803,11 +846,14 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
             bulk_g2s(ovst_region + (uint32_t)b * G2::OVST_B, p.ov.patch + (int64_t)row0 * p.ov.row_stride, pbytes, bar);
     };
 
-    if (warp < 4) {
+    constexpr bool kTwoProd = MODE == 0 && FCP == 0;   // warps 12-15: a second set of producers
+    if (warp < 4 || (kTwoProd && warp >= 12)) {
         // ------------------------------------------------------------ producers --
-        const int r = threadIdx.x;                        // GEMM row in the tile = TMEM lane
-        const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
-        int t = 0;
+        const int r = (warp & 3) * 32 + lane;             // GEMM row in the tile = TMEM lane
+        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+        // two sets of producers take the K-steps in turn (where the A tiles come by tensor-map copies)
+        const int sets = kTwoProd && p.a_tma ? 2 : 1, set = warp >= 12 ? 1 : 0;
+        int t = set;
         uint32_t wraps = 0;                               // completed rounds of the A-stage ring
         // split one K-step of this row into TF32 halves and hand it to the MMA warps
         auto push = [&](float (&hi)[kTileK]) -> bool {
@@ -827,7 +873,8 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bar_afull[t]));
-            if (++t == p.n_stages) { t = 0; ++wraps; }
+            t += sets;
+            if (t >= p.n_stages) { t -= p.n_stages; ++wraps; }   // (an even number of stages)
             return true;
         };
         // tile pairs: the K-step of row r (part 0), then of row 128 + r (part 1), into one
@@ -977,13 +1024,49 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
                 }
             }
         } else if (DENSE && p.a_tma) {
-            // A tiles land by tensor-map copies (warp 10); each thread reads its row
+            // A tiles land by tensor-map copies (warp 10); each thread reads its row.  With an
+            // overlay the thread holds its row's entries of the K-step in registers, loaded a
+            // K-step ahead, and writes them over the landed row.
             bool ok = true;
-            int slot_i = 0;
+            int slot_i = set;
             uint32_t slot_wraps = 0;
-            for (int64_t j = 0; ok && j < total; ++j) {
+            RowInfo pf{};
+            int64_t iss_i = 0, row_i = -1;   // tile and K-step of the next entries, tile of pf
+            int iss_kt = set, n_ov = 0;
+            uint32_t ov_at[kOvMax];   // patch index << 7 | byte in the row's line (swizzled)
+            float ov_val[kOvMax];
+            auto fetch_overlay = [&]() {
+                n_ov = 0;
+                while (iss_kt >= nK) { iss_kt -= nK; ++iss_i; }
+                if (iss_i >= my_tiles) return;
+                if (iss_i != row_i) {
+                    pf = row_info<true>(p, (blockIdx.x + iss_i * gridDim.x) * kTileM + r);
+                    row_i = iss_i;
+                }
+                n_ov = dense_overlay(p, pf, iss_kt * kTileK, [&](int pos, int at) {
+#pragma unroll
+                    for (int e = kOvMax - 1; e > 0; --e) ov_at[e] = ov_at[e - 1];
+                    ov_at[0] = (uint32_t)at << 7 | ((uint32_t)pos << 2 ^ (uint32_t)(r & 7) << 4);
+                });
+#pragma unroll
+                for (int e = 0; e < kOvMax; ++e) {
+                    if (e >= n_ov) break;
+                    ov_val[e] = __ldg(pf.ov_patch + (ov_at[e] >> 7));
+                }
+                iss_kt += sets;
+            };
+            if (p.ov.patch) fetch_overlay();
+            for (int64_t j = set; ok && j < total; j += sets) {
                 if (!warp_wait_phase<32>(smem_u32(&bar_alanded[slot_i]), slot_wraps & 1, abort_flag)) break;
                 const uint32_t slot = a_region + (uint32_t)slot_i * kStageA;
+                if (p.ov.patch) {
+#pragma unroll
+                    for (int e = 0; e < kOvMax; ++e) {
+                        if (e >= n_ov) break;
+                        asm volatile("st.shared.f32 [%0], %1;" ::"r"(slot + (uint32_t)r * 128 + (ov_at[e] & 127)), "f"(ov_val[e])
+                                     : "memory");
+                    }
+                }
                 float v[kTileK];
 #pragma unroll
                 for (int c = 0; c < kTileK / 4; ++c) {
@@ -991,12 +1074,18 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
                                  : "=f"(v[4 * c]), "=f"(v[4 * c + 1]), "=f"(v[4 * c + 2]), "=f"(v[4 * c + 3])
                                  : "r"(slot + sw128_off(r, c)));
                 }
+                if (p.ov.patch) {
+                    // the overlay's writes before the next copy into the slot (async proxy)
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    fetch_overlay();
+                }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&bar_afree[slot_i]));
-                if (++slot_i == kNA) { slot_i = 0; ++slot_wraps; }
+                slot_i += sets;
+                if (slot_i >= kNA) { slot_i -= kNA; ++slot_wraps; }   // (kNA is even)
                 ok = push(v);
             }
-        } else {
+        } else if (set == 0) {
             // issue cursor (tile i, K-tile kt, ring slot) runs kNA - 1 steps ahead
             RowInfo pf{};
             LoadRows lr{};
@@ -1025,20 +1114,7 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
                 cp_async_wait<kNA - 1>();                 // this thread's copies of step j
                 __syncwarp();                             // ... and those of the warp's other lanes
                 const uint32_t slot = a_region + (uint32_t)slot_i * kStageA;
-                if (p.ov.patch) {
-                    // the row's overlay entries of this K-step, written over the landed copy
-                    const uint32_t ov = ov_region + (uint32_t)slot_i * kOvSlotBytes;
-                    uint32_t n;
-                    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(n) : "r"(ov + kTileM * kOvMax * 5 + r));
-                    for (uint32_t e = 0; e < n; ++e) {
-                        uint32_t pos, val;
-                        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(pos) : "r"(ov + kTileM * kOvMax * 4 + e * kTileM + r));
-                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(val) : "r"(ov + (e * kTileM + r) * 4));
-                        asm volatile("st.shared.u32 [%0], %1;" ::"r"(slot + sw128_off(r, pos >> 2) + 4 * (pos & 3)),
-                                     "r"(val)
-                                     : "memory");
-                    }
-                }
+                if (p.ov.patch) overlay_apply(slot, ov_region + (uint32_t)slot_i * kOvSlotBytes, r);
                 if (++slot_i == kNA) slot_i = 0;
                 float v[kTileK];
 #pragma unroll
@@ -1381,20 +1457,32 @@ __global__ void __launch_bounds__(tc_threads<FCP>(), 1) k_tc_gemm(const __grid_c
             int slot_i = 0, kt = 0;
             uint32_t slot_wraps = 0;
             int64_t i = 0, j = 0;
+            int rows[2] = {0, 0};   // input rows of the tile's copies (with an overlay two of 64 rows)
             for (; j < total; ++j) {
                 if (slot_wraps >= 1 &&
                     !wait_phase<32>(smem_u32(&bar_afree[slot_i]), (slot_wraps - 1) & 1, abort_flag))
                     break;
                 // the producers' reads of the slot (generic proxy) before this copy's writes
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                const int64_t m0 = (blockIdx.x + i * gridDim.x) * kTileM;
-                const int row = (int)m0;
+                if (kt == 0) {
+                    const int64_t m0 = (blockIdx.x + i * gridDim.x) * kTileM;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int64_t m = m0 + 64 * h;
+                        // (rows past the end: past the tensor's end too, zero-filled)
+                        rows[h] = p.x_per_input ? (int)(p.t0 + (m < M ? m % p.T : p.T)) : (int)m;
+                    }
+                }
                 const uint32_t bar = smem_u32(&bar_alanded[slot_i]);
                 mbar_expect_tx(bar, (uint32_t)kStageA);
-                asm volatile(
-                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                    ::"r"(a_region + (uint32_t)slot_i * kStageA), "l"(tmap), "r"(kt * kTileK), "r"(row), "r"(bar)
-                    : "memory");
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (h == 0 || p.ov.patch)
+                        asm volatile(
+                            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                            ::"r"(a_region + (uint32_t)slot_i * kStageA + (uint32_t)h * (kStageA / 2)), "l"(tmap),
+                              "r"(kt * kTileK), "r"(rows[h]), "r"(bar)
+                            : "memory");
                 if (++slot_i == kNA) { slot_i = 0; ++slot_wraps; }
                 if (++kt == nK) { kt = 0; ++i; }
             }
@@ -2084,20 +2172,20 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 }
 
 // The A operand of a dense layer as a 2-D tensor [rows][K] with 128-byte swizzled
-// boxes of 128 rows x 32 values (the producers' shared-memory layout): false for
-// per-input rows, unaligned rows or without the encoder.
-static bool dense_a_tensor_map(const Stage &S, Src x, RowMap rm, CUtensorMap &map)
+// boxes of 128 (with an overlay 64) rows x 32 values (the producers' shared-memory layout):
+// false for a compacted batch's per-input rows, unaligned rows or without the encoder.
+static bool dense_a_tensor_map(const Stage &S, Src x, RowMap rm, bool overlay, CUtensorMap &map)
 {
-    // rows of per-input tensors always carry a patch (the first suffix stage), so only
-    // row-per-row tensors take this path
-    if (x.per_input) return false;
+    // rows of per-input tensors always carry a patch (the first suffix stage); with one the
+    // copies take 64 rows, which lie within a mutant's where its inputs are a multiple of 64
+    if (x.per_input && (!overlay || rm.lrow || rm.T % 64 != 0)) return false;
     if ((x.stride * 4) % 16 != 0 || (reinterpret_cast<uintptr_t>(x.p) & 15) != 0) return false;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return false;
     const float *base = x.p;
-    const cuuint64_t dims[2] = {(cuuint64_t)S.K, (cuuint64_t)rm.R};
+    const cuuint64_t dims[2] = {(cuuint64_t)S.K, (cuuint64_t)(x.per_input ? rm.t0 + rm.T : rm.R)};
     const cuuint64_t strides[1] = {(cuuint64_t)x.stride * 4};
-    const cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)kTileM};
+    const cuuint32_t box[2] = {(cuuint32_t)kTileK, (cuuint32_t)(overlay ? 64 : kTileM)};
     const cuuint32_t estr[2] = {1, 1};
     return enc(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -2261,8 +2349,8 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     // the delta GEMM: one issuing warp (or two in turn, which is the same sum), so that a
     // column's sum never depends on how many slots share its batch
     if (ss && !p.mma_chain) p.n_mma = p.n_part = 1;
-    // dense rows without an overlay: A tiles by tensor-map copies from warp 10
-    p.a_tma = dense && !p.ov.patch && p.n_mma <= 2 && dense_a_tensor_map(S, x, rm, p.tmap_a) ? 1 : 0;
+    // dense rows: A tiles by tensor-map copies from warp 10
+    p.a_tma = dense && p.n_mma <= 2 && dense_a_tensor_map(S, x, rm, p.ov.patch != nullptr, p.tmap_a) ? 1 : 0;
     if (S.tc_small || S.tc_conv) {
         // warp 10 stages maps in those modes
         p.n_mma = std::min(p.n_mma, 2);
@@ -2291,7 +2379,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, dense && ff ? tc_threads<kFuseClasses>() : kThreads, smem, s>>>(p);
+        kern<<<grid, dense ? tc_threads<0, 0>() : kThreads, smem, s>>>(p);
     };
     if (dense && ff) { if (three) go(k_tc_gemm<0, true, kFuseClasses>); else go(k_tc_gemm<0, false, kFuseClasses>); }
     else if (dense) { if (three) go(k_tc_gemm<0, true>); else go(k_tc_gemm<0, false>); }

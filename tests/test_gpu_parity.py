@@ -186,6 +186,26 @@ def test_expansion_at_fan_in_edges(M, ctx, oracle_mod, fan):
             assert (got != exp).mean() <= 1e-3 and np.allclose(got, exp, rtol=2.0 ** -23, atol=0)
 
 
+@pytest.mark.parametrize("n_in", [64, 65])
+@pytest.mark.parametrize("widths", [(50, 20, 32, 10), (50, 64, 48, 10), (50, 97, 129, 40, 12), (30, 130, 16, 13), (9, 300, 84, 2)])
+def test_dense_overlay_at_step_edges(M, ctx, oracle_mod, widths, n_in):
+    """Dense layers whose first rows are cached inputs with the mutated neurons' values written in:
+    one K-step to ten (the two sets of producers in turn), tiles of two mutants (64 inputs), one to
+    four neurons per mutant, the output layer fused and not: the oracle's logits, and the bits of
+    vanilla, whose rows are its own."""
+    model = wl.mlp(5, widths)
+    X = wl.inputs(model, n_in, 7)
+    table = wl.concat([wl.mutants(model, 14, seed=50 + l, ratios=(k / widths[l + 1],), ops=("GF", "NEB", "NAI"), layers=[l])
+                       for l in range(model.n_layers()) for k in (1, 3, 4)])
+    ora = oracle_mod.vanilla(model, X, table)
+    m = M.mure_model_load(ctx, model)
+    r = M.mure_eval_mutants(M.mure_build_prefix_cache(m, X), table, logits=True)
+    ok, worst = logits_close(r["logits"], ora["logits"])
+    assert ok, worst
+    v = M.mure_eval_vanilla(m, X, table, logits=True)
+    assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
 @pytest.mark.parametrize("prec", PRECISIONS)
 def test_batch_invariance(M, ctx, prec):
     """Tiny workspaces force many batches (input tiles, mutant chunks): results are
