@@ -718,10 +718,13 @@ int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const P
 }
 
 // Materialise rows: out = base with the overlay's channels written in (for suffix kernels
-// that read plain rows), TPR threads per row (a warp, or the whole block for rows above 2 KB):
-// 16-byte copies through shared memory, the patch written there in between (one element per
-// thread and index division, it took 507 us for 140,800 rows of LeNet's 14 x 14 x 6 maps, now
-// 311).
+// that read plain rows), TPR threads per row: a warp, or the whole block where eight rows don't
+// fit 48 KiB.  16-byte copies through shared memory, the patch written there in between.  A row
+// waits on a chain of loads (its mutant's neurons, then the patch), so what counts is rows in
+// flight and that the chain starts with the copy and all lanes follow it at once.  140,800 rows
+// of LeNet's 14 x 14 x 6 maps: one element per thread and index division 507 us, a block per row
+// 311, now 164 (97 the writes); 279,000 rows of 120 values, a channel at a time per row 123 us,
+// now 63.
 template <int TPR>
 __global__ void __launch_bounds__(256) k_rows_overlay(const float *__restrict__ base, int64_t base_stride,
                                                       int base_per_input, int64_t t0, int T, int R, int n4,
@@ -734,23 +737,29 @@ __global__ void __launch_bounds__(256) k_rows_overlay(const float *__restrict__ 
     float *row = sm + (threadIdx.x / TPR) * 4 * n4;
     const bool ok = r < R;
     const int64_t lr = ok ? logical_row(lrow, r) : 0;
+    const uint32_t g = (uint32_t)lr / (uint32_t)T;   // (a batch's rows are below 2^31)
+    const int n = ok ? __ldg(ov.n_neurons + g) : 0;
+    const int32_t *ids = ov.ids + (ok ? __ldg(ov.neuron_off + g) : 0);
     auto sync = [] {
         if (TPR == 32) __syncwarp();
         else __syncthreads();
     };
     if (ok) {
-        const float4 *src = reinterpret_cast<const float4 *>(base + (base_per_input ? t0 + lr % T : r) * base_stride);
+        const float4 *src =
+            reinterpret_cast<const float4 *>(base + (base_per_input ? t0 + (lr - (int64_t)g * T) : r) * base_stride);
 #pragma unroll 4
         for (int i = tid; i < n4; i += TPR) reinterpret_cast<float4 *>(row)[i] = __ldg(src + i);
     }
     sync();
     if (ok) {
-        const int g = (int)(lr / T), n = ov.n_neurons[g];
-        const int32_t *ids = ov.ids + ov.neuron_off[g];
+        // every lane takes values of every mutated channel: value i is cell i mod cells of channel
+        // i / cells
         const float *patch = ov.patch + lr * ov.row_stride;
-        for (int q = 0; q < n; ++q) {
-            const int j = ids[q];
-            for (int c = tid; c < ov.cells; c += TPR) row[c * ov.ch + j] = __ldg(patch + q * ov.cells + c);
+        const uint32_t cells = (uint32_t)ov.cells;
+#pragma unroll 2
+        for (uint32_t i = tid; i < n * cells; i += TPR) {
+            const uint32_t q = i / cells;
+            row[(i - q * cells) * ov.ch + __ldg(ids + q)] = __ldg(patch + i);
         }
     }
     sync();
@@ -811,7 +820,7 @@ int launch_rows_overlay(Src base, int64_t n_floats, RowMap rm, const Overlay &ov
         return launches;
     }
     const int n4 = (int)((n_floats + 3) / 4);   // rows are whole 16-byte pieces
-    const int per_block = n4 <= 128 ? 8 : 1;
+    const int per_block = n4 <= 384 ? 8 : 1;    // (8 rows in 48 KiB)
     const size_t smem = (size_t)per_block * n4 * 16;
     const unsigned blocks = (unsigned)((rm.R + per_block - 1) / per_block);
     if (per_block == 8)
