@@ -335,6 +335,8 @@ struct TcParams {
     // dense layers: A tiles (128 rows x one K-step) by tensor-map copies from warp 10
     // instead of the producers' 16-byte copies; tile m0 starts at row coordinate m0
     int a_tma;
+    // convolutions: 16-byte gathers (channels a multiple of 4; output positions in 16 bits each)
+    int gather16;
     CUtensorMap tmap_a;
     // MODE 3 (staged convolution): each tile's input rows with their zero border, 32
     // channels at a time, land by tensor-map copies in a ring of cv_nbuf buffers; the
@@ -359,7 +361,7 @@ constexpr uint32_t kOvSlotBytes = kTileM * (kOvMax * 4 + kOvMax + 4);   // value
 struct RowInfo {
     int64_t row;
     int oy, ox, py, px;
-    const float *xrow;
+    int xidx;                 // the input row: a row of p.x
     int ov_k;
     const int32_t *ov_ids;
     const float *ov_patch;
@@ -396,7 +398,7 @@ __device__ __forceinline__ RowInfo row_info(const TcParams &p, int64_t m)
     // per-input sources, the overlay and its group by the logical row; the batch's own
     // row buffers by the physical row
     const int64_t lr = logical_row(p.lrow, ri.row);
-    ri.xrow = p.x + (p.x_per_input ? p.t0 + lr % p.T : ri.row) * p.x_stride;
+    ri.xidx = (int)(p.x_per_input ? p.t0 + lr % p.T : ri.row);
     if (OVERLAY && p.ov.patch) {
         const int g = (int)(lr / p.T);
         ri.ov_k = p.ov.n_neurons[g];
@@ -418,8 +420,8 @@ __device__ __forceinline__ RowInfo row_info(const TcParams &p, int64_t m)
 // instruction covers four whole 128-byte row segments (a thread copying its own row
 // would touch 32 rows per instruction and saturate the load/store unit).
 struct LoadRows {
-    const float *xrow[8];   // null: row past the end
-    int oy[8], ox[8];
+    int row[8];             // row of p.x; -1: past the end
+    int oyx[8];             // convolution: output position, oy << 16 | ox
     int ci, kx, ky;         // convolution: (ky, kx, ci) of this lane's 4-value chunk at the next K-step
 };
 
@@ -430,20 +432,15 @@ __device__ __forceinline__ void load_rows(const RowInfo &pf, LoadRows &lr)
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const int src = 4 * c + (lane >> 3);
-        const unsigned long long xp =
-            __shfl_sync(0xffffffffu, (unsigned long long)(uintptr_t)(pf.ok ? pf.xrow : nullptr), src);
-        lr.xrow[c] = reinterpret_cast<const float *>((uintptr_t)xp);
-        if (!DENSE) {
-            lr.oy[c] = __shfl_sync(0xffffffffu, pf.oy, src);
-            lr.ox[c] = __shfl_sync(0xffffffffu, pf.ox, src);
-        }
+        lr.row[c] = __shfl_sync(0xffffffffu, pf.ok ? pf.xidx : -1, src);
+        if (!DENSE) lr.oyx[c] = __shfl_sync(0xffffffffu, pf.oy << 16 | pf.ox, src);
     }
 }
 
-// The chunk cursor of a convolution's first K-step: k = 4 * (lane mod 8).
-__device__ __forceinline__ void chunk_cursor(const TcParams &p, LoadRows &lr)
+// The chunk cursor of a convolution's K-step kt: k = 32 kt + 4 * (lane mod 8).
+__device__ __forceinline__ void chunk_cursor(const TcParams &p, LoadRows &lr, int kt)
 {
-    const int kk = 4 * ((threadIdx.x & 31) & 7);
+    const int kk = kTileK * kt + 4 * ((threadIdx.x & 31) & 7);
     const int t = kk / p.ic;
     lr.ci = kk - t * p.ic;
     lr.kx = t % p.kw;
@@ -515,7 +512,7 @@ __device__ __forceinline__ void overlay_apply(uint32_t slot, uint32_t ov, int r)
 // the copies have landed.
 template <bool DENSE>
 __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, LoadRows &lr, int r, uint32_t slot,
-                                              uint32_t ov, int k0)
+                                              uint32_t ov, int k0, int sets)
 {
     const float *dummy = p.b;   // a valid address for zero-byte copies
     const int lane = r & 31, wbase = r & ~31, ch = lane & 7;
@@ -527,17 +524,17 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int row = wbase + 4 * c + (lane >> 3);
-            const int nb = lr.xrow[c] ? nbk : 0;
-            cp_async16(slot + sw128_off(row, ch), nb ? (const void *)(lr.xrow[c] + kk) : (const void *)dummy, nb);
+            const int nb = lr.row[c] >= 0 ? nbk : 0;
+            cp_async16(slot + sw128_off(row, ch), nb ? (const void *)(p.x + lr.row[c] * p.x_stride + kk) : (const void *)dummy, nb);
         }
         dense_overlay(p, pf, k0, [&](int pos, int at) { entry(pos, pf.ov_patch + at); });
-    } else if ((p.ic & 3) == 0) {
+    } else if (p.gather16) {
         // 16-byte chunks: 4 channels of one input pixel; this lane's chunk has the same
         // (ky, kx, ci) in all its rows
         const int kk = k0 + 4 * ch;
         const int ci = lr.ci, kx = lr.kx, ky = lr.ky;
         // the cursor of the next K-step, 32 values on (no divisions per K-step)
-        lr.ci += kTileK;
+        lr.ci += kTileK * sets;
         while (lr.ci >= p.ic) {
             lr.ci -= p.ic;
             if (++lr.kx == p.kw) { lr.kx = 0; ++lr.ky; }
@@ -545,9 +542,9 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int row = wbase + 4 * c + (lane >> 3);
-            const int iy = lr.oy[c] * p.stride - p.pad + ky, ix = lr.ox[c] * p.stride - p.pad + kx;
-            const bool in = lr.xrow[c] && kk < p.K && (unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw;
-            cp_async16(slot + sw128_off(row, ch), in ? lr.xrow[c] + ((int64_t)iy * p.iw + ix) * p.ic + ci : dummy,
+            const int iy = (lr.oyx[c] >> 16) * p.stride - p.pad + ky, ix = (lr.oyx[c] & 0xffff) * p.stride - p.pad + kx;
+            const bool in = lr.row[c] >= 0 && kk < p.K && (unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw;
+            cp_async16(slot + sw128_off(row, ch), in ? p.x + lr.row[c] * p.x_stride + (iy * p.iw + ix) * p.ic + ci : dummy,
                        in ? 16 : 0);
         }
         if (pf.ov_k > 0) {
@@ -567,14 +564,14 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
             }
         }
     } else {
-        // channel counts that are not a multiple of 4: 4-byte copies of the thread's own
+        // other channel counts: 4-byte copies of the thread's own
         // row, the patch value taken directly for a mutated channel
         int ci = k0 % p.ic, t = k0 / p.ic, kx = t % p.kw, ky = t / p.kw;
         for (int i = 0; i < kTileK; ++i) {
             const int k = k0 + i;
             const int iy = pf.oy * p.stride - p.pad + ky, ix = pf.ox * p.stride - p.pad + kx;
             const bool in = pf.ok && k < p.K && (unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw;
-            const float *src = in ? pf.xrow + ((int64_t)iy * p.iw + ix) * p.ic + ci : dummy;
+            const float *src = in ? p.x + pf.xidx * p.x_stride + ((int64_t)iy * p.iw + ix) * p.ic + ci : dummy;
             if (in)
                 for (int q = 0; q < pf.ov_k; ++q)
                     if (pf.ov_ids[q] == ci) src = pf.ov_patch + q * p.ov.cells + iy * p.iw + ix;
@@ -666,13 +663,17 @@ struct SmallSteps {
     }
 };
 
-// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; for dense layers another 4.
+// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; for dense layers and gathered
+// convolutions (MODE 1) another 4.
 // Without the output layer in the epilogue (FCP = 0) they are a second set of producers, which
 // take the K-steps in turn: a K-step's way through a producer (wait, read, split, store to tensor
 // memory) is a chain, and writing the overlay's values over the row makes it longer.  LeNet-5's
 // 400 -> 120 over 904,000 rows of cached inputs with 25 overlay values each: 510 us with rows and
 // values by cp.async, 445 with rows by tensor-map copies and values in registers, 318 with two
 // sets of producers (290, the memory bandwidth, for rows of their own without an overlay).
+// Gathered convolutions: ResNet-10's 54 launches of a screen 2.27 -> 1.98 ms, ResNet-20's 25 of a
+// job 1.94 -> 1.66 (each set's copies then run one of its own K-steps ahead, as far as three in
+// turn before).  The staged modes were measured with two sets too, and were no faster.
 // With the output layer (FCP > 0) they are a second set of epilogue warps, since there that bounds it:
 // a row costs F x 12 FMAs and as many weight words from shared memory.  LeNet-5's 120 -> 84 -> 10
 // over 904,000 rows: 275 us with one set that tested each input's index, 208 without the tests
@@ -680,7 +681,7 @@ struct SmallSteps {
 template <int MODE, int FCP>
 constexpr int tc_threads()
 {
-    return MODE == 0 ? kThreads + 128 : kThreads;
+    return MODE <= 1 ? kThreads + 128 : kThreads;
 }
 
 // MODE 0: dense layer (one GEMM row per batch row); 1: implicit-GEMM convolution; 2:
@@ -846,13 +847,13 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             bulk_g2s(ovst_region + (uint32_t)b * G2::OVST_B, p.ov.patch + (int64_t)row0 * p.ov.row_stride, pbytes, bar);
     };
 
-    constexpr bool kTwoProd = MODE == 0 && FCP == 0;   // warps 12-15: a second set of producers
+    constexpr bool kTwoProd = (MODE == 0 && FCP == 0) || MODE == 1;   // warps 12-15: a second set of producers
     if (warp < 4 || (kTwoProd && warp >= 12)) {
         // ------------------------------------------------------------ producers --
         const int r = (warp & 3) * 32 + lane;             // GEMM row in the tile = TMEM lane
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         // two sets of producers take the K-steps in turn (where the A tiles come by tensor-map copies)
-        const int sets = kTwoProd && p.a_tma ? 2 : 1, set = warp >= 12 ? 1 : 0;
+        const int sets = kTwoProd && (MODE == 1 || p.a_tma) ? 2 : 1, set = warp >= 12 ? 1 : 0;
         int t = set;
         uint32_t wraps = 0;                               // completed rounds of the A-stage ring
         // split one K-step of this row into TF32 halves and hand it to the MMA warps
@@ -1085,37 +1086,43 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
                 if (slot_i >= kNA) { slot_i -= kNA; ++slot_wraps; }   // (kNA is even)
                 ok = push(v);
             }
-        } else if (set == 0) {
-            // issue cursor (tile i, K-tile kt, ring slot) runs kNA - 1 steps ahead
+        } else if (MODE == 1 || set == 0) {
+            // issue cursor (tile i, K-tile kt, ring slot) runs kAhead of the set's steps ahead
+            constexpr int kAhead = MODE == 1 ? kNA / 2 - 1 : kNA - 1;
             RowInfo pf{};
             LoadRows lr{};
-            int64_t iss_i = 0, issued = 0;
-            int iss_kt = 0, iss_slot = 0;
+            const int n_steps = (int)total;
+            int iss_i = 0, issued = set, iss_kt = set, iss_slot = set;
+            bool fresh = true;   // the next K-step is the set's first of a tile
             auto issue_next = [&]() {
-                if (iss_kt == 0) {
+                while (iss_kt >= nK) { iss_kt -= nK; ++iss_i; fresh = true; }
+                if (fresh) {
+                    fresh = false;
                     pf = row_info<DENSE>(p, (blockIdx.x + iss_i * gridDim.x) * kTileM + r);
-                    if (DENSE || (p.ic & 3) == 0) load_rows<DENSE>(pf, lr);
-                    if (!DENSE && (p.ic & 3) == 0) chunk_cursor(p, lr);
+                    if (DENSE || p.gather16) load_rows<DENSE>(pf, lr);
+                    if (!DENSE && p.gather16) chunk_cursor(p, lr, iss_kt);
                 }
                 produce_issue<DENSE>(p, pf, lr, r, a_region + (uint32_t)iss_slot * kStageA,
-                                     ov_region + (uint32_t)iss_slot * kOvSlotBytes, iss_kt * kTileK);
-                if (++iss_kt == nK) { iss_kt = 0; ++iss_i; }
-                if (++iss_slot == kNA) iss_slot = 0;
-                ++issued;
+                                     ov_region + (uint32_t)iss_slot * kOvSlotBytes, iss_kt * kTileK, sets);
+                iss_kt += sets;
+                iss_slot += sets;
+                if (iss_slot >= kNA) iss_slot -= kNA;
+                issued += sets;
             };
-            for (int s0 = 0; s0 < kNA - 1; ++s0) {
-                if (issued < total) issue_next();
+            for (int s0 = 0; s0 < kAhead; ++s0) {
+                if (issued < n_steps) issue_next();
                 cp_async_commit();
             }
-            int slot_i = 0;
-            for (int64_t j = 0; j < total; ++j) {
-                if (issued < total) issue_next();
+            int slot_i = set;
+            for (int j = set; j < n_steps; j += sets) {
+                if (issued < n_steps) issue_next();
                 cp_async_commit();
-                cp_async_wait<kNA - 1>();                 // this thread's copies of step j
+                cp_async_wait<kAhead>();                 // this thread's copies of step j
                 __syncwarp();                             // ... and those of the warp's other lanes
                 const uint32_t slot = a_region + (uint32_t)slot_i * kStageA;
                 if (p.ov.patch) overlay_apply(slot, ov_region + (uint32_t)slot_i * kOvSlotBytes, r);
-                if (++slot_i == kNA) slot_i = 0;
+                slot_i += sets;
+                if (slot_i >= kNA) slot_i -= kNA;
                 float v[kTileK];
 #pragma unroll
                 for (int c = 0; c < kTileK / 4; ++c) {
@@ -1253,6 +1260,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             // unpooled outputs go through shared memory: one store instruction then
             // covers 4 rows x 128 bytes instead of 32 rows x 16 bytes
             float *stage = epi_stage[qd];
+            const bool staged = !((!DENSE && p.pool) || FCP > 0 || p.slot.out);
             const bool vec = DENSE || (p.N & 3) == 0;
             // a dense layer's pre-activations (z) go the same way: they are staged, and the
             // activation is applied to what is read back (a store per thread and value took
@@ -1266,11 +1274,10 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             for (int c = 0; c < (FCP > 0 ? FCP : 1); ++c) facc[c] = 0.f;
             for (int n0 = 0; n0 < Nt; n0 += 32) {
                 const int nc = min(32, Nt - n0);
-                float v[32];
 #pragma unroll
                 for (int h = 0; h < 32; h += 16) {
                     if (h >= nc) break;
-                    float *vh = v + h;
+                    float vh[16];
                     // the accumulator: the n_part partials added in a fixed order
                     const uint32_t acc = tmem + lane_off + abase + n0 + h;
                     tmem_ld16(acc, vh);
@@ -1415,12 +1422,14 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
                             }
                         }
                     }
-                }
-                if ((!DENSE && p.pool) || FCP > 0 || p.slot.out) continue;
+                    if (staged) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<float4 *>(stage + lane * kEpiStride + 4 * c) =
-                        make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                        for (int c = 0; c < 4; ++c)
+                            *reinterpret_cast<float4 *>(stage + lane * kEpiStride + h + 4 * c) =
+                                make_float4(vh[4 * c], vh[4 * c + 1], vh[4 * c + 2], vh[4 * c + 3]);
+                    }
+                }
+                if (!staged) continue;
                 __syncwarp();
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
@@ -2369,6 +2378,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     if (ss && !p.mma_chain) p.n_mma = p.n_part = 1;
     // dense rows: A tiles by tensor-map copies from warp 10
     p.a_tma = dense && p.n_mma <= 2 && dense_a_tensor_map(S, x, rm, p.ov.patch != nullptr, p.tmap_a) ? 1 : 0;
+    p.gather16 = (S.ic & 3) == 0 && S.oh < 32768 && S.ow < 32768;
     if (S.tc_small || S.tc_conv) {
         // warp 10 stages maps in those modes
         p.n_mma = std::min(p.n_mma, 2);
@@ -2397,7 +2407,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, dense ? tc_threads<0, 0>() : kThreads, smem, s>>>(p);
+        kern<<<grid, S.tc_small || S.tc_conv ? kThreads : tc_threads<0, 0>(), smem, s>>>(p);
     };
     if (dense && ff) { if (three) go(k_tc_gemm<0, true, kFuseClasses>); else go(k_tc_gemm<0, false, kFuseClasses>); }
     else if (dense) { if (three) go(k_tc_gemm<0, true>); else go(k_tc_gemm<0, false>); }

@@ -206,6 +206,27 @@ def test_dense_overlay_at_step_edges(M, ctx, oracle_mod, widths, n_in):
     assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
 
 
+@pytest.mark.parametrize("ic,k", [(16, 1), (16, 3), (20, 1), (20, 3), (18, 3), (33, 2)])
+def test_gathered_convolutions_at_step_edges(M, ctx, oracle_mod, ic, k):
+    """Stride-2 convolutions (rows gathered per tap, two sets of producers in turn): one K-step to
+    ten, odd counts, 16- and 4-byte gathers, tiles that end inside a mutant's rows: the oracle's
+    logits and the bits of vanilla."""
+    b = wl._Builder("gathered", (11, 9, 3), 5, 17)
+    x = b.conv(-1, ic, 3, pad=1)
+    y = b.gap(b.conv(b.conv(x, 24, k, stride=2, pad=k // 2), 17, 3, stride=2, pad=1))
+    b.dense(y, 5, act="none")
+    X = wl.inputs(b.m, 65, 3)
+    table = wl.concat([wl.mutants(b.m, 9, seed=60 + l, ratios=(0.1,), ops=("GF", "NEB", "NAI"), layers=[l])
+                       for l in range(b.m.n_layers())])
+    ora = oracle_mod.vanilla(b.m, X, table)
+    m = M.mure_model_load(ctx, b.m)
+    r = M.mure_eval_mutants(M.mure_build_prefix_cache(m, X), table, logits=True)
+    ok, worst = logits_close(r["logits"], ora["logits"])
+    assert ok, worst
+    v = M.mure_eval_vanilla(m, X, table, logits=True)
+    assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
 @pytest.mark.parametrize("prec", PRECISIONS)
 def test_batch_invariance(M, ctx, prec):
     """Tiny workspaces force many batches (input tiles, mutant chunks): results are
