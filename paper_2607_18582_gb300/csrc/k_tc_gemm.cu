@@ -8,10 +8,10 @@
 // output channels (a CTA takes a slice of <= 128).  A convolution is an implicit
 // GEMM: the producers gather the im2col rows from the NHWC input.  The CTA is
 // persistent (one per SM) and warp-specialised:
-//   warps 0-3  producers: thread = GEMM row = tensor-memory lane.  Each streams its
-//              row's 32-value K-steps into a private shared-memory ring with
-//              cp.async, several steps ahead (the first suffix stage's mutated
-//              channels are fetched from the patch buffer instead of the cached row),
+//   warps 0-3  producers (and 12-15, in turn): thread = GEMM row = tensor-memory lane.
+//              Each streams its row's 32-value K-steps into a private shared-memory
+//              ring with cp.async, or reads what tensor-map copies have landed (the
+//              first suffix stage's mutated channels come from the patch buffer),
 //              splits them into TF32 halves and stores the halves into a tensor-memory
 //              A stage (tcgen05.st); the MMA reads A from tensor memory, so the
 //              operand never goes through shared memory a second time;
@@ -663,8 +663,8 @@ struct SmallSteps {
     }
 };
 
-// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; for dense layers and gathered
-// convolutions (MODE 1) another 4.
+// Threads: 4 producer, 4 epilogue, 3 MMA and the weight warps; but for the small-image mode
+// another 4.
 // Without the output layer in the epilogue (FCP = 0) they are a second set of producers, which
 // take the K-steps in turn: a K-step's way through a producer (wait, read, split, store to tensor
 // memory) is a chain, and writing the overlay's values over the row makes it longer.  LeNet-5's
@@ -673,7 +673,8 @@ struct SmallSteps {
 // sets of producers (290, the memory bandwidth, for rows of their own without an overlay).
 // Gathered convolutions: ResNet-10's 54 launches of a screen 2.27 -> 1.98 ms, ResNet-20's 25 of a
 // job 1.94 -> 1.66 (each set's copies then run one of its own K-steps ahead, as far as three in
-// turn before).  The staged modes were measured with two sets too, and were no faster.
+// turn before).  Staged convolutions, which wait on the MMA warps more: VGG's 95 launches of a job
+// 118.3 -> 117.5 ms, ResNet-10's 17 of a screen 1.00 -> 0.96.  The small-image mode was no faster.
 // With the output layer (FCP > 0) they are a second set of epilogue warps, since there that bounds it:
 // a row costs F x 12 FMAs and as many weight words from shared memory.  LeNet-5's 120 -> 84 -> 10
 // over 904,000 rows: 275 us with one set that tested each input's index, 208 without the tests
@@ -681,7 +682,7 @@ struct SmallSteps {
 template <int MODE, int FCP>
 constexpr int tc_threads()
 {
-    return MODE <= 1 ? kThreads + 128 : kThreads;
+    return MODE != 2 ? kThreads + 128 : kThreads;
 }
 
 // MODE 0: dense layer (one GEMM row per batch row); 1: implicit-GEMM convolution; 2:
@@ -774,7 +775,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
     }
     if (threadIdx.x == 32) {
         for (int s = 0; s < kNT; ++s) {
-            mbar_init(smem_u32(&bar_afull[s]), 4);
+            mbar_init(smem_u32(&bar_afull[s]), pair ? 8 : 4);      // the producer warps of a K-step
             // each K-step has one issuing warp (two with tile pairs, one per tile)
             mbar_init(smem_u32(&bar_aempty[s]), pair ? 2 : 1);
         }
@@ -794,7 +795,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
         for (int s = 0; s < kNBufMax; ++s) {
             mbar_init(smem_u32(&bar_landed[s]), 1);
             mbar_init(smem_u32(&bar_ready[s]), 1);
-            mbar_init(smem_u32(&bar_released[s]), 4);
+            mbar_init(smem_u32(&bar_released[s]), MODE == 3 ? 8 : 4);   // every producer warp
         }
         abort_sh.abort = 0;
         mbar_init(smem_u32(&bar_turn[0]), 1);
@@ -847,14 +848,15 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             bulk_g2s(ovst_region + (uint32_t)b * G2::OVST_B, p.ov.patch + (int64_t)row0 * p.ov.row_stride, pbytes, bar);
     };
 
-    constexpr bool kTwoProd = (MODE == 0 && FCP == 0) || MODE == 1;   // warps 12-15: a second set of producers
+    constexpr bool kTwoProd = MODE != 2 && FCP <= 0;   // warps 12-15: a second set of producers
     if (warp < 4 || (kTwoProd && warp >= 12)) {
         // ------------------------------------------------------------ producers --
         const int r = (warp & 3) * 32 + lane;             // GEMM row in the tile = TMEM lane
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         // two sets of producers take the K-steps in turn (where the A tiles come by tensor-map copies)
-        const int sets = kTwoProd && (MODE == 1 || p.a_tma) ? 2 : 1, set = warp >= 12 ? 1 : 0;
-        int t = set;
+        // (with tile pairs each takes its tile's rows of every K-step)
+        const int sets = kTwoProd && !pair && (!DENSE || p.a_tma) ? 2 : 1, set = warp >= 12 ? 1 : 0;
+        int t = pair ? 0 : set;
         uint32_t wraps = 0;                               // completed rounds of the A-stage ring
         // split one K-step of this row into TF32 halves and hand it to the MMA warps
         auto push = [&](float (&hi)[kTileK]) -> bool {
@@ -867,7 +869,8 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             }
             if (wraps >= 1 && !warp_wait_phase<32>(smem_u32(&bar_aempty[t]), (wraps - 1) & 1, abort_flag)) return false;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t ta = tmem + lane_off + p.a_col + t * kAColsPerStage;
+            // (tile pairs: a stage holds the K-step of both tiles)
+            const uint32_t ta = tmem + lane_off + p.a_col + (uint32_t)(pair ? 2 * t + set : t) * kAColsPerStage;
             tmem_st32(ta, hi);
             if (THREE) tmem_st32(ta + 32, lo);
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -876,33 +879,6 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             if (lane == 0) mbar_arrive(smem_u32(&bar_afull[t]));
             t += sets;
             if (t >= p.n_stages) { t -= p.n_stages; ++wraps; }   // (an even number of stages)
-            return true;
-        };
-        // tile pairs: the K-step of row r (part 0), then of row 128 + r (part 1), into one
-        // stage of 2 kAColsPerStage columns; the stage goes to the MMA warps after part 1
-        auto push_part = [&](float (&hi)[kTileK], int part) -> bool {
-            float lo[kTileK];
-#pragma unroll
-            for (int i = 0; i < kTileK; ++i) {
-                const float h = tf32_hi(hi[i]);
-                if (THREE) lo[i] = hi[i] - h;
-                hi[i] = h;
-            }
-            if (part == 0) {
-                if (wraps >= 1 && !warp_wait_phase<32>(smem_u32(&bar_aempty[t]), (wraps - 1) & 1, abort_flag))
-                    return false;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            }
-            const uint32_t ta = tmem + lane_off + p.a_col + (uint32_t)(t * 2 + part) * kAColsPerStage;
-            tmem_st32(ta, hi);
-            if (THREE) tmem_st32(ta + 32, lo);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");   // the registers are reused
-            if (part == 1) {
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bar_afull[t]));
-                if (++t == p.n_stages) { t = 0; ++wraps; }
-            }
             return true;
         };
         if constexpr (MODE == 2) {
@@ -934,22 +910,15 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
             const bool fin = p.ov.patch != nullptr;
             bool ok = true;
             int64_t job = 0;
+            int turn = 0;   // whose K-step it is (not with tile pairs)
             for (int64_t i = 0; ok && i < my_tiles; ++i) {
                 const int64_t m0 = (blockIdx.x + i * gridDim.x) * TM;
                 const int64_t row0 = m0 / p.P;
                 const int oy0 = p.cv_imgs > 1 ? 0 : (int)((m0 - row0 * p.P) / TM) * p.cv_rows;
                 // rows past the end gather from the unit's first staged row (dropped later)
-                const RowInfo ri = row_info<false, false>(p, m0 + r);
+                const RowInfo ri = row_info<false, false>(p, m0 + (pair ? set * kTileM : 0) + r);
                 const uint32_t im = ri.ok ? (uint32_t)(ri.row - row0) : 0u;
                 const int line0 = ri.ok ? (ri.oy - oy0) * p.cv_hw + ri.ox : 0;
-                // tile pairs: this thread's row of the second tile too
-                uint32_t im1 = 0;
-                int line1 = 0;
-                if (pair) {
-                    const RowInfo r1 = row_info<false, false>(p, m0 + kTileM + r);
-                    im1 = r1.ok ? (uint32_t)(r1.row - row0) : 0u;
-                    line1 = r1.ok ? (r1.oy - oy0) * p.cv_hw + r1.ox : 0;
-                }
                 for (int c = 0; c < p.cv_nchunk; ++c, ++job) {
                     const int b = (int)(job % p.cv_nbuf);
                     const uint32_t use = (uint32_t)(job / p.cv_nbuf);
@@ -958,7 +927,7 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
                         break;
                     }
                     const uint32_t buf = cv_region + (uint32_t)b * cv_buf_bytes;
-                    const uint32_t base = buf + im * p.cv_img_bytes, base1 = buf + im1 * p.cv_img_bytes;
+                    const uint32_t base = buf + im * p.cv_img_bytes;
                     const int ntap = p.cv_ntap;
                     // the current tap and its line relative to a row's line0 (ky * cv_hw + kx),
                     // over the filter (or a window's 4x4 field)
@@ -994,26 +963,24 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
                             if (tap < ntap) offb = off;
                             next_tap();
                         }
-                        auto gather_k = [&](float (&v)[kTileK], uint32_t bse, int l0) {
-                            if (p.cv_cw == kTileK) {
-                                gather(v, 8, bse, l0 + offa);
-                            } else {
-                                gather(v, 4, bse, l0 + offa);
-                                if (offb >= 0) {
-                                    gather(v + 16, 4, bse, l0 + offb);
-                                } else {
-#pragma unroll
-                                    for (int e = 16; e < kTileK; ++e) v[e] = 0.f;
-                                }
-                            }
-                        };
+                        if (!pair) {
+                            const bool mine = turn == set;
+                            turn ^= 1;
+                            if (!mine) continue;
+                        }
                         float v[kTileK];
-                        gather_k(v, base, line0);
-                        if (pair) {
-                            if (!push_part(v, 0)) { ok = false; break; }
-                            gather_k(v, base1, line1);
-                            if (!push_part(v, 1)) { ok = false; break; }
-                        } else if (!push(v)) {
+                        if (p.cv_cw == kTileK) {
+                            gather(v, 8, base, line0 + offa);
+                        } else {
+                            gather(v, 4, base, line0 + offa);
+                            if (offb >= 0) {
+                                gather(v + 16, 4, base, line0 + offb);
+                            } else {
+#pragma unroll
+                                for (int e = 16; e < kTileK; ++e) v[e] = 0.f;
+                            }
+                        }
+                        if (!push(v)) {
                             ok = false;
                             break;
                         }
@@ -2407,7 +2374,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, S.tc_small || S.tc_conv ? kThreads : tc_threads<0, 0>(), smem, s>>>(p);
+        kern<<<grid, S.tc_small ? tc_threads<2, 0>() : tc_threads<0, 0>(), smem, s>>>(p);
     };
     if (dense && ff) { if (three) go(k_tc_gemm<0, true, kFuseClasses>); else go(k_tc_gemm<0, false, kFuseClasses>); }
     else if (dense) { if (three) go(k_tc_gemm<0, true>); else go(k_tc_gemm<0, false>); }
