@@ -333,7 +333,8 @@ struct TcParams {
     FinalFuse ff;                // the output layer computed in the epilogue (FCP > 0)
     SlotStore slot;              // slot.out: the tensor-core delta's scattered store
     // dense layers: A tiles (128 rows x one K-step) by tensor-map copies from warp 10
-    // instead of the producers' 16-byte copies; tile m0 starts at row coordinate m0
+    // instead of the producers' 16-byte copies: one of 128 rows from row m0, or with an overlay
+    // two of 64 rows, each within the inputs of one mutant
     int a_tma;
     // convolutions: 16-byte gathers (channels a multiple of 4; output positions in 16 bits each)
     int gather16;
@@ -564,8 +565,8 @@ __device__ __forceinline__ void produce_issue(const TcParams &p, RowInfo &pf, Lo
             }
         }
     } else {
-        // other channel counts: 4-byte copies of the thread's own
-        // row, the patch value taken directly for a mutated channel
+        // other channel counts: 4-byte copies of the thread's own row, the patch value taken
+        // directly for a mutated channel
         int ci = k0 % p.ic, t = k0 / p.ic, kx = t % p.kw, ky = t / p.kw;
         for (int i = 0; i < kTileK; ++i) {
             const int k = k0 + i;
