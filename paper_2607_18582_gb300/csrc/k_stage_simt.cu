@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(128) k_final_dense_w(const FinalParams p)
 // The weights come from the input-major copy Wt [F][C] with 16-byte loads all in flight;
 // each warp copies the rows' next 32 inputs (16-byte loads) into its own tile of 36-float
 // lines (16-byte stores and loads without bank conflicts) while it runs the FMAs of the
-// current 32; the warps' sums meet in shared memory and one warp runs the epilogue.  A block
+// current 32; the warps' sums meet in shared memory, the epilogues go round the warps.  A block
 // stays and takes many tiles of 32 rows, its weights placed once (a block per tile: 100 us for
 // 279,000 rows of 84 inputs, now 76).  Needs F a multiple of 4 and 16-byte aligned rows;
 // dynamic shared memory [F][4][4] (class c at
