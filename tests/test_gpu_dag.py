@@ -83,3 +83,38 @@ def test_projection_identity_mutants(M, ctx):
     assert not r["kill_bits"].any()
     for i in range(len(rows)):
         assert np.array_equal(r["logits"][i].view(np.uint32), lg0.view(np.uint32))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "tf32x3"])
+@pytest.mark.parametrize("ch,k", [(16, 1), (16, 3), (24, 3), (18, 3), (12, 0), (64, 0)])
+def test_residual_around_one_layer(M, ctx, oracle_mod, ch, k, prec):
+    """y = act(conv(x) + x), one 1x1 or 3x3 convolution (or a dense layer, k = 0) between a layer and
+    its own add: the first layer after a mutated one reads the mutated rows twice, as its input and as
+    its skip input.  Every operator before, in and after it, in one layer and over several, against
+    the oracle; memoized, vanilla and with the unchanged rows dropped bit for bit."""
+    b = wl._Builder("residual", (8, 8, 3), 5, 23)
+    x = b.conv(-1, ch, 3, pad=1)
+    if k:
+        x = b.add(b.conv(x, ch, k, pad=k // 2, act="none"), x)
+        x = b.gap(b.conv(x, 20, 1))
+    else:
+        # fan-in 16 ch: the tensor cores add with truncation, up to 2^-23 of the running sum per
+        # K = 8 step, 1.5e-5 for 1,024 inputs and half of the rule's 1e-4 for 4,096 (8 x 8 maps)
+        x = b.dense(b.maxpool(x), ch)
+        x = b.dense(b.add(b.dense(x, ch, act="none"), x), 32)
+    b.dense(x, 5, act="none")
+    X = wl.inputs(b.m, 70, 3)
+    ops = ("GF", "NS", "NAI", "WS", "NEB")
+    m = M.mure_model_load(ctx, b.m, precision=prec)
+    cache = M.mure_build_prefix_cache(m, X)
+    # (apart: a batch with mutants over several layers materialises every row)
+    for table in (wl.concat([wl.mutants(b.m, 5, seed=40 + l, ratios=(0.1,), ops=ops, layers=[l]) for l in range(b.m.n_layers())]),
+                  wl.modelwide_mutants(b.m, 10, seed=7, ratio=0.08, ops=ops)):
+        ora = oracle_mod.vanilla(b.m, X, table)
+        r = M.mure_eval_mutants(cache, table, logits=True)
+        ok, worst = logits_close(r["logits"], ora["logits"])
+        assert ok, worst
+        for other in (M.mure_eval_vanilla(m, X, table, logits=True),
+                      M.mure_eval_mutants(cache, table, logits=True, skip_unchanged=True)):
+            assert np.array_equal(other["logits"].view(np.uint32), r["logits"].view(np.uint32))
+            assert np.array_equal(other["kill_bits"], r["kill_bits"])
