@@ -40,9 +40,9 @@ struct StageParams {
 // channels per block, TM x TN sums per thread (simt_tile.cuh), operand tiles
 // double-buffered in shared memory, the next pieces in flight while the current are used.  A4: the
 // input channels come in fours on 16-byte rows, so a thread fetches four k of its row at once.
-// OV (with A4 only): a fetched piece takes the mutated channels from the patch.  Measured on
-// LeNet-5 in fp32 (1,500 x 150, FC 400-120 and 120-84): 0.88 ms with 4 x 4 sums per thread and
-// rows materialised first, 0.69 now; what bounds it is the latency of a tile's loads (few tiles
+// OV (with A4 only): a fetched piece takes the mutated channels from the patch (where: see
+// simt_overlay_inline).  Measured on LeNet-5 in fp32 (1,500 x 150, FC 400-120 and 120-84): 0.88 ms
+// with 4 x 4 sums per thread and rows materialised first, 0.69 now; what bounds it is the latency of a tile's loads (few tiles
 // per SM at these sizes) and 84 or 120 outputs in 128 columns.
 template <int BM, int BN, int TM, int TN, bool A4, bool OV>
 __global__ void __launch_bounds__(BM / TM * (BN / TN), A4 && !OV && BN != 64 ? 4 : 3) k_stage_simt(const StageParams p)
@@ -382,10 +382,22 @@ void stage_tiles(StageParams p, bool a4, cudaStream_t s)
 
 }  // namespace
 
+// Whether the stage's kernel applies the patch as it fetches rows of x; else the rows are
+// materialised first.  The pieces that a block fetches are fetched again for every tap and column
+// tile, and each looks at all mutated channels, so only few channels of rows that are read about
+// once are worth it.  Measured, fp32, 32 mutants, the layer with its rows, materialised / inline:
+// dense layers on cached rows 1.04 to 1.22 at one channel, 1.00 to 1.17 at two, 0.91 to 1.06 at four,
+// 0.7 at sixteen; of 512 outputs 0.98 at one; on rows of their own, where writing the patch over them
+// costs one small launch, 0.8 to 1.0 at one; 3 x 3 convolutions 0.8 to 0.98 at one channel, 0.55 to
+// 0.75 at eight.  The 1 x 1 kernel of few channels, whose tiles of 128 positions are patched in shared
+// memory: on cached rows 1.0 to 1.4 up to an eighth of the channels (64 -> 16: 1.20 at eight, 0.98 at
+// 24; 24 -> 96: 1.02 at two, 0.94 at six); on rows of their own 1.02 to 1.13 where there are more
+// outputs than inputs, else 0.86 to 1.03; tiles of 64 positions 0.94 at two.
 int simt_overlay_inline(const Stage &S, const Overlay &ov, Src x)
 {
-    return !S.tc && S.variant == 0 && (S.kind == MURE_NODE_CONV2D || S.kind == MURE_NODE_DENSE) && S.ic % 4 == 0 &&
-           ov.ch % 4 == 0 && aligned16(x.p, x.stride);
+    if (S.tc || S.variant > 0 || S.ic % 4 != 0 || ov.ch % 4 != 0 || !aligned16(x.p, x.stride)) return 0;
+    if (S.c11) return S.oh * S.ow % 128 == 0 && 8 * ov.kmax <= S.ic && (x.per_input || S.oc > S.ic);
+    return S.kind == MURE_NODE_DENSE && x.per_input && ov.kmax <= 2 && S.oc <= 128;
 }
 
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out,

@@ -494,3 +494,36 @@ def test_bad_labels_are_refused(M, ctx, on_device):
     a = M.mure_eval_mutants(M.mure_build_prefix_cache(model, put(w.X), put(good)), w.table)
     b = M.mure_eval_mutants(M.mure_build_prefix_cache(model, w.X, good), w.table)
     assert np.array_equal(a["kill_bits"], b["kill_bits"]) and a["scoreB"] == b["scoreB"]
+
+
+@pytest.mark.parametrize("kind,c,oc,size,k,rows", [
+    ("dense", 24, 32, 1, 1, 0), ("dense", 24, 128, 1, 2, 0), ("dense", 24, 32, 1, 3, 1), ("dense", 24, 132, 1, 1, 1),
+    ("dense", 26, 32, 1, 1, 1), ("conv3", 16, 20, 8, 1, 1), ("conv3", 64, 72, 8, 24, 1), ("conv1", 96, 96, 16, 2, 1),
+    ("conv1", 16, 64, 16, 2, 0), ("conv1", 16, 64, 16, 3, 1), ("conv1", 64, 16, 16, 8, 0), ("conv1", 64, 16, 16, 9, 1),
+    ("conv1", 16, 64, 8, 1, 1)])
+def test_patch_inline_or_rows(M, ctx, oracle_mod, kind, c, oc, size, k, rows):
+    """fp32: the first suffix layer takes the patch as it fetches its rows, or the rows are
+    materialised first, on both sides of the rule's lines; the oracle's logits and the bits of vanilla
+    either way."""
+    b = wl._Builder("first_suffix", (size, size, 5), 6, 31)
+    if kind == "dense":
+        x = b.dense(b.dense(-1, c), oc)
+    else:
+        x = b.conv(b.conv(-1, c, 3, pad=1), oc, int(kind[-1]), pad=int(kind[-1]) // 2)
+        x = b.gap(b.conv(x, 8, 1))
+    b.dense(x, 6, act="none")
+    X = wl.inputs(b.m, 70, 3)
+    table = wl.mutants(b.m, 5, seed=8, ratios=(k / c,), ops=("GF", "WS", "NEB", "NAI"), layers=[0])
+    assert set(table.n_neurons.tolist()) == {k}
+    ora = oracle_mod.vanilla(b.m, X, table)
+    m = M.mure_model_load(ctx, b.m, precision="fp32")
+    r = M.mure_eval_mutants(M.mure_build_prefix_cache(m, X), table, logits=True, kernel_timing=True)
+    # the values (convolutions of maps up to 48 KiB: operators with and without sums apart), then the
+    # rows (above 8,192 floats: copied, then patched)
+    floats = c * size * size
+    vals = 1 if kind == "dense" or floats * 4 > 48 * 1024 else 2
+    assert r["stats"]["launches_delta"] == vals + rows * (2 if kind != "dense" and floats > 8192 else 1)
+    ok, worst = logits_close(r["logits"], ora["logits"])
+    assert ok, worst
+    v = M.mure_eval_vanilla(m, X, table, logits=True)
+    assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
