@@ -1698,8 +1698,8 @@ mure_status mure_model_load(mure_ctx *c, const mure_model_desc *d, mure_model **
                 // keeps a row per position)
                 S.tc_win = S.tc_conv && getenv("MURE_TC_NOWINDOW") == nullptr && tc_win_geometry(S);
             }
-            // 1 x 1 layers of few channels: bound by HBM, in fp32 in every mode
-            S.c11 = S.variant == 0 && !(force && force[0] == '1') && conv1x1_geometry(S);
+            // 1 x 1 layers of few channels: bound by HBM, in fp32
+            S.c11 = S.variant == 0 && !(force && force[0] == '1') && conv1x1_geometry(S) && (!S.tc || conv1x1_over_tc(S));
             if (S.c11) S.tc = 0;
         }
         std::vector<int> wn;

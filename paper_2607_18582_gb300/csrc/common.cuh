@@ -168,9 +168,10 @@ struct Overlay {
 // scratch (the map before global average pooling; an LSTM's input sums).
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip,
                       float *y_out, int64_t y_stride, float *tmp, cudaStream_t s, const Overlay *ov = nullptr);
-// 1 x 1 convolutions of few channels in fp32: which layers, and the launcher (the map before
-// global average pooling goes to y).
+// 1 x 1 convolutions of few channels in fp32: which layers, which of them instead of the
+// tensor-core kernel, and the launcher (the map before global average pooling goes to y).
 int conv1x1_geometry(const Stage &S);
+int conv1x1_over_tc(const Stage &S);
 int launch_conv1x1(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out, int64_t y_stride,
                    cudaStream_t s, const Overlay *ov);
 // Whether the CUDA-core stage kernels apply the overlay as they fetch rows of x.

@@ -1,5 +1,5 @@
 // 1 x 1 convolutions of few channels (the expansions and projections of MobileNetV2's blocks) in
-// fp32 on the CUDA cores.  Such a layer moves (ic + oc) 4 bytes per position for ic x oc FMAs: at 16
+// fp32 on the CUDA cores, in the tensor-core precision modes too where that is faster.  Such a layer moves (ic + oc) 4 bytes per position for ic x oc FMAs: at 16
 // to 96 channels it is bound by HBM, not by either arithmetic unit, and the tensor-core kernel's
 // per-tile hand-overs (about 1,000 cycles per K-step) cost more than the products themselves.
 //
@@ -162,16 +162,32 @@ __global__ void __launch_bounds__(kThreads11, 4) k_conv1x1(const Conv11Params p)
 
 // Which layers the kernel takes: 1 x 1, stride 1, no pooling, channels in fours, maps of whole
 // tiles, an add only of a map of the same geometry, and at most 4,096 products per position.
-// Measured on 4,096 rows against the tensor-core kernel (3xTF32): 16 x 64 channels on 32 x 32 0.32
-// and 0.81 ms, 64 x 16 0.41 and 0.56, 32 x 128 on 16 x 16 0.23 and 0.37, 64 x 64 0.25 and 0.24 (8 x 8:
-// 0.063 and 0.076); past the line 96 x 96 0.81 and 0.39, 128 x 64 0.56 and 0.28, 128 x 128 1.03
-// and 0.50.  The whole MobileNetV2-style job (500 x 41): 13.4 -> 10.3 ms, and the logits' error
-// against 64 bits falls from 8.4e-7 to 2.3e-7.
+// Measured on 4,096 rows of 8 x 8, 16 x 16 and 32 x 32 maps against the implicit-GEMM kernel of the
+// fp32 mode, 53 shapes of 1,024 to 4,096 products: 0.29 to 0.99 of its time.
 int conv1x1_geometry(const Stage &S)
 {
     return S.kind == MURE_NODE_CONV2D && S.kh == 1 && S.kw == 1 && S.stride == 1 && S.pad == 0 && !S.pool && S.ic % 4 == 0 &&
            S.oc % 4 == 0 && S.ic <= 128 && S.oc <= 128 && S.ic * S.oc <= 4096 && S.oh * S.ow % 64 == 0 &&
            (!S.has_add || (S.sc_stride == 1 && S.sk_w == S.ow));
+}
+
+// Whether it takes them from the tensor-core kernel too.  More input channels mean fewer blocks on
+// an SM (the staged tiles) and no more output channels at once, so the line falls with both.  The
+// same measurement as a share of the tensor-core kernel's time, 3xTF32 (one TF32 product, whose time
+// is only some 5 % shorter: the hand-overs bound it, not the MMAs): 16 -> 64 0.41 to 0.46 (0.41 to
+// 0.49), 36 -> 112 0.75 (0.80), 36 -> 80 0.91 (0.98), 48 -> 64 0.78 to 0.92 (0.83 to 0.98), 48 -> 48 0.78 to
+// 1.01 (0.89 to 1.09), 64 -> 32 0.73 to 0.91 (0.78 to 0.95), 80 -> 32 0.86 to 0.90 (1.00 to 1.05), 96 -> 16
+// 0.74 to 0.99 (0.76 to 1.08), 96 -> 24 1.08 to 1.21 (1.12 to 1.27; kept, its fp32 sums are the more
+// exact ones); past the line 40 -> 80 0.95 to 1.27 (1.04 to 1.38), 64 -> 40 1.13 (1.19), 96 -> 32 1.11 to
+// 1.25, 128 -> 32 1.28 to 1.70.  64 -> 64 is 0.88 (0.91) on 8 x 8 maps, whose tiles of 64 positions leave
+// room for more blocks, and 1.13 to 1.16 (1.17 to 1.21) on larger ones.  The whole MobileNetV2-style
+// job (500 x 41): 13.4 -> 10.3 ms, and the logits' error against 64 bits falls from 8.4e-7 to 2.3e-7
+// (one TF32 product: 1.8e-4 to 4.2e-5).
+int conv1x1_over_tc(const Stage &S)
+{
+    if (S.ic <= 36 || (S.ic <= 48 && S.oc <= 64)) return 1;
+    if (S.oh * S.ow % 128 != 0 && S.ic <= 64 && S.oc <= 64) return 1;
+    return S.ic <= 96 && S.oc <= 32 && S.ic * S.oc <= 2560;
 }
 
 int launch_conv1x1(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip, float *y_out, int64_t y_stride,
