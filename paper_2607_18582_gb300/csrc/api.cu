@@ -801,8 +801,10 @@ void alloc_workspace(mure_ctx *c, Scratch &sc, const mure_model *m, int64_t rows
         ws.z_stride = zs;
         ws.zb = sc.get<float>(rows * zs);
     }
+    // (the stages that row_bytes counts: those that run, and a mutated LSTM layer itself)
     int64_t g = 0;
-    for (int v = 0; v < m->L; ++v) g = std::max(g, stage_scratch(m->st[v]));
+    const int first = vanilla ? 0 : m->st[lmin].kind == MURE_NODE_LSTM ? lmin : lmin + 1;
+    for (int v = first; v < m->L; ++v) g = std::max(g, stage_scratch(m->st[v]));
     if (g) ws.tmp = sc.get<float>(rows * g);
     ws.lw.proj = ws.tmp;
     if (lstm_kmax > 0) {

@@ -8,6 +8,8 @@ rule, kill bits exact outside near ties), memoized == vanilla bit for bit, the
 unchanged-row elimination exact, identity mutants never killed; the IMDB-sized model of
 Table 1 (vocabulary 20,000, width 128, 64 units, 80 steps) on a sample; an id outside the
 table is refused."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -135,3 +137,52 @@ def test_recurrent_identity_mutants_and_bad_ids(M, ctx):
     # the context stays usable
     again = M.mure_eval_mutants(M.mure_build_prefix_cache(m, X), wl.table_from_rows(rows), logits=True)
     assert np.array_equal(again["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
+class CountedMemory:
+    """A context whose device memory is counted: `live` and `peak` bytes."""
+
+    def __init__(self, M):
+        import torch
+        self.live = self.peak = 0
+        self.size = {}
+
+        def alloc(n, stream, user):
+            p = torch.cuda.caching_allocator_alloc(int(n), 0, int(stream or 0))
+            self.size[p] = n
+            self.live += n
+            self.peak = max(self.peak, self.live)
+            return p
+
+        def free(p, stream, user):
+            self.live -= self.size.pop(p)
+            torch.cuda.caching_allocator_delete(p)
+
+        self.keep = M._Allocator(M._ALLOC_FN(alloc), M._FREE_FN(free), None)
+        h = ctypes.c_void_p()
+        assert M.lib().mure_create(0, torch.cuda.current_stream().cuda_stream, ctypes.byref(self.keep), ctypes.byref(h)) == 0
+        self.ctx = M.Context(h.value, [self.keep])
+
+    def peak_of(self, call):
+        """(the call's result, the most bytes it held beyond those held before it)."""
+        before = self.peak = self.live
+        r = call()
+        return r, self.peak - before
+
+
+@pytest.mark.parametrize("layer", [0, 1, 2, 3])
+def test_scratch_within_the_workspace(M, layer):
+    """The scratch of a call stays within workspace_bytes (and 4 MiB for the table and the results),
+    whichever layers run: with output-layer mutants no LSTM does, so none of its sums (80 KiB a row here)
+    are allocated.  Memoized and vanilla give the same bits."""
+    model = wl.rnn(3, n_classes=3, vocab=60, dim=8, units=(64, 64), steps=80, name="rnn_scratch")
+    X = wl.inputs(model, 256, 2)
+    table = wl.mutants(model, 64, seed=5, ratios=(0.02,), ops=("GF", "NAI", "NEB"), layers=[layer])
+    mem = CountedMemory(M)
+    m = M.mure_model_load(mem.ctx, model)
+    cache = M.mure_build_prefix_cache(m, X)
+    cap = 32 << 20
+    r, peak = mem.peak_of(lambda: M.mure_eval_mutants(cache, table, logits=True, workspace_bytes=cap))
+    assert peak <= cap + (4 << 20), peak
+    v = M.mure_eval_vanilla(m, X, table, logits=True, workspace_bytes=cap)
+    assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
