@@ -1482,9 +1482,18 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
             CK(c, cudaMemcpy2DAsync(ca->x[0], str * 4, X, sz * 4, sz * 4, n_in,
                                     on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
         Scratch sc(c);
-        int64_t g = 0;
-        for (int v = 0; v < L; ++v) g = std::max(g, stage_scratch(m->st[v]));
-        float *tmp = g ? sc.get<float>(ca->n_pad * g) : nullptr;
+        // row scratch: the maps before global average pooling for all rows at once, an LSTM's input
+        // sums for as many rows as fit kLstmFloats (its layer then runs in parts: rows are independent)
+        constexpr int64_t kLstmFloats = (int64_t)1 << 28;
+        auto lstm_rows = [&](const Stage &S) {
+            return std::min(ca->n_pad, std::max<int64_t>(64, kLstmFloats / lstm_proj_floats(S)));
+        };
+        int64_t floats = 0;
+        for (const Stage &S : m->st) {
+            const bool lstm = S.kind == MURE_NODE_LSTM;
+            floats = std::max(floats, lstm ? lstm_rows(S) * lstm_proj_floats(S) : ca->n_pad * stage_scratch(S));
+        }
+        float *tmp = floats ? sc.get<float>(floats) : nullptr;
         // intermediate activations: in the cache (full) or in scratch rows (vanilla
         // only needs the predictions)
         std::vector<float *> xs(L + 1), zs(L);
@@ -1509,7 +1518,8 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         }
         for (int v = 0; v < L - 1; ++v) {
             const Stage &S = m->st[v];
-            if (v == 1 && ca->tok && tk.n <= ca->n_pad * S.iw) {
+            // by token where the tokens' sums fit the scratch
+            if (v == 1 && ca->tok && tk.n <= lstm_rows(S) * S.iw) {
                 LstmWs lw;
                 lw.proj = tmp;
                 c->launches += launch_lstm(S, Src{nullptr, 0, 0}, rm, zs[1], m->zd[1].stride, xs[2], m->xd[2].stride, nullptr,
@@ -1518,8 +1528,13 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
                 continue;
             }
             const Src skip = S.has_add ? Src{xs[S.skip_src], m->xd[S.skip_src].stride, 0} : Src{nullptr, 0, 0};
-            c->launches += launch_stage_simt(S, Src{xs[S.in_src], m->xd[S.in_src].stride, 0}, rm, zs[v], m->zd[v].stride, skip,
-                                             xs[v + 1], m->xd[v + 1].stride, tmp, s);
+            const int64_t part = S.kind == MURE_NODE_LSTM ? lstm_rows(S) : ca->n_pad;
+            for (int64_t r0 = 0; r0 < ca->n_pad; r0 += part) {
+                const int R = (int)std::min(part, ca->n_pad - r0);
+                const Src x{xs[S.in_src] + r0 * m->xd[S.in_src].stride, m->xd[S.in_src].stride, 0};
+                c->launches += launch_stage_simt(S, x, RowMap{0, R, R}, zs[v] + r0 * m->zd[v].stride, m->zd[v].stride, skip,
+                                                 xs[v + 1] + r0 * m->xd[v + 1].stride, m->xd[v + 1].stride, tmp, s);
+            }
             check_launch(c);
         }
         FinalArgs fa{};

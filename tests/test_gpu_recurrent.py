@@ -186,3 +186,24 @@ def test_scratch_within_the_workspace(M, layer):
     assert peak <= cap + (4 << 20), peak
     v = M.mure_eval_vanilla(m, X, table, logits=True, workspace_bytes=cap)
     assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
+@pytest.mark.parametrize("vocab", [60, 1500000])
+def test_cache_build_in_parts(M, vocab):
+    """Building a cache holds at most 1 GiB of an LSTM's input sums (80 KiB a row here; and 32 MiB for
+    the tokens' tables) beside the cache itself: the layer runs in parts.  The logits of inputs in
+    every part are those of a cache of these inputs alone; with few tokens, and with more than the
+    scratch has sums for."""
+    model = wl.rnn(3, n_classes=3, vocab=vocab, dim=4, units=(64, 64), steps=80, name="rnn_parts")
+    X = wl.inputs(model, 20000, 2)
+    mem = CountedMemory(M)
+    m = M.mure_model_load(mem.ctx, model)
+    held = mem.live
+    cache, peak = mem.peak_of(lambda: M.mure_build_prefix_cache(m, X))
+    scratch = peak - (mem.live - held)
+    assert scratch <= (1 << 30) + (32 << 20), scratch
+    logits, pred = M.mure_cache_outputs(cache)
+    cache.free()
+    some = np.r_[0:70, 13070:13140, 19940:20000]
+    lg, pr = M.mure_cache_outputs(M.mure_build_prefix_cache(m, X[some]))
+    assert np.array_equal(lg.view(np.uint32), logits[some].view(np.uint32)) and np.array_equal(pr, pred[some])
