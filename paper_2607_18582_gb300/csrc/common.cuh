@@ -164,6 +164,16 @@ struct Overlay {
     const int32_t *op = nullptr;
 };
 
+// Lets a kernel be launched with up to `most` bytes of dynamic shared memory.  The limit belongs to
+// the kernel in the process, not to a stream or context, and other host threads launch the same
+// kernel: `most` is the largest that any call of it needs, never one call's own size, which
+// another thread could set lower between this call's setting and its launch.
+template <class Kern>
+inline void allow_dynamic_smem(Kern kern, int most)
+{
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // Stage v over R rows: z (optional) and y = post(act1(conv(x) + b)).  tmp: the stage's row
 // scratch (the map before global average pooling; an LSTM's input sums).
 int launch_stage_simt(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, Src skip,

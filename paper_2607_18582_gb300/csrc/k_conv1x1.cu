@@ -38,6 +38,8 @@ struct Conv11Params {
 };
 
 constexpr int kThreads11 = 128;
+// the largest layer's weights and staged tiles: 4,096 products (conv1x1_geometry), 128 channels
+constexpr int kSmemMax11 = (4096 + 2 * 128 * (128 + 4)) * (int)sizeof(float);
 
 __device__ __forceinline__ void copy16(float *dst, const float *src)
 {
@@ -209,7 +211,7 @@ int launch_conv1x1(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_str
     const int smem = (S.ic * S.oc + 2 * p.tp * (S.ic + 4)) * (int)sizeof(float);
     const unsigned blocks = (unsigned)std::min<int64_t>(p.tiles, 4 * 152);
     auto go = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        allow_dynamic_smem(kern, kSmemMax11);
         kern<<<blocks, kThreads11, smem, s>>>(p);
     };
     // the positions per thread with the fewer rounds over a tile (of 16 outputs eight per thread

@@ -285,7 +285,7 @@ int launch_conv_small(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     p.y = y_out; p.y_stride = y_stride;
     auto go = [&](auto kern, int rows, int threads, int floats) {
         const int smem = floats * (int)sizeof(float);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        allow_dynamic_smem(kern, smem);
         kern<<<(unsigned)((rm.R + rows - 1) / rows), threads, smem, s>>>(p);
     };
     if (S.variant == 1) go(k_conv_small<5, 5, 6, 16, 4, 14, 14, 0, true, 2, 25>, 2, 200, 150 * 16 + 2 * 14 * 14 * 6);
@@ -534,14 +534,13 @@ int launch_dot(const Stage &S, Src z, Src x, RowMap rm, const PatchArgs &pa, int
             ((size_t)HP * WP * IC + (EG ? 0 : (size_t)SMAX * KH * KW * IC) + (size_t)S.oc * S.oh * S.ow) * sizeof(float);
         if (smem2 <= 200 * 1024) {
             auto kern = k_patch_dot_in<KH, KW, IC, WP, HP, PAD, POOL, CW, SG, SMAX, NT, EG>;
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+            allow_dynamic_smem(kern, (int)smem2);
             kern<<<(unsigned)rm.T, NT, smem2, s>>>(p);
             return 1;
         }
     }
     const size_t smem = ((size_t)KMAX * KH * KW * IC + (size_t)p.rows_per_block * HP * WP * IC) * sizeof(float);
-    cudaFuncSetAttribute(k_patch_dot<KH, KW, IC, WP, HP, PAD, POOL, KMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+    allow_dynamic_smem(k_patch_dot<KH, KW, IC, WP, HP, PAD, POOL, KMAX>, (int)smem);
     const dim3 grid((unsigned)p.G, (unsigned)((rm.T + p.rows_per_block - 1) / p.rows_per_block));
     k_patch_dot<KH, KW, IC, WP, HP, PAD, POOL, KMAX><<<grid, 256, smem, s>>>(p);
     return 1;

@@ -132,7 +132,7 @@ int launch_expand(const ExpandArgs &ea, cudaStream_t s)
         }
         if (ea.max_ws > 0) {
             const int smem = 2 * f_ws * (int)sizeof(int);
-            cudaFuncSetAttribute(k_expand_ws, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            allow_dynamic_smem(k_expand_ws, 2 * kShuffleMax * (int)sizeof(int));
             k_expand_ws<<<n, f_ws > 1024 ? 1024 : 256, smem, s>>>(a);
             ++launches;
         }

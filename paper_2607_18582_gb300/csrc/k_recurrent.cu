@@ -705,8 +705,7 @@ int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride
     }
     p.bm = bm;
     p.blocks_per_g = (rows_per_g + bm - 1) / bm;
-    const size_t smem = (size_t)bm * (2 * kRecLine + kMaxUnits) * 4;
-    cudaFuncSetAttribute(k_lstm_rec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = (size_t)bm * (2 * kRecLine + kMaxUnits) * 4;   // (26 KiB at most)
     k_lstm_rec<<<(unsigned)(G * p.blocks_per_g), kRecThreads, smem, s>>>(p);
     return launches + 1;
 }

@@ -990,17 +990,18 @@ int launch_final_dense(const Stage &S, Src x, RowMap rm, const FinalArgs &fa, cu
     if (x.per_input && fa.mode == 0 && !fa.z_out && p.F <= kRowsF - 4 && p.F % 4 == 0 && cp == 12 &&
         (x.stride & 3) == 0 && (reinterpret_cast<uintptr_t>(x.p) & 15) == 0 && (!ov || (ov->cells == 1 && ov->kmax <= 4))) {
         const size_t smem = ((size_t)p.F * 12 + 128 * kRowsF) * sizeof(float);
-        cudaFuncSetAttribute(k_final_dense_rows<12, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_dynamic_smem(k_final_dense_rows<12, 3>, ((kRowsF - 4) * 12 + 128 * kRowsF) * (int)sizeof(float));
         k_final_dense_rows<12, 3><<<blocks, 128, smem, s>>>(p);
         return 1;
     }
     // aligned rows of whole 16-byte pieces, weights that fit in shared memory: per-warp rows
     // with the next inputs in flight
     const size_t wbytes = (size_t)p.F * cp * sizeof(float);
+    constexpr int kWeightBytes = 96 * 1024;
     if (p.F % 4 == 0 && (x.stride & 3) == 0 && (reinterpret_cast<uintptr_t>(x.p) & 15) == 0 && cp <= 12 &&
-        wbytes <= 96 * 1024) {
+        wbytes <= kWeightBytes) {
         auto go = [&](auto kern) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wbytes);
+            allow_dynamic_smem(kern, kWeightBytes);
             kern<<<blocks, 128, wbytes, s>>>(p);
         };
         if (cp <= 4) go(k_final_dense_w<4>);
@@ -1008,7 +1009,7 @@ int launch_final_dense(const Stage &S, Src x, RowMap rm, const FinalArgs &fa, cu
         else {
             // 9 to 12 classes: a block's 32 rows shared by four warps
             const size_t sbytes = (size_t)p.F * 16 * sizeof(float);
-            cudaFuncSetAttribute(k_final_dense_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sbytes);
+            allow_dynamic_smem(k_final_dense_split, kWeightBytes / 12 * 16);
             // blocks that stay (four per SM) and take several tiles: the weights are placed once
             // per block, not once per 32 rows
             const int tiles = (rm.R + 31) / 32;

@@ -2207,20 +2207,22 @@ static bool conv_x_tensor_map(const Stage &S, Src x, RowMap rm, const ConvTile &
 
 // Dynamic shared memory a k_tc_gemm instance may use: the device's opt-in maximum less
 // the kernel's static shared memory.
-template <class Kern>
-static size_t tc_dyn_smem_max(Kern kern)
+template <void (*KERN)(TcParams)>
+static size_t tc_dyn_smem_max()
 {
-    static size_t cached = 0;
-    if (!cached) {
+    static const size_t most = [] {
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         cudaFuncAttributes fa{};
-        cudaFuncGetAttributes(&fa, kern);
-        cached = optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
-    }
-    return cached;
+        cudaFuncGetAttributes(&fa, KERN);
+        return optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    }();
+    return most;
 }
+
+template <int MODE, bool THREE, int FCP = 0>
+using TcKernel = std::integral_constant<void (*)(TcParams), k_tc_gemm<MODE, THREE, FCP>>;
 
 int tc_final_fusable(const Stage &S, const Stage &SL)
 {
@@ -2296,7 +2298,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
         // their staged rows fit (measured: conv 64->64 -14%, ResNet-20's 16- to 64-channel
         // convolutions -9..-10%; at 128 outputs the pair's single accumulator set, which
         // no longer overlaps the epilogue, made it 4-20% slower)
-        const size_t room = three ? tc_dyn_smem_max(k_tc_gemm<3, true>) : tc_dyn_smem_max(k_tc_gemm<3, false>);
+        const size_t room = three ? tc_dyn_smem_max<k_tc_gemm<3, true>>() : tc_dyn_smem_max<k_tc_gemm<3, false>>();
         bool ok = false;
         if (!ss && !S.tc_win && nt_max <= 64 && conv_tile(S, ct, 2 * kTileM, 64 * 1024) &&
             room >= 1024 + b_bytes + 2 * (size_t)ct.imgs * ct.img_bytes)
@@ -2373,16 +2375,18 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     }
     const int ny = (p.Np + p.slice_w - 1) / p.slice_w;
     const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
-    auto go = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto go = [&](auto kernel) {
+        constexpr auto kern = decltype(kernel)::value;
+        allow_dynamic_smem(kern, (int)tc_dyn_smem_max<kern>());
         kern<<<grid, S.tc_small ? tc_threads<2, 0>() : tc_threads<0, 0>(), smem, s>>>(p);
     };
-    if (dense && ff) { if (three) go(k_tc_gemm<0, true, kFuseClasses>); else go(k_tc_gemm<0, false, kFuseClasses>); }
-    else if (dense) { if (three) go(k_tc_gemm<0, true>); else go(k_tc_gemm<0, false>); }
-    else if (S.tc_small) { if (three) go(k_tc_gemm<2, true>); else go(k_tc_gemm<2, false>); }
-    else if (S.tc_conv && ss && S.has_add) { if (three) go(k_tc_gemm<3, true, -1>); else go(k_tc_gemm<3, false, -1>); }
-    else if (S.tc_conv) { if (three) go(k_tc_gemm<3, true>); else go(k_tc_gemm<3, false>); }
-    else { if (three) go(k_tc_gemm<1, true>); else go(k_tc_gemm<1, false>); }
+    auto either = [&](auto x3, auto x1) { three ? go(x3) : go(x1); };
+    if (dense && ff) either(TcKernel<0, true, kFuseClasses>(), TcKernel<0, false, kFuseClasses>());
+    else if (dense) either(TcKernel<0, true>(), TcKernel<0, false>());
+    else if (S.tc_small) either(TcKernel<2, true>(), TcKernel<2, false>());
+    else if (S.tc_conv && ss && S.has_add) either(TcKernel<3, true, -1>(), TcKernel<3, false, -1>());
+    else if (S.tc_conv) either(TcKernel<3, true>(), TcKernel<3, false>());
+    else either(TcKernel<1, true>(), TcKernel<1, false>());
     int launches = 1;
     if (S.gap) launches += launch_gap(gap_tmp, map_stride, mh * mw, S.oc, rm.R, y_out, y_stride, s);
     return launches;
