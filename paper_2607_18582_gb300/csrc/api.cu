@@ -1409,14 +1409,26 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
     FAILIF(n_in < 0, c, MURE_ERR_INVALID_ARG, "n_inputs < 0");
     FAILIF(n_in > 0 && !X, c, MURE_ERR_INVALID_ARG, "NULL X");
     FAILIF(n_in > ((int64_t)1 << 30), c, MURE_ERR_UNSUPPORTED, "more than 2^30 inputs");
-    auto check_labels = [&](const int32_t *lab) {
+    cudaStream_t s = c->stream;
+    if (labels && n_in > 0) {
+        // labels on the device are fetched for the check, after what was queued to write them on the
+        // context's stream or on the default stream
+        std::vector<int32_t> fetched;
+        const int32_t *lab = labels;
+        if (on_dev) {
+            fetched.resize(n_in);
+            if (s && s != cudaStreamLegacy) {
+                CK(c, cudaEventRecord(c->ev[7], cudaStreamLegacy));
+                CK(c, cudaStreamWaitEvent(s, c->ev[7], 0));
+            }
+            CK(c, cudaMemcpyAsync(fetched.data(), labels, n_in * 4, cudaMemcpyDeviceToHost, s));
+            CK(c, cudaStreamSynchronize(s));
+            lab = fetched.data();
+        }
         for (int64_t t = 0; t < n_in; ++t)
             FAILIF(lab[t] < 0 || lab[t] >= m->n_classes, c, MURE_ERR_INVALID_ARG, "label %d of input %lld", lab[t],
                    (long long)t);
-    };
-    // labels on the device are counted there (k_label_set, below)
-    if (labels && !on_dev) check_labels(labels);
-    cudaStream_t s = c->stream;
+    }
     auto *ca = new mure_cache();
     ca->model = m;
     ca->full = full;
@@ -1546,31 +1558,19 @@ mure_cache *build_cache(mure_model *m, const float *X, int64_t n_in, const int32
         fa.pred_out = ca->pred0;
         c->launches += launch_final_dense(m->st[L - 1], Src{xs[L - 1], m->xd[L - 1].stride, 0}, rm, fa, s);
         check_launch(c);
-        if (labels && on_dev && s && s != cudaStreamLegacy) {
-            // labels written on the default stream are waited for whatever the context's stream
-            CK(c, cudaEventRecord(c->ev[7], cudaStreamLegacy));
-            CK(c, cudaStreamWaitEvent(s, c->ev[7], 0));
-        }
         CK(c, cudaMemcpyAsync(ca->label, labels ? labels : ca->pred0, n_in * 4,
                               labels && !on_dev ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, s));
-        uint32_t *mask = sc.get<uint32_t>(kLabelWords + 1);
-        CK(c, cudaMemsetAsync(mask, 0, 4 * (kLabelWords + 1), s));
-        c->launches += launch_label_set(ca->label, n_in, m->n_classes, mask, s);
+        uint32_t *mask = sc.get<uint32_t>(kLabelWords);
+        CK(c, cudaMemsetAsync(mask, 0, 4 * kLabelWords, s));
+        c->launches += launch_label_set(ca->label, n_in, mask, s);
         check_launch(c);
-        uint32_t hm[kLabelWords + 1] = {};
+        uint32_t hm[kLabelWords] = {};
         int dev_err = 0;
         Results res(c);
         res.add(hm, mask, sizeof hm);
         res.add(&dev_err, c->err_dev, sizeof(int));
         if (tok_count) res.add(&ca->tok_n, tok_count, sizeof(int));
         res.finish();
-        if (hm[kLabelWords]) {
-            // the first bad label, as for labels on the host
-            std::vector<int32_t> lab(n_in);
-            CK(c, cudaMemcpy(lab.data(), ca->label, n_in * 4, cudaMemcpyDeviceToHost));
-            if (dev_err) CK(c, cudaMemset(c->err_dev, 0, sizeof(int)));
-            check_labels(lab.data());
-        }
         ca->n_label_values = 0;
         for (int k = 0; k < kLabelWords; ++k) ca->n_label_values += __builtin_popcount(hm[k]);
         if (dev_err) {

@@ -415,9 +415,8 @@ int launch_unchanged(const UnchangedArgs &ua, RowMap rm, int32_t *flags, int32_t
 int launch_scores(const uint32_t *kill32, int64_t n_mut, int64_t words32, const int32_t *label, int n_classes,
                   unsigned long long *totals /* [2]: killed, sum of label counts */, cudaStream_t s);
 
-// Distinct labels among n inputs: a bitset of kLabelWords words, then the number of labels
-// outside [0, n_classes) (all zeroed by the caller).
-int launch_label_set(const int32_t *label, int64_t n, int n_classes, uint32_t *mask, cudaStream_t s);
+// Distinct labels among n inputs (bitset of kLabelWords words; mask zeroed by the caller).
+int launch_label_set(const int32_t *label, int64_t n, uint32_t *mask, cudaStream_t s);
 
 // Rows of n floats without their padding: out [R][n].
 int launch_pack_rows(const float *in, int64_t in_stride, int n, int64_t R, float *out, cudaStream_t s);

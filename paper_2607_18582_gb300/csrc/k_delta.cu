@@ -886,17 +886,15 @@ int launch_scores(const uint32_t *kill32, int64_t n_mut, int64_t words32, const 
     return 1;
 }
 
-__global__ void k_label_set(const int32_t *__restrict__ label, int64_t n, int n_classes, uint32_t *mask)
+__global__ void k_label_set(const int32_t *__restrict__ label, int64_t n, uint32_t *mask)
 {
-    uint32_t m[kLabelWords] = {}, bad = 0;
+    uint32_t m[kLabelWords] = {};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int lb = label[i];
-        if (lb < 0 || lb >= n_classes) ++bad;
 #pragma unroll
         for (int k = 0; k < kLabelWords; ++k)
             if ((lb >> 5) == k) m[k] |= 1u << (lb & 31);
     }
-    if (bad) atomicAdd(mask + kLabelWords, bad);
 #pragma unroll
     for (int k = 0; k < kLabelWords; ++k) {
         uint32_t v = m[k];
@@ -906,12 +904,12 @@ __global__ void k_label_set(const int32_t *__restrict__ label, int64_t n, int n_
     }
 }
 
-int launch_label_set(const int32_t *label, int64_t n, int n_classes, uint32_t *mask, cudaStream_t s)
+int launch_label_set(const int32_t *label, int64_t n, uint32_t *mask, cudaStream_t s)
 {
     if (n <= 0) return 0;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 1024) blocks = 1024;
-    k_label_set<<<(unsigned)blocks, 256, 0, s>>>(label, n, n_classes, mask);
+    k_label_set<<<(unsigned)blocks, 256, 0, s>>>(label, n, mask);
     return 1;
 }
 

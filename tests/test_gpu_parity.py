@@ -491,6 +491,13 @@ def test_bad_labels_are_refused(M, ctx, on_device):
         with pytest.raises(M.MureError, match=f"label {bad_value} of input 41") as ei:
             M.mure_build_prefix_cache(model, put(w.X), put(bad))
         assert ei.value.status == 1
+    # before any kernel is launched, by either entry point
+    launched = M.mure_kernel_launches(ctx)
+    for call in (lambda: M.mure_build_prefix_cache(model, put(w.X), put(bad)),
+                 lambda: M.mure_eval_vanilla(model, put(w.X), w.table, put(bad))):
+        with pytest.raises(M.MureError, match="of input 41"):
+            call()
+    assert M.mure_kernel_launches(ctx) == launched
     a = M.mure_eval_mutants(M.mure_build_prefix_cache(model, put(w.X), put(good)), w.table)
     b = M.mure_eval_mutants(M.mure_build_prefix_cache(model, w.X, good), w.table)
     assert np.array_equal(a["kill_bits"], b["kill_bits"]) and a["scoreB"] == b["scoreB"]
