@@ -1233,12 +1233,20 @@ struct Outputs {
     const mure_eval_opts *opts;
 };
 
+// The checks of a call's outputs and options (before any device work is queued).
+void check_outputs(mure_ctx *c, const Outputs &out, int64_t n, int64_t n_in)
+{
+    if (n <= 0 || n_in <= 0) return;   // nothing is evaluated
+    FAILIF(!out.kill_bits, c, MURE_ERR_INVALID_ARG, "NULL kill_bits");
+    FAILIF(out.opts && out.opts->skip_unchanged != 0 && out.opts->skip_unchanged != 1, c, MURE_ERR_INVALID_ARG,
+           "skip_unchanged must be 0 or 1");
+}
+
 void evaluate(mure_ctx *c, const mure_model *m, const mure_cache *ca, const mure_mutant *t, int64_t n,
               const int32_t *pool, int64_t pool_len, bool vanilla, const Outputs &out)
 {
     const mure_eval_opts dflt{};
     const mure_eval_opts *o = out.opts ? out.opts : &dflt;
-    FAILIF(n > 0 && ca->n_in > 0 && !out.kill_bits, c, MURE_ERR_INVALID_ARG, "NULL kill_bits");
     cudaStream_t s = c->stream;
     Scratch sc(c);
     CK(c, cudaEventRecord(c->ev[0], s));
@@ -1311,7 +1319,6 @@ void evaluate(mure_ctx *c, const mure_model *m, const mure_cache *ca, const mure
         Workspace ws;
         alloc_workspace(c, sc, m, rows, vanilla, lmin, patch_floats, delta_slots, delta_k, lstm_kmax,
                         std::min(Gmax, gbig), ws, dt.has_later);
-        FAILIF(o->skip_unchanged != 0 && o->skip_unchanged != 1, c, MURE_ERR_INVALID_ARG, "skip_unchanged must be 0 or 1");
         if (!vanilla && o->skip_unchanged) {
             ec.skip_unchanged = true;
             ws.uflags = sc.get<int32_t>(rows);
@@ -1885,8 +1892,9 @@ mure_status mure_eval_mutants(mure_cache *ca, const mure_mutant *table, int64_t 
         CK(c, cudaSetDevice(c->device));
         FAILIF(!ca->full, c, MURE_ERR_INVALID_ARG, "cache holds no activations");
         check_table(c, ca->model, table, n_mutants, neuron_pool, pool_len);
-        evaluate(c, ca->model, ca, table, n_mutants, neuron_pool, pool_len, false,
-                 Outputs{kill_bits, score_killed_frac, score_deepmutation, stats, opts});
+        const Outputs out{kill_bits, score_killed_frac, score_deepmutation, stats, opts};
+        check_outputs(c, out, n_mutants, ca->n_in);
+        evaluate(c, ca->model, ca, table, n_mutants, neuron_pool, pool_len, false, out);
     });
 }
 
@@ -1900,13 +1908,14 @@ mure_status mure_eval_vanilla(mure_model *m, const float *X, int64_t n_inputs, c
     return run(c, [&] {
         CK(c, cudaSetDevice(c->device));
         check_table(c, m, table, n_mutants, neuron_pool, pool_len);
+        const Outputs out{kill_bits, score_killed_frac, score_deepmutation, stats, opts};
+        check_outputs(c, out, n_mutants, n_inputs);
         mure_cache *ca = build_cache(m, X, n_inputs, labels, x_on_device, false);
         struct Free {
             mure_cache *ca;
             ~Free() { mure_cache_free(ca); }
         } fr{ca};
-        evaluate(c, m, ca, table, n_mutants, neuron_pool, pool_len, true,
-                 Outputs{kill_bits, score_killed_frac, score_deepmutation, stats, opts});
+        evaluate(c, m, ca, table, n_mutants, neuron_pool, pool_len, true, out);
     });
 }
 

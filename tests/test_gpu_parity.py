@@ -534,3 +534,23 @@ def test_patch_inline_or_rows(M, ctx, oracle_mod, kind, c, oc, size, k, rows):
     assert ok, worst
     v = M.mure_eval_vanilla(m, X, table, logits=True)
     assert np.array_equal(v["logits"].view(np.uint32), r["logits"].view(np.uint32))
+
+
+@pytest.mark.parametrize("bad", ["kill_bits", "skip_unchanged"])
+def test_bad_outputs_and_options_are_refused_first(M, ctx, bad):
+    """A missing kill matrix or an option that is neither 0 nor 1: INVALID_ARG from both entry points
+    with nothing launched."""
+    import ctypes
+    w = wl.workload("mlp", 70, 8)
+    model = M.mure_model_load(ctx, w.model)
+    cache = M.mure_build_prefix_cache(model, w.X)
+    arr, pool, plen = M.table_array(w.table)
+    kill = np.zeros((8, 2), np.uint64)
+    opts = M._Opts(0, 0, 0, None, 2 if bad == "skip_unchanged" else 0, 0)
+    rest = (arr.ctypes.data, 8, pool.ctypes.data, plen, ctypes.byref(opts), kill.ctypes.data if bad != "kill_bits" else None,
+            None, None, None)
+    X = np.ascontiguousarray(w.X)
+    launched = M.mure_kernel_launches(ctx)
+    for st in (M.lib().mure_eval_mutants(cache.h, *rest), M.lib().mure_eval_vanilla(model.h, X.ctypes.data, 70, None, 0, *rest)):
+        assert st == 1 and bad in M.lib().mure_last_error(ctx.h).decode()
+    assert M.mure_kernel_launches(ctx) == launched and not kill.any()
