@@ -139,6 +139,69 @@ def test_recurrent_identity_mutants_and_bad_ids(M, ctx):
     assert np.array_equal(again["logits"].view(np.uint32), r["logits"].view(np.uint32))
 
 
+def cell_outputs(M, ctx, x):
+    """h of one LSTM step on the scalars x, [len(x)][units], one unit per form (biases +-100
+    saturate a gate to 1 or 0):
+      0: sigmoid(x) tanh(1)   1: tanh(tanh(x))   2: tanh(sigmoid(x))   3, 4, 5: the same with 3e38 x"""
+    H, on = 6, 100.0
+    W, b = np.zeros((H, 4, 1 + H), np.float32), np.full((H, 4), on, np.float32)
+    for u in range(H):
+        gate = (3, 2, 0)[u % 3]   # the gates are i, f, g, o
+        W[u, gate, 0] = 1.0 if u < 3 else 3e38
+        b[u, gate] = 0.0
+    net = wl.Model("cell", (1, 1, 1), H)
+    net.nodes.append(wl.Node("lstm", (-1,), "none", 0, 1, 1, 0, 1, H, W, b))
+    net.nodes.append(wl.Node("dense", (0,), "none", 1, 1, 1, 0, H, H, np.eye(H, dtype=np.float32), np.zeros(H, np.float32)))
+    X = np.asarray(x, np.float32).reshape(-1, 1, 1, 1)
+    return M.mure_cache_outputs(M.mure_build_prefix_cache(M.mure_model_load(ctx, net), X))[0]
+
+
+def test_cell_functions(M, ctx):
+    """The cell's sigmoid and tanh against 64 bits, over [-100, 100] densely and around 0, the change
+    of form at 0.6 (in either place of tanh(tanh(x))) and the clamps.  Bounds: the worst relative
+    error that the kernel's comment states, 1.6e-7 each (the inner tanh's arrives damped), and 2^-24
+    per product.  The mean matters more than the spread, since a recurrence adds it up."""
+    near = lambda v: np.float32(v) * (1 + np.arange(-40, 41, dtype=np.float32) * np.float32(2.0 ** -23))  # noqa: E731
+    x = np.concatenate([np.linspace(-100, 100, 200001), np.linspace(-1, 1, 50001)] +
+                       [s * near(v) for s in (1, -1) for v in (0.6, np.arctanh(0.6), 40.0, 87.0, 1e-30, 1e-6, 20.0)]).astype(np.float32)
+    h = cell_outputs(M, ctx, x).astype(np.float64)
+    x64 = x.astype(np.float64)
+    u = 2.0 ** -24
+    sig, tanh = 1 / (1 + np.exp(-x64)), np.tanh(x64)
+    live = x64 >= -87                       # below, sigmoid is 0 (it would be a subnormal number)
+    assert not h[~live, 0].any() and not h[~live, 2].any()
+    one = cell_outputs(M, ctx, [100.0])[0, 0].astype(np.float64)   # tanh(1), the gate at 1
+    assert abs(one / np.tanh(1.0) - 1) <= 2 * 1.6e-7 + 2 * u
+    e = h[live, 0] / (one * sig[live]) - 1
+    assert np.abs(e).max() <= 1.6e-7 + 2 * u, np.abs(e).max()
+    dense = np.abs(x64[live]) <= 20
+    assert abs(e[dense].mean()) <= 1e-8 and e[dense].std() <= 6e-8, (e[dense].mean(), e[dense].std())
+    with np.errstate(divide="ignore", invalid="ignore"):
+        e = np.where(x64 == 0, h[:, 1], h[:, 1] / np.tanh(tanh) - 1)
+    assert np.abs(e).max() <= 2 * 1.6e-7 + 2 * u, np.abs(e).max()
+    e = h[live, 2] / np.tanh(sig[live]) - 1
+    assert np.abs(e).max() <= 2 * 1.6e-7 + 2 * u, np.abs(e).max()
+
+
+def test_cell_functions_at_the_ends(M, ctx):
+    """Signs, zeros, subnormal numbers, infinities and NaN."""
+    x = np.array([0.0, -0.0, 1e-40, -1e-40, 1e-45, 200.0, -200.0, 3e38, -3e38], np.float32)
+    h = cell_outputs(M, ctx, x)
+    tanh1 = cell_outputs(M, ctx, [100.0])[0, 0]
+    half = np.float32(0.5) * tanh1
+    assert np.abs(h[:5, 0] - half).max() <= 2.0 ** -24 and np.abs(h[:5, 2] - np.tanh(0.5)).max() <= 2.0 ** -23
+    # an argument below the normal numbers may come back as 0 of either sign, no more
+    assert np.abs(h[:5, 1]).max() <= 1e-40
+    assert np.array_equal(h[5:, 0], np.float32([tanh1, 0, tanh1, 0]))
+    assert np.allclose(h[5:, 1], np.tanh(1.0) * np.float32([1, -1, 1, -1]), rtol=5e-7, atol=0)
+    # 3e38 x: infinite from |x| >= 2 on
+    inf = cell_outputs(M, ctx, np.array([10.0, -10.0], np.float32))
+    assert np.array_equal(inf[:, 3], np.float32([tanh1, 0]))
+    assert np.allclose(inf[:, 4], np.tanh(1.0) * np.float32([1, -1]), rtol=5e-7, atol=0)
+    assert np.allclose(inf[:, 5], np.float32([np.tanh(1.0), 0]), rtol=5e-7, atol=0)
+    assert np.isnan(cell_outputs(M, ctx, np.array([np.nan], np.float32))).all()
+
+
 class CountedMemory:
     """A context whose device memory is counted: `live` and `peak` bytes."""
 
