@@ -554,3 +554,33 @@ def test_bad_outputs_and_options_are_refused_first(M, ctx, bad):
     for st in (M.lib().mure_eval_mutants(cache.h, *rest), M.lib().mure_eval_vanilla(model.h, X.ctypes.data, 70, None, 0, *rest)):
         assert st == 1 and bad in M.lib().mure_last_error(ctx.h).decode()
     assert M.mure_kernel_launches(ctx) == launched and not kill.any()
+
+
+@pytest.mark.parametrize("prec", ["tf32x3", "tf32"])
+@pytest.mark.parametrize("ic,oc,k,pool,res", [(32, 256, 1, False, False), (32, 241, 3, False, False), (64, 250, 3, True, False),
+                                              (256, 256, 3, False, True), (96, 248, 3, True, False)])
+def test_wide_slices(M, ctx, oracle_mod, monkeypatch, ic, oc, k, pool, res, prec):
+    """Convolutions of 241 to 256 outputs: two issuing warps with half of the columns each, from one
+    K-step to 72.  The bits of the form with slices of 128, whose warps take turns on the K-steps,
+    of small batches and of vanilla; the oracle's logits (3xTF32)."""
+    b = wl._Builder("wide", (16, 16, 3), 5, 29)
+    x = b.conv(-1, ic, 3, pad=1)
+    y = b.conv(x, oc, k, pad=k // 2, act="none" if res else "relu")
+    y = b.add(y, x) if res else b.maxpool(y) if pool else y
+    b.dense(b.gap(b.conv(y, 16, 1)), 5, act="none")
+    X = wl.inputs(b.m, 66, 3)
+    table = wl.concat([wl.mutants(b.m, 6, seed=70 + l, ratios=(0.02,), ops=("GF", "NEB", "NAI"), layers=[l])
+                       for l in range(b.m.n_layers())])
+    m = M.mure_model_load(ctx, b.m, precision=prec)
+    monkeypatch.setenv("MURE_TC_NARROW", "1")
+    narrow = M.mure_model_load(ctx, b.m, precision=prec)
+    monkeypatch.delenv("MURE_TC_NARROW")
+    cache = M.mure_build_prefix_cache(m, X)
+    r = M.mure_eval_mutants(cache, table, logits=True)
+    if prec == "tf32x3":
+        ok, worst = logits_close(r["logits"], oracle_mod.vanilla(b.m, X, table)["logits"])
+        assert ok, worst
+    for other in (M.mure_eval_mutants(M.mure_build_prefix_cache(narrow, X), table, logits=True),
+                  M.mure_eval_mutants(cache, table, logits=True, workspace_bytes=1 << 22),
+                  M.mure_eval_vanilla(m, X, table, logits=True)):
+        assert np.array_equal(other["logits"].view(np.uint32), r["logits"].view(np.uint32))
