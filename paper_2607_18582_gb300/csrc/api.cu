@@ -132,8 +132,7 @@ int64_t round_up(int64_t n, int64_t a) { return (n + a - 1) / a * a; }
 
 // A call's results on their way to the host: small ones through the context's pinned memory,
 // queued without waiting and handed over by finish() after one synchronisation (a copy into
-// pageable memory waits for the stream by itself, each of them); larger ones, and those of a
-// call that finds another thread's call holding the memory, straight.
+// pageable memory waits for the stream by itself, each of them); larger ones straight.
 struct Results {
     static constexpr size_t kPinned = 1 << 20;
     mure_ctx *c;
@@ -143,12 +142,11 @@ struct Results {
         size_t off, bytes;
     };
     std::vector<Item> items;
-    std::unique_lock<std::mutex> lock;
-    explicit Results(mure_ctx *ctx) : c(ctx), lock(ctx->pinned_mu, std::try_to_lock) {}
+    explicit Results(mure_ctx *ctx) : c(ctx) {}
     void add(void *dst, const void *dev, size_t bytes)
     {
         const size_t need = round_up(bytes, 16);
-        if (lock.owns_lock() && c->pinned && used + need <= kPinned) {
+        if (c->pinned && used + need <= kPinned) {
             CK(c, cudaMemcpyAsync(c->pinned + used, dev, bytes, cudaMemcpyDeviceToHost, c->stream));
             items.push_back({dst, used, bytes});
             used += need;

@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <mutex>
 #include <string>
 #include <vector>
 
@@ -82,7 +81,6 @@ struct mure_ctx {
     // pinned host memory for a call's small results (created with the context, freed with it):
     // copies into it are queued without waiting, one synchronisation then covers all of them
     char *pinned = nullptr;           // null: not available, results are copied straight
-    std::mutex pinned_mu;             // held from a call's first copy to its hand-over
 };
 
 struct mure_model {

@@ -17,7 +17,7 @@ namespace mure {
 struct ConvSmallParams {
     const float *x; int64_t x_stride; int x_per_input;
     int64_t t0; int T; int R;
-    int ih, iw, oh, ow;
+    int iw;
     const float *Wt;  // [K][OC]
     const float *b;
     int act1;
@@ -155,109 +155,72 @@ __global__ void __launch_bounds__(kC1Threads, 2) k_conv1_pairs(const ConvSmallPa
     }
 }
 
-// The other geometry (5 x 5, 6 -> 16 channels on 14 x 14, LeNet's second layer): KH x KW filter,
-// IC input channels, OC output channels (OCT of them per thread), WP / HP padded input width /
-// height, PAD zero padding, POOL: 2x2 max pool after the activation; ROWS rows of CELLS windows
-// (or groups of four positions) per block.
-template <int KH, int KW, int IC, int OC, int OCT, int WP, int HP, int PAD, bool POOL, int ROWS, int CELLS>
+// The other geometry, 5 x 5, 6 -> 16 channels, no padding, on 14 x 14, pooled (LeNet's second layer):
+// a thread takes four output channels of a pooling window, two rows of 25 windows per block.
+constexpr int kC2K = 5 * 5 * 6, kC2Oc = 16, kC2Line = 14 * 6, kC2Tile = 14 * kC2Line, kC2Rows = 2, kC2Threads = kC2Rows * 25 * 4;
+
 __global__ void __launch_bounds__(256, 3) k_conv_small(const ConvSmallParams p)
 {
-    constexpr int K = KH * KW * IC;
-    constexpr int TILE = HP * WP * IC;
-    constexpr int NSPLIT = OC / OCT;
     extern __shared__ __align__(16) float sm[];
-    float *ws = sm;              // [K][OC]
-    float *xs = sm + K * OC;     // [rows_per_block][TILE]
+    float *ws = sm;                  // [150][16]
+    float *xs = sm + kC2K * kC2Oc;   // [rows][14][14][6]
     __shared__ SmallRows sr;
     const int tid = threadIdx.x;
-    const int64_t row0 = (int64_t)blockIdx.x * ROWS;
-    const int nrows = (int)(p.R - row0 < ROWS ? p.R - row0 : ROWS);
+    const int64_t row0 = (int64_t)blockIdx.x * kC2Rows;
+    const int nrows = (int)(p.R - row0 < kC2Rows ? p.R - row0 : kC2Rows);
     small_rows(p, sr, row0, nrows);
-    for (int i = tid; i < K * OC; i += blockDim.x) ws[i] = __ldg(p.Wt + i);
-    if (PAD == 0 && TILE % 4 == 0 && p.x_stride % 4 == 0) {
-        // the padded tile is the row itself: 16-byte copies, several in flight
-        constexpr int T4 = TILE / 4;
+    for (int i = tid; i < kC2K * kC2Oc; i += kC2Threads) ws[i] = __ldg(p.Wt + i);
+    // whole rows (their stride is a multiple of four) in 16-byte copies, several in flight
 #pragma unroll 4
-        for (int i = tid; i < nrows * T4; i += blockDim.x) {
-            const int rl = i / T4, e = i - rl * T4;
-            reinterpret_cast<float4 *>(xs)[i] = __ldg(reinterpret_cast<const float4 *>(sr.src[rl]) + e);
-        }
-    } else {
-#pragma unroll 4
-        for (int i = tid; i < nrows * TILE; i += blockDim.x) {
-            const int rl = i / TILE, e = i - rl * TILE;
-            const int ci = e % IC, pix = e / IC, px = pix % WP, py = pix / WP;
-            const int iy = py - PAD, ix = px - PAD;
-            float v = 0.f;
-            if ((unsigned)iy < (unsigned)p.ih && (unsigned)ix < (unsigned)p.iw)
-                v = __ldg(sr.src[rl] + (iy * p.iw + ix) * IC + ci);
-            xs[i] = v;
-        }
+    for (int i = tid; i < nrows * (kC2Tile / 4); i += kC2Threads) {
+        const int rl = i / (kC2Tile / 4), e = i - rl * (kC2Tile / 4);
+        reinterpret_cast<float4 *>(xs)[i] = __ldg(reinterpret_cast<const float4 *>(sr.src[rl]) + e);
     }
     __syncthreads();
-    if (p.ov.patch) small_overlay<IC>(p, sr, row0, nrows, xs, TILE, WP * IC, PAD, PAD);
+    if (p.ov.patch) small_overlay<6>(p, sr, row0, nrows, xs, kC2Tile, kC2Line, 0, 0);
 
-    const int per_row = CELLS * NSPLIT;
-    const int rl = tid / per_row, cell = (tid % per_row) / NSPLIT, n0 = (tid % NSPLIT) * OCT;
+    const int rl = tid / 100, cell = tid % 100 / 4, n0 = tid % 4 * 4;
     if (rl >= nrows) return;
     const int64_t row = row0 + rl;
-    // the four positions this thread computes: a pooling window, or 4 consecutive
-    // positions of one output row (ow % 4 == 0 when not pooling)
-    int oy[4], ox[4];
-    if (POOL) {
-        const int pw = p.ow / 2, py = cell / pw, px = cell % pw;
+    const int py = cell / 5, px = cell % 5;
+    const float *xt = xs + rl * kC2Tile;
+    int base[4];   // the window's positions
 #pragma unroll
-        for (int s = 0; s < 4; ++s) { oy[s] = 2 * py + (s >> 1); ox[s] = 2 * px + (s & 1); }
-    } else {
-        const int q = cell * 4;
-#pragma unroll
-        for (int s = 0; s < 4; ++s) { oy[s] = (q + s) / p.ow; ox[s] = (q + s) % p.ow; }
-    }
-    const float *xt = xs + rl * TILE;
-    float acc[4][OCT];
+    for (int s = 0; s < 4; ++s) base[s] = (2 * py + (s >> 1)) * kC2Line + (2 * px + (s & 1)) * 6;
+    float acc[4][4];
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
-        for (int n = 0; n < OCT; ++n) acc[s][n] = 0.f;
-    int base[4];
-#pragma unroll
-    for (int s = 0; s < 4; ++s) base[s] = (oy[s] * WP + ox[s]) * IC;
+        for (int n = 0; n < 4; ++n) acc[s][n] = 0.f;
 #pragma unroll 1
-    for (int ky = 0; ky < KH; ++ky)
+    for (int ky = 0; ky < 5; ++ky)
 #pragma unroll
-        for (int kx = 0; kx < KW; ++kx)
+        for (int kx = 0; kx < 5; ++kx)
 #pragma unroll
-            for (int ci = 0; ci < IC; ++ci) {
-                const int k = (ky * KW + kx) * IC + ci;
-                float w[OCT];
+            for (int ci = 0; ci < 6; ++ci) {
+                const int k = (ky * 5 + kx) * 6 + ci;
+                float w[4];
 #pragma unroll
-                for (int n = 0; n < OCT; ++n) w[n] = ws[k * OC + n0 + n];
+                for (int n = 0; n < 4; ++n) w[n] = ws[k * kC2Oc + n0 + n];
 #pragma unroll
                 for (int s = 0; s < 4; ++s) {
-                    const float a = xt[base[s] + (ky * WP + kx) * IC + ci];
+                    const float a = xt[base[s] + ky * kC2Line + kx * 6 + ci];
 #pragma unroll
-                    for (int n = 0; n < OCT; ++n) acc[s][n] = fmaf(a, w[n], acc[s][n]);
+                    for (int n = 0; n < 4; ++n) acc[s][n] = fmaf(a, w[n], acc[s][n]);
                 }
             }
-
-    float *yrow = p.y + row * p.y_stride;
 #pragma unroll
-    for (int nn = 0; nn < OCT; ++nn) {
+    for (int nn = 0; nn < 4; ++nn) {
         const int n = n0 + nn;
         const float bias = __ldg(p.b + n);
         float v[4];
 #pragma unroll
         for (int s = 0; s < 4; ++s) {
             const float zz = acc[s][nn] + bias;
-            if (p.z) p.z[row * p.z_stride + (int64_t)n * (p.oh * p.ow) + oy[s] * p.ow + ox[s]] = zz;
+            if (p.z) p.z[row * p.z_stride + n * 100 + (2 * py + (s >> 1)) * 10 + 2 * px + (s & 1)] = zz;
             v[s] = act_apply(p.act1, zz);
         }
-        if (POOL) {
-            yrow[(int64_t)cell * OC + n] = max4_first(v[0], v[1], v[2], v[3]);
-        } else {
-#pragma unroll
-            for (int s = 0; s < 4; ++s) yrow[((int64_t)oy[s] * p.ow + ox[s]) * OC + n] = v[s];
-        }
+        p.y[row * p.y_stride + cell * kC2Oc + n] = max4_first(v[0], v[1], v[2], v[3]);
     }
 }
 
@@ -279,7 +242,7 @@ int launch_conv_small(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
     if (ov) p.ov = *ov;
     p.x = x.p; p.x_stride = x.stride; p.x_per_input = x.per_input;
     p.t0 = rm.t0; p.T = rm.T; p.R = rm.R;
-    p.ih = S.ih; p.iw = S.iw; p.oh = S.oh; p.ow = S.ow;
+    p.iw = S.iw;
     p.Wt = S.Wt; p.b = S.b; p.act1 = S.act1;
     p.z = z_out; p.z_stride = z_stride;
     p.y = y_out; p.y_stride = y_stride;
@@ -288,7 +251,7 @@ int launch_conv_small(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_
         allow_dynamic_smem(kern, smem);
         kern<<<(unsigned)((rm.R + rows - 1) / rows), threads, smem, s>>>(p);
     };
-    if (S.variant == 1) go(k_conv_small<5, 5, 6, 16, 4, 14, 14, 0, true, 2, 25>, 2, 200, 150 * 16 + 2 * 14 * 14 * 6);
+    if (S.variant == 1) go(k_conv_small, kC2Rows, kC2Threads, kC2K * kC2Oc + kC2Rows * kC2Tile);
     else go(k_conv1_pairs, kC1Rows, kC1Threads, 25 * 8 + kC1Rows * kC1Tile);
     return 1;
 }

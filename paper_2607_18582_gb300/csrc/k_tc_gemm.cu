@@ -683,7 +683,7 @@ struct SmallSteps {
 // a row costs F x 12 FMAs and as many weight words from shared memory.  LeNet-5's 120 -> 84 -> 10
 // over 904,000 rows: 275 us with one set that tested each input's index, 208 without the tests
 // (the weights' loads then run ahead of the sums), 162 with two sets.
-template <int MODE, int FCP>
+template <int MODE>
 constexpr int tc_threads()
 {
     return MODE != 2 ? kThreads + 128 : kThreads;
@@ -695,7 +695,7 @@ constexpr int tc_threads()
 // each row's outputs in the epilogue, followed by the kill epilogue, and the rows
 // themselves are not stored.
 template <int MODE, bool THREE, int FCP = 0>
-__global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __grid_constant__ TcParams p)
+__global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_constant__ TcParams p)
 {
     static_assert(FCP == 0 || (MODE == 0 && FCP % 4 == 0) || (MODE == 3 && FCP == -1),
                   "the output layer is fused into dense layers only; -1: the staged mode's slot GEMM with a residual add");
@@ -749,13 +749,13 @@ __global__ void __launch_bounds__(tc_threads<MODE, FCP>(), 1) k_tc_gemm(const __
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if constexpr (FCP > 0) {
-        for (int i = threadIdx.x; i < p.ff.F * FCP; i += tc_threads<MODE, FCP>()) {
+        for (int i = threadIdx.x; i < p.ff.F * FCP; i += tc_threads<MODE>()) {
             const int f = i / FCP, c = i % FCP;
             const float wv = c < p.ff.C ? p.ff.W[(int64_t)c * p.ff.F + f] : 0.f;
             asm volatile("st.shared.f32 [%0], %1;" ::"r"(fw_region + 4 * i), "f"(wv) : "memory");
         }
     }
-    for (int n = threadIdx.x; n < kSliceMax; n += tc_threads<MODE, FCP>()) {
+    for (int n = threadIdx.x; n < kSliceMax; n += tc_threads<MODE>()) {
         if (MODE == 2) bias_sh[n] = n < SmallConv::N ? p.b[n % SmallConv::OC] : 0.f;
         else bias_sh[n] = n_base + n < p.N ? p.b[n_base + n] : 0.f;
     }
@@ -2371,7 +2371,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     auto go = [&](auto kernel) {
         constexpr auto kern = decltype(kernel)::value;
         allow_dynamic_smem(kern, (int)tc_dyn_smem_max<kern>());
-        kern<<<grid, S.tc_small ? tc_threads<2, 0>() : tc_threads<0, 0>(), smem, s>>>(p);
+        kern<<<grid, S.tc_small ? tc_threads<2>() : tc_threads<0>(), smem, s>>>(p);
     };
     auto either = [&](auto x3, auto x1) { three ? go(x3) : go(x1); };
     if (dense && ff) either(TcKernel<0, true, kFuseClasses>(), TcKernel<0, false, kFuseClasses>());
