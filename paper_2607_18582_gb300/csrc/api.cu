@@ -1628,7 +1628,6 @@ mure_status mure_create(int device, void *cuda_stream, const mure_allocator *all
     if (alloc) { c->alloc = *alloc; c->has_alloc = true; }
     mure_status st = run(c, [&] {
         CK(c, cudaSetDevice(device));
-        CK(c, cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, device));
         for (auto &e : c->ev) CK(c, cudaEventCreate(&e));
         CK(c, cudaMalloc(&c->err_dev, sizeof(int)));
         CK(c, cudaMemset(c->err_dev, 0, sizeof(int)));

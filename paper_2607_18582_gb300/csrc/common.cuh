@@ -74,7 +74,6 @@ struct mure_ctx {
     std::string err;
     cudaEvent_t ev[8]{};
     std::vector<cudaEvent_t> evpool;  // per-launch timing events, reused across calls
-    int n_sms = 0;
     int64_t launches = 0;             // kernels launched since creation
     int *err_dev = nullptr;           // device error word written by bounded waits
     int64_t wait_limit = 0;           // limit of the device-side waits in SM cycles (0 = default)
@@ -161,6 +160,19 @@ struct Overlay {
     // the patch values of those rows are not read (the delta need not write them)
     const int32_t *op = nullptr;
 };
+
+// Multiprocessors of the current device (152 on a GB300), looked up once.
+inline int sm_count()
+{
+    static const int n = [] {
+        int dev = 0, v = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+            v = 152;
+        return v;
+    }();
+    return n;
+}
 
 // Lets a kernel be launched with up to `most` bytes of dynamic shared memory.  The limit belongs to
 // the kernel in the process, not to a stream or context, and other host threads launch the same

@@ -209,7 +209,7 @@ int launch_conv1x1(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_str
     p.y = y_out; p.y_stride = y_stride;
     if (ov) p.ov = *ov;
     const int smem = (S.ic * S.oc + 2 * p.tp * (S.ic + 4)) * (int)sizeof(float);
-    const unsigned blocks = (unsigned)std::min<int64_t>(p.tiles, 4 * 152);
+    const unsigned blocks = (unsigned)std::min<int64_t>(p.tiles, 4 * sm_count());
     auto go = [&](auto kern) {
         allow_dynamic_smem(kern, kSmemMax11);
         kern<<<blocks, kThreads11, smem, s>>>(p);

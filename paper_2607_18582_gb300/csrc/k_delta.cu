@@ -610,7 +610,7 @@ static int launch_dense_rows(const PatchValsParams &p, float *y, int64_t y_strid
 {
     // rows per warp: enough to pay for the deltas in registers, few enough to fill the GPU
     int rpw = 8;
-    while (rpw < 32 && (int64_t)p.G * p.T > (int64_t)152 * 64 * rpw) rpw *= 2;
+    while (rpw < 32 && (int64_t)p.G * p.T > (int64_t)sm_count() * 64 * rpw) rpw *= 2;
     while ((p.T + 8 * rpw - 1) / (8 * rpw) > 65535) rpw *= 2;
     const dim3 grid((unsigned)p.G, (unsigned)((p.T + 8 * rpw - 1) / (8 * rpw)));
     if (p.K <= 128) k_patch_dense_rows<4><<<grid, 256, 0, s>>>(p, y, y_stride, rpw);
@@ -670,11 +670,11 @@ int launch_patch_vals(const Stage &S, Src z, Src x, Src skip, RowMap rm, const P
     const int64_t gx = (n_items + 7) / 8;
     const bool lane_per_input = skip_dot_ops && S.kind != MURE_NODE_DWCONV && (p.warp_dot || p.cells < 32);
     const int64_t gy = std::max<int64_t>(1, std::min<int64_t>(lane_per_input ? (rm.T + 31) / 32 : rm.T,
-                                                              (152 * 16 + gx - 1) / gx));
+                                                              (sm_count() * 16 + gx - 1) / gx));
     // few slots and inputs: a slot's cells are split over blocks too (MobileNetV2's depthwise
     // layers, 4 mutants x 320 inputs on 320 blocks: 20 launches of a job 1.00 ms, now 0.59)
     const int64_t gz = !S.gap && !p.warp_dot
-                           ? std::max<int64_t>(1, std::min<int64_t>(p.cells / 64, 152 * 16 / std::max<int64_t>(gx * gy, 1)))
+                           ? std::max<int64_t>(1, std::min<int64_t>(p.cells / 64, sm_count() * 16 / std::max<int64_t>(gx * gy, 1)))
                            : 1;
     const dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)gz);
     const size_t smem = (S.gap && !p.warp_dot) ? 8 * (size_t)p.mcells * sizeof(float) : 0;
@@ -820,7 +820,7 @@ int launch_rows_overlay(Src base, int64_t n_floats, RowMap rm, const Overlay &ov
         }
         const int64_t total = (int64_t)rm.R * ov.kmax * ov.cells;
         if (total > 0) {
-            const int64_t blocks = std::min<int64_t>((total + 255) / 256, 152 * 64);
+            const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)sm_count() * 64);
             k_overlay_scatter<<<(unsigned)blocks, 256, 0, s>>>(rm.T, rm.R, ov, out, out_stride, rm.lrow);
             ++launches;
         }

@@ -693,7 +693,7 @@ int launch_lstm(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride
     }
     // rows per block: the split whose waves (two blocks per SM) take the fewest row steps; a
     // pair on one SM takes about 1.5 times as long as one block alone
-    const int slots = 2 * 152;
+    const int slots = 2 * sm_count();
     int bm = 4;
     int64_t least = INT64_MAX;
     for (int b = 4; b <= 32; b += 4) {

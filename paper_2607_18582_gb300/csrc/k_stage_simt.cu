@@ -1013,7 +1013,7 @@ int launch_final_dense(const Stage &S, Src x, RowMap rm, const FinalArgs &fa, cu
             // blocks that stay (four per SM) and take several tiles: the weights are placed once
             // per block, not once per 32 rows
             const int tiles = (rm.R + 31) / 32;
-            k_final_dense_split<<<(unsigned)std::min(tiles, 4 * 152), 128, sbytes, s>>>(p, tiles);
+            k_final_dense_split<<<(unsigned)std::min(tiles, 4 * sm_count()), 128, sbytes, s>>>(p, tiles);
         }
         return 1;
     }

@@ -2359,15 +2359,8 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     const int64_t M = (int64_t)rm.R * p.P;
     const int64_t unit = p.cv_pair ? 2 * kTileM : kTileM;
     const int64_t tiles = S.tc_small ? small_tiles(rm.R) : (M + unit - 1) / unit;
-    static int n_sm = 0;
-    if (!n_sm) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        if (n_sm <= 0) n_sm = 148;
-    }
     const int ny = (p.Np + p.slice_w - 1) / p.slice_w;
-    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, n_sm / ny))), (unsigned)ny);
+    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, std::max(1, sm_count() / ny))), (unsigned)ny);
     auto go = [&](auto kernel) {
         constexpr auto kern = decltype(kernel)::value;
         allow_dynamic_smem(kern, (int)tc_dyn_smem_max<kern>());
