@@ -98,11 +98,12 @@ enum { MURE_OP_GF = 0, MURE_OP_NEB = 1, MURE_OP_NAI = 2, MURE_OP_NS = 3, MURE_OP
  * (fp32-level accuracy).  In fp32 on the CUDA cores in every mode: layers of fewer
  * outputs, recurrent and depthwise layers, and the 1x1 convolutions of few channels (at
  * most 4,096 weights) that run faster there; the sum over a GF or WS neuron's weight
- * changes in such a 1x1 layer follows the mode.  TF32: the same layer selection with one TF32 product (the reduced-precision variant; its kill verdicts are
- * compared with the fp32 oracle's, not bit-matched).  BF16: reserved.  The output layer
- * always uses the fp32 CUDA-core kernel.  One model uses
- * one arithmetic for every layer computation (cache build, vanilla prefix and
- * suffix), so memoized and vanilla results stay bit-identical under every mode. */
+ * changes in such a 1x1 layer follows the mode.  TF32: the same layer selection with one
+ * TF32 product (the reduced-precision variant; its kill verdicts are compared with the
+ * fp32 oracle's, not bit-matched).  BF16: reserved.  The output layer always uses the
+ * fp32 CUDA-core kernel.  One model uses one arithmetic for every layer computation
+ * (cache build, vanilla prefix and suffix), so memoized and vanilla results stay
+ * bit-identical under every mode. */
 enum { MURE_PREC_FP32 = 0, MURE_PREC_TF32X3 = 1, MURE_PREC_BF16 = 2, MURE_PREC_TF32 = 3 };
 
 /* One node.  in0/in1 are node ids (< this node's id) or -1 for the network input.

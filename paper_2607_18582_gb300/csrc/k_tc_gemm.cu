@@ -2126,8 +2126,7 @@ static void tc_config(TcParams &p, int nt_max, bool three, bool chain)
     p.n_part = m;
     p.mma_chain = 0;
     if (chain && nK >= 2 && mma_gap(nK, 2) <= depth) {
-        // two issuing warps in turn on one accumulator per set: two sets up to 128
-        // columns, one wide set
+        // two issuing warps in turn on one accumulator per set
         p.n_mma = 2;
         p.n_part = 1;
         p.mma_chain = 1;
