@@ -711,8 +711,6 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_
     // dense A tiles by tensor-map copies: slot landed, slot read by the producers
     __shared__ __align__(8) uint64_t bar_alanded[kNA], bar_afree[kNA];
     __shared__ uint32_t tmem_sh;
-    // mma_chain: warp w's turn comes when the other warp's MMAs complete (a commit to bar_turn[w])
-    __shared__ __align__(8) uint64_t bar_turn[2];
     __shared__ WaitCtl abort_sh;
     __shared__ float bias_sh[kSliceMax];
     __shared__ __align__(16) float epi_stage[4][32 * kEpiStride];   // per epilogue warp: 32 rows x 32 values
@@ -802,8 +800,6 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_
             mbar_init(smem_u32(&bar_released[s]), MODE == 3 ? 8 : 4);   // every producer warp
         }
         abort_sh.abort = 0;
-        mbar_init(smem_u32(&bar_turn[0]), 1);
-        mbar_init(smem_u32(&bar_turn[1]), 1);
         abort_sh.limit = p.spin > 0 ? p.spin : kSpin;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1677,16 +1673,16 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_
         // (kt mod n_mma = w), each warp into its own partial accumulator: a split that
         // depends on kt alone, so a row's partial sums never depend on its place in the
         // batch.  With mma_chain the warps share one accumulator and take the K-steps
-        // in turn: a warp issues K-step g only once the MMAs of g - 1 have completed (the other
-        // warp's commit to the turn barrier), so they run in K-step order, as from one warp, while each
-        // warp's waits for its operands overlap the other's MMAs.  (A barrier is never two phases
-        // ahead of its waiter: the other warp's next turn waits for this warp's commit.)
+        // in turn: a warp issues K-step g only once the MMAs of g - 1 have completed, which the
+        // other warp's commit to the barrier of their A stage tells, so they run in K-step order, as
+        // from one warp, while each warp's waits for its operands overlap the other's MMAs.  (That
+        // barrier is never two phases ahead: its stage's next K-step comes after g.)
         // Completion, not issue: handing the turn over when the MMAs have been issued (fences before
         // and after an arrival) held their order only while one lane issued them slowly; with an
         // elected lane the other warp's MMAs passed them, and 3xTF32 sums came out differently on
         // VGG, LeNet-5, ResNet-10 and dense networks.  It was no faster on the whole (1,000 x 120 VGG
-        // mutants, ms: conv 64->128 7.46 and 7.11 now, 128->128 16.24 and 17.24, dense 2.18 and 2.37, the
-        // deltas 2.93 and 2.29); one warp without turns took 15 % longer on VGG.
+        // mutants, ms: conv 64->128 7.42 and 7.09 now, 128->128 16.26 and 17.28, dense 2.19 and 2.39, the
+        // deltas 2.94 and 2.30); one warp without turns took 15 % longer on VGG.
         const int w = warp - 8;
         if (pair) {
             // tile pairs: warp w issues tile w of each unit into its own accumulator, both
@@ -1768,10 +1764,11 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_
                         if (!wait(&bar_afull[t], t_wraps & 1)) { ok = false; break; }
                         if (!p.b_resident && !wait(&bar_bfull[sb], b_wraps & 1)) { ok = false; break; }
                         const uint32_t g = (uint32_t)(i * nK + kt);
-                        // K-step g goes to warp g mod 2; it waits for the commit of K-step g - 1
-                        // by the other warp, the ((g + w) / 2)-th arrival on its barrier
+                        // K-step g goes to warp g mod 2; it waits for the release of the A stage of
+                        // K-step g - 1 by the other warp's commit
+                        const int tp = (t > 0 ? t : p.n_stages) - 1;
                         if (chain && g > 0 &&
-                            !warp_wait_phase<0>(smem_u32(&bar_turn[w]), (((g + (uint32_t)w) >> 1) + 1) & 1, abort_flag)) {
+                            !warp_wait_phase<0>(smem_u32(&bar_aempty[tp]), (t > 0 ? t_wraps : t_wraps - 1) & 1, abort_flag)) {
                             ok = false;
                             break;
                         }
@@ -1782,7 +1779,9 @@ __global__ void __launch_bounds__(tc_threads<MODE>(), 1) k_tc_gemm(const __grid_
                         if (elect_one()) {
                             if (merged) mma_block_merged(d, tmem + p.a_col + t * kAColsPerStage, dh, id2, id, acc0);
                             else mma_block<THREE, 0, Q>(d, tmem + p.a_col + t * kAColsPerStage, dh, dl, id, acc0);
-                            if (chain) mma_commit(smem_u32(&bar_turn[1 - w]));
+                            // (this lane alone, so no wait: it keeps the commits' preparation from
+                            // being moved between the MMAs; the window GEMM 3.91 -> 3.81 ms)
+                            __syncwarp(1u << lane);
                             mma_commit(smem_u32(&bar_aempty[t]));
                             if (!p.b_resident) mma_commit(smem_u32(&bar_bempty[sb]));
                         }
@@ -2349,7 +2348,7 @@ int launch_tc(const Stage &S, Src x, RowMap rm, float *z_out, int64_t z_stride, 
     }
     if (p.slice_w > kSlice) {
         // a wide slice: both issuing warps take every K-step, each its half of the columns, so that
-        // no turn is handed over (VGG's conv 256->256: 22.1 ms with turns, 20.4 without)
+        // no turn is handed over (VGG's conv 256->256, 1,000 x 120: 22.1 ms with turns, 19.9 without)
         p.n_mma = 2;
         p.n_part = 1;
         p.mma_chain = 0;
