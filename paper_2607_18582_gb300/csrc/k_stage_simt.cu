@@ -42,8 +42,8 @@ struct StageParams {
 // input channels come in fours on 16-byte rows, so a thread fetches four k of its row at once.
 // OV (with A4 only): a fetched piece takes the mutated channels from the patch (where: see
 // simt_overlay_inline).  Measured on LeNet-5 in fp32 (1,500 x 150, FC 400-120 and 120-84): 0.88 ms
-// with 4 x 4 sums per thread and rows materialised first, 0.69 now; what bounds it is the latency of a tile's loads (few tiles
-// per SM at these sizes) and 84 or 120 outputs in 128 columns.
+// with 4 x 4 sums per thread and rows materialised first, 0.69 now; what bounds it is the latency
+// of a tile's loads (few tiles per SM at these sizes) and 84 or 120 outputs in 128 columns.
 template <int BM, int BN, int TM, int TN, bool A4, bool OV>
 __global__ void __launch_bounds__(BM / TM * (BN / TN), A4 && !OV && BN != 64 ? 4 : 3) k_stage_simt(const StageParams p)
 {
